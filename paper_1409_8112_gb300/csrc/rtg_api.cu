@@ -578,7 +578,9 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
       if ((s = ensure(c, c->tc_norms, (size_t)(n_total + 128) * 4)) != RTG_OK) return s;
       if ((s = ensure(c, c->tc_plan, sizeof(rtg::TcPlan))) != RTG_OK) return s;
     }
-    int sorted = 0;
+    // (known without running the sort: a replayed graph launches no kernel from here, and a
+    // second enumeration after it reads the sorted keys)
+    const int sorted = rtg::sorted_buffer(a);
     // phase marks: recorded as real event records even inside a captured graph
     auto mark = [&](int i) {
       cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -599,7 +601,7 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
         rtg::launch_keys(a, st);
         l += 1;
         if (timing) mark(2);
-        sorted = rtg::launch_sort(a, st);
+        rtg::launch_sort(a, st);
         l += (a.passes > 0 && N > 1)
                  ? (rtg::hist_in_keys(a) ? 0 : 1) +
                        (a.sort_mode == rtg::kSortCoop

@@ -428,8 +428,11 @@ __device__ __forceinline__ void finish_digit_count_bits(const unsigned int* sh, 
 // for small batches); returns the kernels launched.
 int launch_prep_plan(const BuildArgs& a, cudaStream_t s);
 void launch_keys(const BuildArgs& a, cudaStream_t s);
-// returns the ping-pong buffer (0 or 1) that holds the sorted data
+// returns the ping-pong buffer (0 or 1) that holds the sorted data: sorted_buffer(a)
 int launch_sort(const BuildArgs& a, cudaStream_t s);
+inline int sorted_buffer(const BuildArgs& a) {
+  return a.passes > 0 && a.n_total * a.m > 1 ? (a.passes - 1) & 1 : 0;
+}
 // the launch_* functions returning int return the number of kernels they launched
 int launch_pairs(const BuildArgs& a, int sorted_buf, Mode mode, cudaStream_t s);
 int launch_brute(const BuildArgs& a, Mode mode, cudaStream_t s);

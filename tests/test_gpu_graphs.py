@@ -93,3 +93,25 @@ def test_pair_buffer_growth_falls_back_and_recaptures():
             assert np.array_equal(rp, ref.csr.row_ptr) and np.array_equal(col, ref.csr.col)
     finally:
         ctx.close()
+
+
+def test_overflow_after_a_replay_with_an_even_pass_count():
+    # a replayed build whose pairs overflow its buffer writes the columns by a second
+    # enumeration, which has to read the buffer the sort ended in (the second one for an even
+    # number of passes)
+    d, n, m, r = 3, 6000, 6, 0.06
+    corners = np.array([[0.0] * d, [1.0] * d])
+    loose = np.vstack([gen.points_mixture(21, n - 2, d, k=8, sigma=0.08, dtype=np.float64), corners])
+    tight = np.vstack([gen.points_mixture(21, n - 2, d, k=8, sigma=0.05, dtype=np.float64), corners])
+    T = gen.transforms(21, d, m, r)
+    ctx = rtg.Context(0)
+    for k in range(5):
+        pts = loose if k < 3 else tight
+        res = ctx.all_pairs(pts, r, T, r)
+        st, (rp, col) = res.stats, res.download()
+        res.release()
+        assert st["sort_passes"] % 2 == 0 and st["max_cell"] > 24
+        assert st["attempts"] == (2 if k == 3 else 1) or k == 0
+        ref = oracle.rtg(pts, r, T, r).csr
+        assert np.array_equal(rp, ref.row_ptr) and np.array_equal(col, ref.col), k
+    ctx.close()
