@@ -401,6 +401,7 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
   a.dtype = q.dtype;
   a.dpad = dpad;
   a.d_common = mind == maxd ? maxd : 0;
+  a.d_max = maxd;
   a.symmetric = sym;
   a.n_total = n_total;
   a.blocks = blk0;
@@ -494,7 +495,6 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
     // warps with heavy spans do not trail
     a.spans_per_warp = g.pairs_tuned ? g.spans_per_warp
                                      : (g.cand_per_pos < 0.0f ? 2 : (g.cand_per_pos >= 3.0f ? 4 : 1));
-    a.dense_min = g.pairs_tuned ? g.dense_min : 0;
     if (m > 0) {
       const size_t ksz = a.key64 ? 8 : 4;
       if ((s = ensure(c, c->key_mat, (size_t)N * ksz)) != RTG_OK) return s;
@@ -534,9 +534,7 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
         // enumerates every candidate, would cost seconds
         if (g.cand_per_pos >= 0.0f &&
             (double)g.cand_per_pos * (double)N <= c->tune_pairs_max_cand) {
-          if ((s = tune_pairs(c, a, best, sort_key_bits, &g.spans_per_warp, &g.dense_min)) !=
-              RTG_OK)
-            return s;
+          if ((s = tune_pairs(c, a, best, sort_key_bits, &g.spans_per_warp)) != RTG_OK) return s;
           g.pairs_tuned = g.spans_per_warp > 0;
         }
         tuned_now = true;
@@ -928,7 +926,7 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
     S.launches = launches;
     S.attempts = attempt + 1 - (tuned_now ? 1 : 0) + recovered;
     S.pairs_spans_per_warp = m > 0 ? a.spans_per_warp : 0;
-    S.dense_cell_min = m > 0 ? (a.dense_min > 0 ? a.dense_min : 256) : 0;
+    S.dense_cell_min = m > 0 ? 256 : 0;
     S.pairs_tuned = m > 0 && g.pairs_tuned ? 1 : 0;
     S.sort_cell_major = m > 0 && a.cell_major ? 1 : 0;
     S.sort_key_bits = m > 0 ? (a.cell_major ? (int32_t)h.cell_bits : (int32_t)h.sort_bits) : 0;

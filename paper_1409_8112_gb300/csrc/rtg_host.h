@@ -43,7 +43,6 @@ struct ShapeGuess {
   float cand_per_pos = -1.0f;  // in-cell candidates per sorted position at the last build
   bool pairs_tuned = false;    // enumeration knobs measured for this shape
   int spans_per_warp = 0;      // (tuned) spans per resident warp
-  int dense_min = 0;           // (tuned) cells of more points take the tiled kernels
   bool no_dense = false;       // the last build had no cell of more than 32 points
   bool no_long_rows = false;   // the last build had no row of more than 32 entries
 };
@@ -190,11 +189,10 @@ rtg::SortConfig sort_default(long long N, int num_sms);
 // it in the context's table and JSON cache.  Needs a's buffers sized for any variant.
 rtg_status tune_sort(rtg_ctx* c, rtg::BuildArgs& a, long long N, int key_bits,
                      rtg::SortConfig* out);
-// Times the in-cell enumeration of a's keys (sorted with cfg) for each (spans per warp,
-// dense-cell threshold) candidate and returns the fastest; 0, 0 (the defaults) when a first
-// trial takes long.
+// Times the in-cell enumeration of a's keys (sorted with cfg) for each spans-per-warp candidate
+// and returns the fastest; 0 (the default) when a first trial takes long.
 rtg_status tune_pairs(rtg_ctx* c, rtg::BuildArgs& a, const rtg::SortConfig& cfg, int key_bits,
-                      int* spans_per_warp, int* dense_min);
+                      int* spans_per_warp);
 size_t sort_scratch_bytes(long long N, const rtg::SortConfig& cfg);  // look-back / counts
 size_t sort_scratch_bytes_max(long long N);
 void tune_load(rtg_ctx* c);

@@ -65,7 +65,7 @@ enum : uint32_t {
 
 // Kernels a build leaves out because the last build of its shape gave them nothing to do
 // (BuildArgs::skip_tail); the kernels before them flag kErrTailSkipped if work turns up.
-constexpr int kSkipDense = 1;     // the medium-cell, large-cell set-up and large-cell kernels
+constexpr int kSkipDense = 1;     // the tile, large-cell set-up and large-cell kernels
 constexpr int kSkipLongRows = 2;  // the warp and block row sorts
 // A shape whose last build had no cell and no row longer than this leaves those kernels (for
 // more than 32 points or entries) out of its next builds; the margin keeps new data of the
@@ -88,7 +88,7 @@ enum : unsigned int {
   kInjectTcWait = 4u     // the tensor-core kernel waits on an mbarrier nothing arrives on
 };
 
-// Cells with more points than this are enumerated by the tiled large-cell kernel.
+// Cells with more points than this are enumerated by the tiled kernels.
 constexpr int kSmallCell = 32;
 
 // Enumeration modes.
@@ -128,10 +128,13 @@ struct Status {
   unsigned long long key_rechecks;
   unsigned long long dist_rechecks;
   unsigned long long large_cells;
+  unsigned long long dense_cells;  // cells queued for the 128 x 128 tile kernels
   unsigned long long large_jobs;
   unsigned long long max_cell;
   unsigned int sort_tiles[kMaxPasses];
   unsigned int span_next[2];  // pair enumeration: next unclaimed span (count/emit, write)
+  unsigned int tile_jobs;     // pair enumeration: jobs queued for the 32 x 32 tile kernel
+  unsigned int tile_next[2];  // next unclaimed tile job (count/emit, write)
   unsigned int coop_count;  // single-launch sort: blocks arrived at the current grid barrier
   unsigned int coop_gen;    // single-launch sort: grid barriers completed
   unsigned int long_rows;  // rows queued for the block row sort
@@ -232,12 +235,12 @@ struct OutSlot {
 // ---- launch arguments ----------------------------------------------------------------------
 struct BuildArgs {
   int spans_per_warp;  // pair enumeration: spans per resident warp (1: static, one each)
-  int dense_min;       // cells of more points than this take the tiled kernels (0: 256)
   int B;              // instances
   int m;              // grids per instance (0: brute force)
   int dtype;          // 0 FP64, 1 FP32 (common to the batch)
   int dpad;           // padded row width (common to the batch)
   int d_common;       // d of every instance when they share one, else 0
+  int d_max;          // widest d
   int symmetric;
   long long n_total;  // sum of n
   long long blocks;   // per-point kernel blocks (sum of ceil(n / kPointBlock))

@@ -42,10 +42,11 @@ constexpr int kRing = 64;  // staged positions per warp: covers the 31 partners 
 static_assert(kRing >= kSmallCell - 1 + 32 && (kRing & (kRing - 1)) == 0, "ring too small");
 constexpr int kWarpEmit = 128;             // EMIT: reported pairs buffered per warp
 constexpr int kWarpFlush = kWarpEmit - 32;  // written out once more than this many are held
-constexpr int kTL = 128;                   // large-cell tile
-constexpr int kMediumMax = 256;            // large cells up to this size: one warp per cell
-constexpr int kMediumWarps = 4;            // warps per block of the medium-cell kernel
-constexpr int kMediumKeyBytes = 8192;      // per warp: staged key rows of a medium cell
+constexpr int kTL = 128;                   // dense-cell tile (tensor cores, huge cells)
+constexpr int kTcCellMin = 256;            // cells of more points take the tensor-core tiles
+                                           // (when a build asks for them)
+constexpr int kTileCellMax = 8192;         // larger cells take k_pairs_large
+constexpr int kTileWarps = 8;              // warps per block of the tile kernel
 
 __device__ __forceinline__ double load_coord(const void* pts, int dtype, long long i, int d,
                                              int l) {
@@ -146,29 +147,15 @@ __device__ __forceinline__ float2 band_of(const InstPlan& IP) {
   return IP.filter_on ? make_float2(IP.s_lo, IP.s_hi) : make_float2(-1.0f, __int_as_float(0x7f800000));
 }
 
-// Decide one candidate pair (i < j, global indices) of grid t of instance I; ki and kj are the
-// two points' key rows (shared or global memory); band is band_of(IP).
-template <typename K, int DPAD, int MODE, bool VEC = false>
-__device__ __forceinline__ bool decide_pair(unsigned int i, unsigned int j, int t, const float* pa,
-                                            const float* pb, const K* ki, const K* kj,
-                                            const Inst* __restrict__ Ip,
-                                            const InstPlan* __restrict__ IPp, float2 band,
-                                            int dtype, Tally& tl, unsigned long long* near_r) {
-  float sf = 0.0f;
-#pragma unroll
-  for (int v = 0; v < DPAD / 4; ++v) {
-    const float4 x = reinterpret_cast<const float4*>(pa)[v];
-    const float4 y = reinterpret_cast<const float4*>(pb)[v];
-    float e = x.x - y.x;
-    sf = fmaf(e, e, sf);
-    e = x.y - y.y;
-    sf = fmaf(e, e, sf);
-    e = x.z - y.z;
-    sf = fmaf(e, e, sf);
-    e = x.w - y.w;
-    sf = fmaf(e, e, sf);
-  }
-  if (sf > band.y) return false;  // beyond r for certain: no ownership test needed
+// Decides a pair (i < j, global indices) that the FP32 distance did not rule out, of grid t of
+// instance I: the ownership test, then the FP64 distance unless FP32 was `sure` that it is
+// within r.  ki and kj are the two points' key rows (shared or global memory).
+template <typename K, int MODE, bool VEC>
+__device__ __forceinline__ bool decide_survivor(bool sure, unsigned int i, unsigned int j, int t,
+                                                const K* ki, const K* kj,
+                                                const Inst* __restrict__ Ip,
+                                                const InstPlan* __restrict__ IPp, int dtype,
+                                                Tally& tl, unsigned long long* near_r) {
   // an earlier grid owns the pair if it co-locates it; grids in batches of four (the loads of
   // a batch issued together), stopping at the first batch with a match: a close pair usually
   // shares a cell in one of the first grids
@@ -199,7 +186,7 @@ __device__ __forceinline__ bool decide_pair(unsigned int i, unsigned int j, int 
   }
   if (MODE != kWrite && MODE != kBits) ++tl.owned;
   bool keep;
-  if (sf < band.x) {
+  if (sure) {
     keep = true;
   } else {
     const Inst& I = *Ip;
@@ -213,6 +200,32 @@ __device__ __forceinline__ bool decide_pair(unsigned int i, unsigned int j, int 
   }
   if (keep && MODE != kWrite) ++tl.pairs;
   return keep;
+}
+
+// Decide one candidate pair (i < j, global indices) of grid t of instance I; ki and kj are the
+// two points' key rows (shared or global memory); band is band_of(IP).
+template <typename K, int DPAD, int MODE, bool VEC = false>
+__device__ __forceinline__ bool decide_pair(unsigned int i, unsigned int j, int t, const float* pa,
+                                            const float* pb, const K* ki, const K* kj,
+                                            const Inst* __restrict__ Ip,
+                                            const InstPlan* __restrict__ IPp, float2 band,
+                                            int dtype, Tally& tl, unsigned long long* near_r) {
+  float sf = 0.0f;
+#pragma unroll
+  for (int v = 0; v < DPAD / 4; ++v) {
+    const float4 x = reinterpret_cast<const float4*>(pa)[v];
+    const float4 y = reinterpret_cast<const float4*>(pb)[v];
+    float e = x.x - y.x;
+    sf = fmaf(e, e, sf);
+    e = x.y - y.y;
+    sf = fmaf(e, e, sf);
+    e = x.z - y.z;
+    sf = fmaf(e, e, sf);
+    e = x.w - y.w;
+    sf = fmaf(e, e, sf);
+  }
+  if (sf > band.y) return false;  // beyond r for certain: no ownership test needed
+  return decide_survivor<K, MODE, VEC>(sf < band.x, i, j, t, ki, kj, Ip, IPp, dtype, tl, near_r);
 }
 
 // A candidate that a tensor-core tile proved to be within r (its tile d^2 is below the band
@@ -378,6 +391,47 @@ __device__ long long run_end(const K* __restrict__ skeys, long long N, long long
   return lo;
 }
 
+// Work of one warp in a cell of more than kSmallCell points.  The cell's members form T blocks
+// of 32; the job pairs the members of block r = T - 1 - b with those of the blocks
+// [r + a0, r + min(a0 + chunk, b + 1)).
+struct TileJob {
+  unsigned int start, size;       // the cell: first sorted position, points
+  unsigned short b, a0;
+  unsigned short grid, inst;
+};
+
+// Blocks per job: long enough to keep the fixed block's rows and keys in use, short
+// enough that the last jobs of a launch end together.  A cell of s <= kTileCellMax points
+// makes at most 0.15 s jobs (1152 at 8192 points), which is why the jobs fit the unused key
+// buffer (N / 4 jobs with 32-bit keys).
+__device__ __forceinline__ unsigned int tile_job_chunk(unsigned int blocks) {
+  return blocks <= 128 ? 16u : 32u;
+}
+
+// One lane: appends the jobs of a cell.
+__device__ void append_tile_jobs(TileJob* jobs, unsigned int cap, Status* st, unsigned int start,
+                                 unsigned int size, unsigned int cell) {
+  const unsigned int T = (size + 31) / 32, A = tile_job_chunk(T), q = T / A, r = T % A;
+  // sum over b < T of ceil((b + 1) / A)
+  const unsigned int count = A * (q * (q + 1) / 2) + r * (q + 1);
+  unsigned int slot = atomicAdd(&st->tile_jobs, count);
+  if (slot + count > cap) {
+    atomicOr(&st->errors, kErrLargeOverflow);
+    return;
+  }
+  TileJob j;
+  j.start = start;
+  j.size = size;
+  j.grid = (unsigned short)(cell & 0xffu);
+  j.inst = (unsigned short)(cell >> 8);
+  for (unsigned int b = 0; b < T; ++b)
+    for (unsigned int a0 = 0; a0 <= b; a0 += A) {
+      j.b = (unsigned short)b;
+      j.a0 = (unsigned short)a0;
+      jobs[slot++] = j;
+    }
+}
+
 // Segment detection and in-cell enumeration for cells of at most kSmallCell points.
 //
 // Each warp owns the cells whose first sorted position lies in its span of positions and walks
@@ -401,8 +455,9 @@ __global__ void __launch_bounds__(kPairThreads, RTG_PAIRS_MIN_BLOCKS) k_pairs_wa
     const float* __restrict__ pf, int dtype, const K* __restrict__ key_mat, int m,
     const Inst* __restrict__ inst, const InstPlan* __restrict__ iplan,
     const unsigned long long* __restrict__ bases, int nbt, Status* st, Sink sk,
-    LargeCell* large, unsigned int large_cap, int warp_bytes, unsigned int* span_next,
-    int skip_dense, int cell_major) {
+    LargeCell* large, unsigned int large_cap, TileJob* jobs, unsigned int job_cap,
+    unsigned int tile_max, int warp_bytes, unsigned int* span_next, int skip_dense,
+    int cell_major) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned long long s_gcand[kMaxGrids];
   __shared__ unsigned int s_maxcell;
@@ -506,14 +561,19 @@ __global__ void __launch_bounds__(kPairThreads, RTG_PAIRS_MIN_BLOCKS) k_pairs_wa
             // the dense-cell kernels were left out of this launch: the host runs it again
             if (skip_dense) atomicOr(&st->errors, kErrTailSkipped);
             const unsigned long long size = (unsigned long long)(e - (P0 + p));
-            const unsigned long long slot = atomicAdd(&st->large_cells, 1ull);
-            if (slot < large_cap) {
-              large[slot].start = (unsigned long long)(P0 + p);
-              large[slot].size = (unsigned int)size;
-              large[slot].grid = (unsigned short)(cell & 0xffu);
-              large[slot].inst = (unsigned short)(cell >> 8);
+            atomicAdd(&st->large_cells, 1ull);
+            if (size <= tile_max) {
+              append_tile_jobs(jobs, job_cap, st, (unsigned int)(P0 + p), (unsigned int)size, cell);
             } else {
-              atomicOr(&st->errors, kErrLargeOverflow);
+              const unsigned long long slot = atomicAdd(&st->dense_cells, 1ull);
+              if (slot < large_cap) {
+                large[slot].start = (unsigned long long)(P0 + p);
+                large[slot].size = (unsigned int)size;
+                large[slot].grid = (unsigned short)(cell & 0xffu);
+                large[slot].inst = (unsigned short)(cell >> 8);
+              } else {
+                atomicOr(&st->errors, kErrLargeOverflow);
+              }
             }
             atomicAdd(&s_gcand[cell & 0xffu], size * (size - 1) / 2);
             maxcell = max(maxcell, (unsigned int)min(size, 0xffffffffull));
@@ -667,22 +727,19 @@ __global__ void __launch_bounds__(kPairThreads, RTG_PAIRS_MIN_BLOCKS) k_pairs_wa
   flush_tally<MODE>(tl, st, s_tally);
 }
 
-// Job offsets for the tiled kernel: a cell of more than dense_min (<= kMediumMax) points and
-// T = ceil(size / kTL) tiles has T (T + 1) / 2 tile pairs; smaller cells have none (the
-// medium-cell kernel takes them).
+// Job offsets for the 128 x 128 tile kernels: a listed cell of T = ceil(size / kTL) tiles has
+// T (T + 1) / 2 tile pairs.
 __global__ void __launch_bounds__(1024) k_large_setup(const LargeCell* __restrict__ large,
                                                       unsigned int cap, Status* st,
-                                                      unsigned long long* job_off,
-                                                      unsigned int dense_min) {
+                                                      unsigned long long* job_off) {
   __shared__ unsigned long long sbuf[32];
   __shared__ unsigned long long carry;
-  const unsigned long long L = min(st->large_cells, (unsigned long long)cap);
+  const unsigned long long L = min(st->dense_cells, (unsigned long long)cap);
   if (threadIdx.x == 0) carry = 0;
   __syncthreads();
   for (unsigned long long base = 0; base < L; base += blockDim.x) {
     const unsigned long long e = base + threadIdx.x;
-    const unsigned long long T =
-        e < L && large[e].size > dense_min ? (large[e].size + kTL - 1) / kTL : 0;
+    const unsigned long long T = e < L ? (large[e].size + kTL - 1) / kTL : 0;
     const unsigned long long v = T * (T + 1) / 2;
     unsigned long long tot;
     const unsigned long long ex = block_excl_scan64(v, &tot, sbuf);
@@ -697,89 +754,193 @@ __global__ void __launch_bounds__(1024) k_large_setup(const LargeCell* __restric
   }
 }
 
-// Cells of kSmallCell + 1 .. kMediumMax points, one warp per cell: the warp stages the members
-// (FP32 rows, indices) in shared memory and walks the cell's s (s - 1) / 2 pairs 32 at a time,
-// pair k = b (b - 1) / 2 + a (a < b) advanced incrementally, so that every lane is busy
-// whatever the cell size.
-template <typename K, int DPAD, int MODE>
-__global__ void __launch_bounds__(kMediumWarps * 32) k_pairs_medium(
+// Bytes of one warp's shared memory in k_pairs_tiles: staged key rows of the fixed and the
+// walked 32 members (when they are staged), the walked members' FP32 rows, both index lists, the
+// survivors of a tile and the reported pairs held back.
+template <typename K, int DPAD>
+__host__ __device__ inline int tile_region_bytes(int m, bool stage_rows) {
+  const int b = kWarpEmit * 8 + 32 * DPAD * 4 +
+                (stage_rows ? 64 * staged_row_stride<K>(m) * (int)sizeof(K) : 0) + 64 * 4 + 1024 * 2;
+  return (b + 15) & ~15;
+}
+
+// Cells of kSmallCell + 1 .. kTileCellMax points, 32 x 32 members at a time, one warp per job
+// (TileJob), jobs claimed from a counter.  A lane keeps one member's FP32 row in registers and
+// walks the later members, whose rows all lanes read at one shared-memory address; the walk
+// only marks the pairs not beyond r (two masks per lane: not beyond, certainly inside), 2 D + 4
+// instructions a pair.  The survivors of the tile are then listed, lane by lane, and taken 32 at
+// a time, one per lane, through the ownership test, the rare FP64 recheck and the emission.
+// Members are in point order, so the pairs of a lane share their CSR row and leave together:
+// the scatter takes such a run's slots with one atomic (walking the earlier members instead
+// tripled the scatter's time on clustered points).
+// The kernel this replaced took pairs through all of that at once, one per lane: the lanes
+// whose pair was beyond r waited for the others' ownership tests (211 warp instructions per 32
+// pairs on the Table II workload below).  Bound by instruction issue.  Pairs phase before and
+// after: 100k points in 6-D, m = 20 shift-only grids of 1.35 r (6.7e7 candidates) 1552 -> 342
+// us; clustered, c = r: 100k points in 3-D 956 -> 510 us, 50k in 9-D 3891 -> 2886 us.
+template <typename K, int DPAD, int D, int MODE, int STAGE>
+__global__ void __launch_bounds__(kTileWarps * 32) k_pairs_tiles(
     const uint32_t* __restrict__ svals, const float* __restrict__ pf, int dtype,
     const K* __restrict__ key_mat, int m, const Inst* __restrict__ inst,
-    const InstPlan* __restrict__ iplan, Status* st, const LargeCell* __restrict__ large,
-    unsigned int cap, Sink sk, unsigned int dense_min) {
+    const InstPlan* __restrict__ iplan, Status* st, const TileJob* __restrict__ jobs,
+    unsigned int job_cap, unsigned int N, int nbt, Sink sk, int warp_bytes, unsigned int* next) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ unsigned long long s_emit[kMediumWarps][kWarpEmit];
   __shared__ unsigned int s_tally[4];
+  if (st->errors & (kErrTimeout | kErrSortRange | kErrLargeOverflow)) return;
+  const unsigned int J = min(st->tile_jobs, job_cap);
+  if (J == 0) return;
   if (threadIdx.x < 4) s_tally[threadIdx.x] = 0;
+  __syncthreads();
+  const unsigned int full = 0xffffffffu;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  float* w_pt = reinterpret_cast<float*>(smem) + (size_t)wib * kMediumMax * DPAD;
-  uint32_t* w_idx = reinterpret_cast<uint32_t*>(reinterpret_cast<float*>(smem) +
-                                                (size_t)kMediumWarps * kMediumMax * DPAD) +
-                    wib * kMediumMax;
-  K* w_keys = reinterpret_cast<K*>(reinterpret_cast<unsigned char*>(smem) +
-                                   (size_t)kMediumWarps * kMediumMax * (DPAD * 4 + 4) +
-                                   (size_t)wib * kMediumKeyBytes);
-  unsigned long long* w_emit = s_emit[wib];
+  unsigned char* ws = smem + (size_t)wib * warp_bytes;
+  unsigned long long* w_emit = reinterpret_cast<unsigned long long*>(ws);
+  float* w_row = reinterpret_cast<float*>(ws + kWarpEmit * 8);
+  K* w_ka = reinterpret_cast<K*>(w_row + 32 * DPAD);  // fixed members' key rows
+  const int kst = staged_row_stride<K>(m);
+  K* w_kb = w_ka + (STAGE != 0 ? 32 * kst : 0);       // walked members' key rows
+  uint32_t* w_ia = reinterpret_cast<uint32_t*>(w_kb + (STAGE != 0 ? 32 * kst : 0));
+  uint32_t* w_ib = w_ia + 32;
+  unsigned short* w_q = reinterpret_cast<unsigned short*>(w_ib + 32);  // survivors of a tile
   unsigned int ecnt = 0;
   Tally tl;
-  const unsigned long long L = min(st->large_cells, (unsigned long long)cap);
-  const unsigned long long W = (unsigned long long)gridDim.x * kMediumWarps;
-  for (unsigned long long e = (unsigned long long)blockIdx.x * kMediumWarps + wib; e < L; e += W) {
-    const LargeCell cell = large[e];
-    const unsigned int s = cell.size;
-    if (s > dense_min) continue;  // warp-uniform (the tiled kernels take it)
-    const int t = (int)cell.grid, kst = t + 1;  // staged keys per member (odd stride)
-    const bool kstage = (size_t)s * kst * sizeof(K) <= (size_t)kMediumKeyBytes;
-    for (unsigned int x = lane; x < s; x += 32) {
-      const uint32_t idx = svals[cell.start + x];
-      w_idx[x] = idx;
+  // copies the first t keys of member idx's key row to dst
+  auto stage_keys = [&](K* dst, uint32_t idx, int t) {
+    const K* kr = key_mat + (size_t)idx * m;
+    if (STAGE == 2) {
+      constexpr int kpv = 16 / (int)sizeof(K);
+      for (int u = 0; u < t; u += kpv) cp_async16(dst + u, kr + u);
+    } else if (STAGE == 1) {
+      for (int u = 0; u < t; ++u) cp_async_small<(int)sizeof(K)>(dst + u, kr + u);
+    }
+  };
+  // the next job is claimed while this one runs
+  unsigned int claim = 0;
+  if (lane == 0) claim = atomicAdd(next, 1u);
+  for (;;) {
+    const unsigned int job = __shfl_sync(full, claim, 0);
+    if (job >= J) break;
+    const TileJob jb = jobs[job];
+    if (lane == 0) claim = atomicAdd(next, 1u);
+    const int t = (int)jb.grid;
+    const unsigned int s = jb.size, T = (s + 31) / 32, r = T - 1 - jb.b;
+    if (jb.start + s > N || jb.b >= T || jb.inst >= nbt / m) {  // not a job of this build
+      if (lane == 0) atomicOr(&st->errors, kErrLargeOverflow);
+      continue;
+    }
+    const uint32_t* members = svals + jb.start;
+    const float2 band = band_of(iplan[jb.inst]);
+    float y[D];
+    __syncwarp();  // the previous job's survivors are done with the staged rows
+    {
+      const uint32_t idx = members[min(32u * r + lane, s - 1)];
+      w_ia[lane] = idx;
+      if (STAGE != 0) stage_keys(w_ka + lane * kst, idx, t);
       const float4* src = reinterpret_cast<const float4*>(pf + (size_t)idx * DPAD);
-      float4* dst = reinterpret_cast<float4*>(w_pt + x * DPAD);
 #pragma unroll
-      for (int v = 0; v < DPAD / 4; ++v) dst[v] = __ldg(src + v);
-      if (kstage) {
-        const K* kr = key_mat + (size_t)idx * m;
-        for (int u = 0; u < t; ++u) w_keys[x * kst + u] = __ldg(kr + u);
+      for (int v = 0; v < (D + 3) / 4; ++v) {
+        const float4 q = __ldg(src + v);
+        y[4 * v] = q.x;
+        if (4 * v + 1 < D) y[4 * v + 1] = q.y;
+        if (4 * v + 2 < D) y[4 * v + 2] = q.z;
+        if (4 * v + 3 < D) y[4 * v + 3] = q.w;
       }
     }
-    __syncwarp();
-    const float2 band = band_of(iplan[cell.inst]);
-    const unsigned int P = s * (s - 1) / 2;
-    // pair `lane`: b from the triangular root, then a
-    unsigned int b = (unsigned int)((1.0f + sqrtf(8.0f * (float)lane + 1.0f)) * 0.5f);
-    while (b * (b - 1) / 2 > (unsigned int)lane) --b;
-    while ((b + 1) * b / 2 <= (unsigned int)lane) ++b;
-    unsigned int a = (unsigned int)lane - b * (b - 1) / 2;
-    for (unsigned int base = 0; base < P; base += 32) {
-      bool keep = false;
-      unsigned int i = 0, j = 0;
-      if (base + lane < P) {
-        const uint32_t ia = w_idx[a], ib = w_idx[b];
-        i = min(ia, ib);
-        j = max(ia, ib);
-        const K* ka = kstage ? w_keys + a * kst : key_mat + (size_t)ia * m;
-        const K* kb = kstage ? w_keys + b * kst : key_mat + (size_t)ib * m;
-        keep = decide_pair<K, DPAD, MODE>(i, j, t, w_pt + a * DPAD, w_pt + b * DPAD, ka, kb,
-                                          inst + cell.inst, iplan + cell.inst, band, dtype, tl,
-                                          sk.near_r);
+    const unsigned int w_end = r + min(jb.a0 + tile_job_chunk(T), jb.b + 1u);
+    uint32_t idx_next = members[min(32u * (r + jb.a0) + lane, s - 1)];
+    for (unsigned int w = r + jb.a0; w < w_end; ++w) {
+      __syncwarp();  // the previous tile's survivors are done with the walked members
+      {
+        const uint32_t idx = idx_next;
+        w_ib[lane] = idx;
+        const float* src = pf + (size_t)idx * DPAD;
+#pragma unroll
+        for (int v = 0; v < (D + 3) / 4; ++v) cp_async16(w_row + lane * DPAD + 4 * v, src + 4 * v);
+        if (STAGE != 0) stage_keys(w_kb + lane * kst, idx, t);
+        if (w + 1 < w_end) idx_next = members[min(32u * (w + 1) + lane, s - 1)];
       }
-      if (MODE == kBits) deliver_bits(keep, i, j, inst + cell.inst, sk);
-      else if (MODE == kEmit) warp_emit(keep, i, j, w_emit, ecnt, sk);
-      else deliver<MODE>(keep, i, j, sk, tl);
-      a += 32;  // next pair of this lane: 32 on
-      while (a >= b) {
-        a -= b;
-        ++b;
+      cp_async_wait_all();
+      __syncwarp();
+      const int nw = (int)min(32u, s - 32u * w);  // only the cell's last block is short
+      unsigned int hits = 0, sure = 0;  // walked members not beyond r, certainly within r
+      for (int x0 = 0; x0 < nw; x0 += 8) {
+        unsigned int h8 = 0, s8 = 0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const float* xr = w_row + (x0 + q) * DPAD;
+          float sf = 0.0f;
+#pragma unroll
+          for (int v = 0; v < (D + 3) / 4; ++v) {
+            const float4 x = reinterpret_cast<const float4*>(xr)[v];
+            float e = x.x - y[4 * v];
+            sf = fmaf(e, e, sf);
+            if (4 * v + 1 < D) {
+              e = x.y - y[4 * v + 1];
+              sf = fmaf(e, e, sf);
+            }
+            if (4 * v + 2 < D) {
+              e = x.z - y[4 * v + 2];
+              sf = fmaf(e, e, sf);
+            }
+            if (4 * v + 3 < D) {
+              e = x.w - y[4 * v + 3];
+              sf = fmaf(e, e, sf);
+            }
+          }
+          if (!(sf > band.y)) h8 |= 1u << q;
+          if (sf < band.x) s8 |= 1u << q;
+        }
+        hits |= h8 << x0;
+        sure |= s8 << x0;
+      }
+      if (nw < 32) hits &= (1u << nw) - 1u;
+      if (w == r) hits &= ~((2u << lane) - 1u);  // a block with itself: later members only
+      // list the survivors: (certain, walked member, fixed member)
+      const int nh = __popc(hits);
+      int incl = nh;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int z = __shfl_up_sync(full, incl, o);
+        if (lane >= o) incl += z;
+      }
+      const int total = __shfl_sync(full, incl, 31);
+      {
+        int pos = incl - nh;
+        unsigned int left = hits;
+        while (left) {
+          const int x = __ffs(left) - 1;
+          left &= left - 1;
+          w_q[pos++] = (unsigned short)((((sure >> x) & 1u) << 10) | (unsigned int)(x << 5) |
+                                        (unsigned int)lane);
+        }
+      }
+      __syncwarp();
+      for (int base = 0; base < total; base += 32) {
+        bool keep = false;
+        unsigned int i = 0, j = 0;
+        if (base + lane < total) {
+          const unsigned int e = w_q[base + lane], x = (e >> 5) & 31u, c = e & 31u;
+          const uint32_t ia = w_ia[c], ib = w_ib[x];
+          i = min(ia, ib);
+          j = max(ia, ib);
+          const K* ka = STAGE != 0 ? w_ka + c * kst : key_mat + (size_t)ia * m;
+          const K* kb = STAGE != 0 ? w_kb + x * kst : key_mat + (size_t)ib * m;
+          keep = decide_survivor<K, MODE, STAGE != 0>((e >> 10) != 0u, i, j, t, ka, kb,
+                                                      inst + jb.inst, iplan + jb.inst, dtype, tl,
+                                                      sk.near_r);
+        }
+        if (MODE == kBits) deliver_bits(keep, i, j, inst + jb.inst, sk);
+        else if (MODE == kEmit) warp_emit(keep, i, j, w_emit, ecnt, sk);
+        else deliver<MODE>(keep, i, j, sk, tl);
       }
     }
-    __syncwarp();
   }
   if (MODE == kEmit && ecnt) warp_flush(w_emit, ecnt, sk);
   __syncthreads();
   flush_tally<MODE>(tl, st, s_tally);
 }
 
-// Cells of more than kSmallCell points, as 128 x 128 tiles of member pairs: job = (cell, row
+// Cells of more than kTileCellMax points, as 128 x 128 tiles of member pairs: job = (cell, row
 // tile a, column tile b >= a), so every job is one tile pair however large the cell.  Each
 // thread keeps one column member (y) and walks the row members (x), which all lanes of a warp
 // read at the same address.
@@ -799,7 +960,7 @@ __global__ void __launch_bounds__(kPairThreads) k_pairs_large(
   __shared__ unsigned long long s_emit[kPairThreads / 32][kWarpEmit];
   __shared__ unsigned int s_tally[4];
   if (threadIdx.x < 4) s_tally[threadIdx.x] = 0;
-  const unsigned long long L = min(st->large_cells, (unsigned long long)cap);
+  const unsigned long long L = min(st->dense_cells, (unsigned long long)cap);
   const unsigned long long J = L ? job_off[L] : 0;
   unsigned long long* w_emit = s_emit[threadIdx.x >> 5];
   unsigned int ecnt = 0;
@@ -919,7 +1080,7 @@ __global__ void __launch_bounds__(128) k_pairs_large_tc(
   __shared__ float s_thr, s_thr_in;
   __shared__ unsigned int s_mbits[4];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const unsigned long long L = min(st->large_cells, (unsigned long long)cap);
+  const unsigned long long L = min(st->dense_cells, (unsigned long long)cap);
   const unsigned long long J = L ? job_off[L] : 0;
   if ((unsigned long long)blockIdx.x >= J) return;  // no job for this block: no TMEM either
   if (tid < 4) s_tally[tid] = 0;
@@ -1712,13 +1873,6 @@ void brute_impl(const BuildArgs& a, cudaStream_t s) {
                                                       make_sink(a));
 }
 
-// Cells of more points than this go to the tiled kernels (the tuned value, else kMediumMax;
-// never above kMediumMax, the medium kernel's staging capacity).
-inline unsigned int dense_min_of(const BuildArgs& a) {
-  return a.dense_min > 0 && a.dense_min <= kMediumMax ? (unsigned int)a.dense_min
-                                                      : (unsigned int)kMediumMax;
-}
-
 // The dense-cell jobs on the tensor cores (FP16 or BF16 halves), 4 blocks of 128 threads per
 // SM (128 TMEM columns each).
 template <typename K, int DPAD, int MODE>
@@ -1739,6 +1893,70 @@ void large_tc_launch(const BuildArgs& a, const uint32_t* sv, cudaStream_t s) {
   kern<<<(unsigned)(4 * a.num_sms), 128, SM::kBytes, s>>>(
       sv, a.pf, a.dtype, (const K*)a.key_mat, a.m, a.inst, a.iplan, a.st, a.large, a.large_cap,
       a.large_job_off, make_sink(a), spin_limit_of(a.spin_limit) * 16u, a.inject);
+}
+
+// The tile jobs of a build sit in the key buffer that does not hold the sorted keys (its
+// contents are dead after the sort).
+template <typename K>
+TileJob* tile_jobs_of(const BuildArgs& a, int sorted_buf) {
+  return reinterpret_cast<TileJob*>(a.keys[sorted_buf ^ 1]);
+}
+template <typename K>
+unsigned int tile_job_cap(const BuildArgs& a) {
+  return (unsigned int)((size_t)a.n_total * a.m * sizeof(K) / sizeof(TileJob));
+}
+
+template <typename K, int DPAD, int D, int MODE, int STAGE>
+void tiles_launch(const BuildArgs& a, int sorted_buf, cudaStream_t s) {
+  auto kern = k_pairs_tiles<K, DPAD, D, MODE, STAGE>;
+  const int wbytes = tile_region_bytes<K, DPAD>(a.m, STAGE != 0);
+  const size_t smem = (size_t)wbytes * kTileWarps;
+  // one wave of resident blocks (warps claim their jobs)
+  static size_t attr_smem[64] = {};  // largest size granted so far, per device
+  static size_t occ_smem[64] = {};   // size the cached occupancy is for
+  static int occ[64] = {};
+  int dev = 0, per = 2;
+  cudaGetDevice(&dev);
+  {
+    std::lock_guard<std::mutex> lk(launch_attr_mutex());
+    if (dev < 0 || dev >= 64 || smem > attr_smem[dev]) {
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (dev >= 0 && dev < 64) attr_smem[dev] = smem;
+    }
+    if (dev >= 0 && dev < 64) {
+      if (occ_smem[dev] != smem) {
+        int o = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, kTileWarps * 32, smem) !=
+            cudaSuccess)
+          o = 0;
+        occ[dev] = o;
+        occ_smem[dev] = smem;
+      }
+      if (occ[dev] > 0) per = occ[dev];
+    }
+  }
+  kern<<<(unsigned)(per * a.num_sms), kTileWarps * 32, smem, s>>>(
+      a.vals[sorted_buf], a.pf, a.dtype, (const K*)a.key_mat, a.m, a.inst, a.iplan, a.st,
+      tile_jobs_of<K>(a, sorted_buf), tile_job_cap<K>(a),
+      (unsigned int)(a.n_total * a.m), a.B * a.m, make_sink(a), wbytes, &a.st->tile_next[MODE == kWrite ? 1 : 0]);
+}
+
+template <typename K, int DPAD, int D, int MODE>
+void tiles_stage(const BuildArgs& a, int sorted_buf, cudaStream_t s) {
+  const int row = a.m * (int)sizeof(K);
+  if (row > kMaxStagedRow) tiles_launch<K, DPAD, D, MODE, 0>(a, sorted_buf, s);
+  else if (row % 16 == 0) tiles_launch<K, DPAD, D, MODE, 2>(a, sorted_buf, s);
+  else tiles_launch<K, DPAD, D, MODE, 1>(a, sorted_buf, s);
+}
+
+// Coordinates evaluated: the padded width, or less where the widest instance leaves half a
+// vector or more unused (d <= 6 of 8, d <= 12 of 16: the padding is zero).
+template <typename K, int DPAD, int MODE>
+void tiles_dims(const BuildArgs& a, int sorted_buf, cudaStream_t s) {
+  if (DPAD == 8 && a.d_max <= 6) tiles_stage<K, DPAD, DPAD == 8 ? 6 : DPAD, MODE>(a, sorted_buf, s);
+  else if (DPAD == 16 && a.d_max <= 12)
+    tiles_stage<K, DPAD, DPAD == 16 ? 12 : DPAD, MODE>(a, sorted_buf, s);
+  else tiles_stage<K, DPAD, DPAD, MODE>(a, sorted_buf, s);
 }
 
 template <typename K, int DPAD, int MODE>
@@ -1781,39 +1999,13 @@ void pairs_mode(const BuildArgs& a, int sorted_buf, cudaStream_t s) {
   }
   kern<<<(unsigned)blocks, kPairThreads, smem, s>>>(
       sk, sv, N, span, a.pf, a.dtype, (const K*)a.key_mat, a.m, a.inst, a.iplan, a.bases,
-      a.B * a.m, a.st, make_sink(a), a.large, a.large_cap, wbytes,
+      a.B * a.m, a.st, make_sink(a), a.large, a.large_cap, tile_jobs_of<K>(a, sorted_buf),
+      tile_job_cap<K>(a), MODE != kBits && a.tc_cells ? kTcCellMin : kTileCellMax, wbytes,
       &a.st->span_next[MODE == kWrite ? 1 : 0], (a.skip_tail & kSkipDense) ? 1 : 0,
       a.cell_major);
   if (a.skip_tail & kSkipDense) return;  // (k_pairs_warp flags any dense cell it meets)
-  {
-    const size_t msmem =
-        (size_t)kMediumWarps * kMediumMax * (DPAD * 4 + 4) + (size_t)kMediumWarps * kMediumKeyBytes;
-    // one wave of resident blocks (the kernel loops over the cells): a build without medium
-    // cells pays for a single wave of blocks that find nothing to do
-    static bool mattr[64] = {};
-    static int mocc[64] = {};
-    int mper = 2;
-    {
-      std::lock_guard<std::mutex> lk(launch_attr_mutex());
-      if (dev >= 0 && dev < 64 && !mattr[dev]) {
-        cudaFuncSetAttribute(k_pairs_medium<K, DPAD, MODE>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)msmem);
-        int occ = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_pairs_medium<K, DPAD, MODE>,
-                                                          kMediumWarps * 32,
-                                                          msmem) != cudaSuccess)
-          occ = 0;
-        mocc[dev] = occ;
-        mattr[dev] = true;
-      }
-      if (dev >= 0 && dev < 64 && mocc[dev] > 0) mper = mocc[dev];
-    }
-    k_pairs_medium<K, DPAD, MODE><<<(unsigned)(mper * a.num_sms), kMediumWarps * 32, msmem, s>>>(
-        sv, a.pf, a.dtype, (const K*)a.key_mat, a.m, a.inst, a.iplan, a.st, a.large, a.large_cap,
-        make_sink(a), dense_min_of(a));
-  }
-  if (MODE != kWrite)
-    k_large_setup<<<1, 1024, 0, s>>>(a.large, a.large_cap, a.st, a.large_job_off, dense_min_of(a));
+  tiles_dims<K, DPAD, MODE>(a, sorted_buf, s);
+  if (MODE != kWrite) k_large_setup<<<1, 1024, 0, s>>>(a.large, a.large_cap, a.st, a.large_job_off);
   if constexpr (MODE != kBits) {
     if (a.tc_cells) {
       large_tc_launch<K, DPAD, MODE>(a, sv, s);
@@ -1856,6 +2048,9 @@ int launch_pairs(const BuildArgs& a, int sorted_buf, Mode mode, cudaStream_t s) 
 void reset_pairs_state(const BuildArgs& a, cudaStream_t s) {
   cudaMemsetAsync(&a.st->large_cells, 0, sizeof(a.st->large_cells), s);
   cudaMemsetAsync(&a.st->large_jobs, 0, sizeof(a.st->large_jobs), s);
+  cudaMemsetAsync(&a.st->dense_cells, 0, sizeof(a.st->dense_cells), s);
+  cudaMemsetAsync(&a.st->tile_jobs, 0, sizeof(a.st->tile_jobs), s);
+  cudaMemsetAsync(&a.st->tile_next[0], 0, sizeof(a.st->tile_next), s);
   cudaMemsetAsync(&a.st->span_next[0], 0, sizeof(a.st->span_next), s);
   cudaMemsetAsync(&a.st->emitted, 0, sizeof(a.st->emitted), s);
 }

@@ -6,8 +6,7 @@
 // the gaps of direct launches), and keeps the lowest median, per (sorted elements, key bits),
 // in the context and, when RTG_TUNE_CACHE names a file, in a JSON cache shared by later
 // contexts and processes.  The same build also times the in-cell enumeration over spans per
-// warp {1, 2, 4} and the dense-cell threshold {64, 128, 256} on the sorted keys and keeps the
-// fastest (in the context).
+// warp {1, 2, 4} on the sorted keys and keeps the fastest (in the context).
 // The sort is stable in every variant, so the choice never changes a result.
 #include <cuda_runtime.h>
 
@@ -290,10 +289,9 @@ rtg_status tune_sort(rtg_ctx* c, rtg::BuildArgs& a, long long N, int key_bits,
 constexpr float kTunePairsTrialMaxMs = 25.0f;
 
 rtg_status tune_pairs(rtg_ctx* c, rtg::BuildArgs& a, const rtg::SortConfig& cfg, int key_bits,
-                      int* spans_per_warp, int* dense_min) {
+                      int* spans_per_warp) {
   static const int kSpans[] = {1, 2, 4};
-  static const int kDense[] = {64, 128, 256};
-  constexpr int kCands = 9;
+  constexpr int kCands = 3;
   const cudaStream_t st = c->stream;
   rtg::BuildArgs b = a;
   b.skip_tail = 0;  // every kernel of the enumeration is timed
@@ -313,7 +311,6 @@ rtg_status tune_pairs(rtg_ctx* c, rtg::BuildArgs& a, const rtg::SortConfig& cfg,
     // one trial first: an enumeration that takes long keeps the defaults (the trials would
     // cost more than the knobs can save)
     b.spans_per_warp = kSpans[0];
-    b.dense_min = kDense[0];
     rtg::reset_pairs_state(b, st);
     cudaEventRecord(ev[0], st);
     rtg::launch_pairs(b, sorted, rtg::kCount, st);
@@ -324,14 +321,12 @@ rtg_status tune_pairs(rtg_ctx* c, rtg::BuildArgs& a, const rtg::SortConfig& cfg,
       cudaGetLastError();
       for (auto& x : ev) cudaEventDestroy(x);
       *spans_per_warp = 0;
-      *dense_min = 0;
       return RTG_OK;
     }
   }
   for (int rep = 0; rep < kTuneReps; ++rep)
     for (int k = 0; k < kCands; ++k) {
-      b.spans_per_warp = kSpans[k / 3];
-      b.dense_min = kDense[k % 3];
+      b.spans_per_warp = kSpans[k];
       rtg::reset_pairs_state(b, st);
       cudaEventRecord(ev[2 * (rep * kCands + k)], st);
       rtg::launch_pairs(b, sorted, rtg::kCount, st);
@@ -354,8 +349,7 @@ rtg_status tune_pairs(rtg_ctx* c, rtg::BuildArgs& a, const rtg::SortConfig& cfg,
   int k = 0;
   for (int q = 1; q < kCands; ++q)
     if (best[q] < best[k]) k = q;
-  *spans_per_warp = kSpans[k / 3];
-  *dense_min = kDense[k % 3];
+  *spans_per_warp = kSpans[k];
   return RTG_OK;
 }
 
