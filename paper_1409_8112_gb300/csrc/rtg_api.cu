@@ -632,7 +632,8 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
       // before them flag any work that turns up, and the build runs again with them
       if (m > 0 && known)
         a.skip_tail =
-            (g.no_dense ? rtg::kSkipDense : 0) | (g.no_long_rows ? rtg::kSkipLongRows : 0);
+            (g.no_dense ? rtg::kSkipDense : 0) | (g.no_long_rows ? rtg::kSkipLongRows : 0) |
+            (g.no_rows_left ? rtg::kSkipRowsLeft : 0) | (g.no_bitmap ? rtg::kSkipBitmap : 0);
       if ((s = ensure(c, c->pair_buf, (size_t)g.pair_cap * 8)) != RTG_OK) return s;
       a.pair_buf = (unsigned long long*)c->pair_buf.p;
       a.pair_cap = g.pair_cap;
@@ -742,6 +743,7 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
         RTG_CUDA(c, cudaMemsetAsync(a.row_cnt, 0, sizeof(unsigned int) * (size_t)n_total, st));
         RTG_CUDA(c, cudaMemsetAsync(&a.st->long_rows, 0, sizeof(a.st->long_rows), st));
         RTG_CUDA(c, cudaMemsetAsync(&a.st->mid_rows, 0, sizeof(a.st->mid_rows), st));
+        RTG_CUDA(c, cudaMemsetAsync(&a.st->rows_left, 0, sizeof(a.st->rows_left), st));
         set_slot();
         launches += pairs(rtg::kWrite);
         if (timing) RTG_CUDA(c, cudaEventRecord(c->ev[6], st));
@@ -854,6 +856,8 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
       if (h.errors & rtg::kErrTailSkipped) {
         g.no_dense = false;
         g.no_long_rows = false;
+        g.no_rows_left = false;
+        g.no_bitmap = false;
       }
       if (h.errors & rtg::kErrKeyBits) {
         g.key64 = h.sort_bits > 32;
@@ -880,6 +884,8 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
       // with a margin, so that new data of the same shape seldom brings such work back
       g.no_dense = h.max_cell <= (unsigned long long)rtg::kSkipMargin;
       g.no_long_rows = h.rows_over_margin == 0;
+      g.no_rows_left = h.rows_left == 0;
+      g.no_bitmap = h.long_rows == 0;
     }
     if (m > 0 && n_total > 0 && !q.count_only) {
       c->ppp_hint.put(maxd, (double)h.pairs / (double)n_total);

@@ -45,6 +45,8 @@ struct ShapeGuess {
   int spans_per_warp = 0;      // (tuned) spans per resident warp
   bool no_dense = false;       // the last build had no cell of more than 32 points
   bool no_long_rows = false;   // the last build had no row of more than 32 entries
+  bool no_bitmap = false;      // the last build had no row of more than 256 entries
+  bool no_rows_left = false;   // the last build left no row to the block row sort
 };
 
 // A build's launch sequence captured once and replayed for later builds of the same shape.

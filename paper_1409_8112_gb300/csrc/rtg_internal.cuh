@@ -67,6 +67,8 @@ enum : uint32_t {
 // (BuildArgs::skip_tail); the kernels before them flag kErrTailSkipped if work turns up.
 constexpr int kSkipDense = 1;     // the tile, large-cell set-up and large-cell kernels
 constexpr int kSkipLongRows = 2;  // the warp and block row sorts
+constexpr int kSkipRowsLeft = 4;  // the block row sort (no row was left to it)
+constexpr int kSkipBitmap = 8;    // the bitmaps of the warp row sort (no row was queued for them)
 // A shape whose last build had no cell and no row longer than this leaves those kernels (for
 // more than 32 points or entries) out of its next builds; the margin keeps new data of the
 // same shape from flipping the decision often.
@@ -139,6 +141,7 @@ struct Status {
   unsigned int coop_gen;    // single-launch sort: grid barriers completed
   unsigned int long_rows;  // rows queued for the block row sort
   unsigned int mid_rows;   // rows queued for the warp row sort
+  unsigned int rows_left;  // long rows whose columns span more than a warp's bitmap
   unsigned int rows_over_margin;  // 1 if a row holds more than kSkipMargin entries
   unsigned int cell_bits;  // bits of the widest grid's cell index range (set by the plan)
   unsigned int tc_max_err_bits;  // tensor-core path: max |FP32 d^2 - FP64 d^2| (float bits)
@@ -284,7 +287,7 @@ struct BuildArgs {
                             // 1 FP16 halves, 2 BF16 halves
   unsigned int spin_limit;  // bounded waits: iterations before giving up (0: the default)
   unsigned int inject;      // test hooks (kInject*), 0 in normal use
-  int skip_tail;            // kSkipDense | kSkipLongRows: kernels left out of this launch
+  int skip_tail;            // kSkip* bits: kernels left out of this launch
   int scan_zeroed;          // the scan's look-back words were zeroed with the counters
   // Cell-major sort (one instance): the sort key is the cell index alone, the first pass reads
   // a grid-major copy of the cell indices (keys[1], written by the key kernel) with their
