@@ -130,11 +130,12 @@ struct Status {
   unsigned long long key_rechecks;
   unsigned long long dist_rechecks;
   unsigned long long large_cells;
-  unsigned long long dense_cells;  // cells queued for the 128 x 128 tile kernels
   unsigned long long large_jobs;
   unsigned long long max_cell;
   unsigned int sort_tiles[kMaxPasses];
   unsigned int span_next[2];  // pair enumeration: next unclaimed span (count/emit, write)
+  unsigned int tile_cells;    // cells listed for the 32 x 32 tile kernel (front of the list)
+  unsigned int dense_cells;   // cells listed for the 128 x 128 tile kernels (back of the list)
   unsigned int tile_jobs;     // pair enumeration: jobs queued for the 32 x 32 tile kernel
   unsigned int tile_next[2];  // next unclaimed tile job (count/emit, write)
   unsigned int coop_count;  // single-launch sort: blocks arrived at the current grid barrier

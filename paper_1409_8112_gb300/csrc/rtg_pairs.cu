@@ -46,7 +46,7 @@ constexpr int kTL = 128;                   // dense-cell tile (tensor cores, hug
 constexpr int kTcCellMin = 256;            // cells of more points take the tensor-core tiles
                                            // (when a build asks for them)
 constexpr int kTileCellMax = 8192;         // larger cells take k_pairs_large
-constexpr int kTileWarps = 8;              // warps per block of the tile kernel
+constexpr int kTileWarps = 4;              // warps per block of the tile kernel
 
 __device__ __forceinline__ double load_coord(const void* pts, int dtype, long long i, int d,
                                              int l) {
@@ -423,22 +423,21 @@ __device__ long long run_end(const K* __restrict__ skeys, long long N, long long
 // of 32; the job pairs the members of block r = T - 1 - b with those of the blocks
 // [r + a0, r + min(a0 + chunk, b + 1)).
 struct TileJob {
-  unsigned int start, size;       // the cell: first sorted position, points
+  unsigned int cell;  // its entry in the large-cell list
   unsigned short b, a0;
-  unsigned short grid, inst;
 };
 
-// Blocks per job: long enough to keep the fixed block's rows and keys in use, short
-// enough that the last jobs of a launch end together.  A cell of s <= kTileCellMax points
-// makes at most 0.15 s jobs (1152 at 8192 points), which is why the jobs fit the unused key
-// buffer (N / 4 jobs with 32-bit keys).
+// Blocks per job: short, so that the last jobs of a launch end together (jobs of 16 tiles left
+// a third of the warps idle at the end of a clustered build).  A cell of s <= kTileCellMax
+// points makes at most 0.27 s jobs, which is why the jobs fit the unused key buffer (N / 2 jobs
+// with 32-bit keys).
 __device__ __forceinline__ unsigned int tile_job_chunk(unsigned int blocks) {
-  return blocks <= 128 ? 16u : 32u;
+  return blocks <= 64 ? 4u : (blocks <= 128 ? 8u : 16u);
 }
 
 // One lane: appends the jobs of a cell.
-__device__ void append_tile_jobs(TileJob* jobs, unsigned int cap, Status* st, unsigned int start,
-                                 unsigned int size, unsigned int cell) {
+__device__ void append_tile_jobs(TileJob* jobs, unsigned int cap, Status* st, unsigned int cell,
+                                 unsigned int size) {
   const unsigned int T = (size + 31) / 32, A = tile_job_chunk(T), q = T / A, r = T % A;
   // sum over b < T of ceil((b + 1) / A)
   const unsigned int count = A * (q * (q + 1) / 2) + r * (q + 1);
@@ -448,10 +447,7 @@ __device__ void append_tile_jobs(TileJob* jobs, unsigned int cap, Status* st, un
     return;
   }
   TileJob j;
-  j.start = start;
-  j.size = size;
-  j.grid = (unsigned short)(cell & 0xffu);
-  j.inst = (unsigned short)(cell >> 8);
+  j.cell = cell;
   for (unsigned int b = 0; b < T; ++b)
     for (unsigned int a0 = 0; a0 <= b; a0 += A) {
       j.b = (unsigned short)b;
@@ -590,18 +586,18 @@ __global__ void __launch_bounds__(kPairThreads, RTG_PAIRS_MIN_BLOCKS) k_pairs_wa
             if (skip_dense) atomicOr(&st->errors, kErrTailSkipped);
             const unsigned long long size = (unsigned long long)(e - (P0 + p));
             atomicAdd(&st->large_cells, 1ull);
-            if (size <= tile_max) {
-              append_tile_jobs(jobs, job_cap, st, (unsigned int)(P0 + p), (unsigned int)size, cell);
+            // cells for the tile kernel from the front of the list, larger ones from its back
+            const bool tiled = size <= tile_max;
+            const unsigned int slot = atomicAdd(tiled ? &st->tile_cells : &st->dense_cells, 1u);
+            if (slot < large_cap) {
+              LargeCell& lc = large[tiled ? slot : large_cap - 1 - slot];
+              lc.start = (unsigned long long)(P0 + p);
+              lc.size = (unsigned int)size;
+              lc.grid = (unsigned short)(cell & 0xffu);
+              lc.inst = (unsigned short)(cell >> 8);
+              if (tiled) append_tile_jobs(jobs, job_cap, st, slot, (unsigned int)size);
             } else {
-              const unsigned long long slot = atomicAdd(&st->dense_cells, 1ull);
-              if (slot < large_cap) {
-                large[slot].start = (unsigned long long)(P0 + p);
-                large[slot].size = (unsigned int)size;
-                large[slot].grid = (unsigned short)(cell & 0xffu);
-                large[slot].inst = (unsigned short)(cell >> 8);
-              } else {
-                atomicOr(&st->errors, kErrLargeOverflow);
-              }
+              atomicOr(&st->errors, kErrLargeOverflow);
             }
             atomicAdd(&s_gcand[cell & 0xffu], size * (size - 1) / 2);
             maxcell = max(maxcell, (unsigned int)min(size, 0xffffffffull));
@@ -762,12 +758,12 @@ __global__ void __launch_bounds__(1024) k_large_setup(const LargeCell* __restric
                                                       unsigned long long* job_off) {
   __shared__ unsigned long long sbuf[32];
   __shared__ unsigned long long carry;
-  const unsigned long long L = min(st->dense_cells, (unsigned long long)cap);
+  const unsigned long long L = (unsigned long long)min(st->dense_cells, cap);
   if (threadIdx.x == 0) carry = 0;
   __syncthreads();
   for (unsigned long long base = 0; base < L; base += blockDim.x) {
     const unsigned long long e = base + threadIdx.x;
-    const unsigned long long T = e < L ? (large[e].size + kTL - 1) / kTL : 0;
+    const unsigned long long T = e < L ? (large[cap - 1 - e].size + kTL - 1) / kTL : 0;
     const unsigned long long v = T * (T + 1) / 2;
     unsigned long long tot;
     const unsigned long long ex = block_excl_scan64(v, &tot, sbuf);
@@ -782,38 +778,61 @@ __global__ void __launch_bounds__(1024) k_large_setup(const LargeCell* __restric
   }
 }
 
-// Bytes of one warp's shared memory in k_pairs_tiles: staged key rows of the fixed and the
-// walked 32 members (when they are staged), the walked members' FP32 rows, both index lists, the
-// survivors of a tile and the reported pairs held back.
-template <typename K, int DPAD>
+// Floats between staged FP32 rows of D coordinates.
+__host__ __device__ constexpr int tile_row_floats(int D) { return (D + 3) / 4 * 4; }
+
+// Walked tiles staged at a time in k_pairs_tiles: two (the next one copied in while this one is
+// worked on), or one where key rows of more than 64 bytes would cost too many resident warps
+// (m = 20 with 32-bit keys, cells of 33 to 187 points: 407 us with two, 375 with one).
+template <typename K>
+__host__ __device__ inline int tile_buffers(int m) {
+  return m * (int)sizeof(K) <= 64 ? 2 : 1;
+}
+
+// Bytes of one warp's shared memory in k_pairs_tiles: the reported pairs held back, the walked
+// members' FP32 rows, the fixed members' and the walked members' key rows when they are staged,
+// the index lists and the survivors of a tile.
+template <typename K, int D>
 __host__ __device__ inline int tile_region_bytes(int m, bool stage_rows) {
-  const int b = kWarpEmit * 8 + 32 * DPAD * 4 +
-                (stage_rows ? 64 * staged_row_stride<K>(m) * (int)sizeof(K) : 0) + 64 * 4 + 1024 * 2;
+  const int nb = tile_buffers<K>(m);
+  const int b = kWarpEmit * 8 + nb * 32 * tile_row_floats(D) * 4 +
+                (stage_rows ? (1 + nb) * 32 * staged_row_stride<K>(m) * (int)sizeof(K) : 0) +
+                (1 + nb) * 32 * 4 + 1024 * 2;
   return (b + 15) & ~15;
 }
+
+// A tile with more survivors than this (of 1024) takes its ownership test in the walk: one
+// broadcast load of 16 key bytes and their compares for every pair of the tile, against two
+// loads and the compares for every survivor, one per lane.
+constexpr int kWalkOwnerMin = 448;
 
 // Cells of kSmallCell + 1 .. kTileCellMax points, 32 x 32 members at a time, one warp per job
 // (TileJob), jobs claimed from a counter.  A lane keeps one member's FP32 row in registers and
 // walks the later members, whose rows all lanes read at one shared-memory address; the walk
 // only marks the pairs not beyond r (two masks per lane: not beyond, certainly inside), 2 D + 4
-// instructions a pair.  The survivors of the tile are then listed, lane by lane, and taken 32 at
-// a time, one per lane, through the ownership test, the rare FP64 recheck and the emission.
+// instructions a pair.  Where most pairs survive, the ownership test is a second walk over the
+// members' key rows.  The survivors of the tile are then listed, lane by lane, and taken 32 at
+// a time, one per lane, through the ownership test (if it has not been made), the rare FP64
+// recheck and the emission.  The next tile's rows and keys are copied in (cp.async) meanwhile.
 // Members are in point order, so the pairs of a lane share their CSR row and leave together:
 // the scatter takes such a run's slots with one atomic (walking the earlier members instead
 // tripled the scatter's time on clustered points).
 // The kernel this replaced took pairs through all of that at once, one per lane: the lanes
 // whose pair was beyond r waited for the others' ownership tests (211 warp instructions per 32
 // pairs on the Table II workload below).  Bound by instruction issue.  Pairs phase before and
-// after: 100k points in 6-D, m = 20 shift-only grids of 1.35 r (6.7e7 candidates) 1552 -> 342
-// us; clustered, c = r: 100k points in 3-D 956 -> 510 us, 50k in 9-D 3891 -> 2886 us.
-template <typename K, int DPAD, int D, int MODE, int STAGE>
+// after: 100k points in 6-D, m = 20 shift-only grids of 1.35 r (6.7e7 candidates) 1552 -> 375
+// us; clustered, c = r: 100k points in 3-D 956 -> 333 us, 50k in 9-D 3891 -> 1644 us.
+template <typename K, int DPAD, int D, int MODE, bool STAGED>
 __global__ void __launch_bounds__(kTileWarps * 32) k_pairs_tiles(
     const uint32_t* __restrict__ svals, const float* __restrict__ pf, int dtype,
     const K* __restrict__ key_mat, int m, const Inst* __restrict__ inst,
-    const InstPlan* __restrict__ iplan, Status* st, const TileJob* __restrict__ jobs,
-    unsigned int job_cap, unsigned int N, int nbt, Sink sk, int warp_bytes, unsigned int* next) {
+    const InstPlan* __restrict__ iplan, Status* st, const LargeCell* __restrict__ cells,
+    unsigned int cell_cap, const TileJob* __restrict__ jobs, unsigned int job_cap, unsigned int N,
+    int nbt, Sink sk, int warp_bytes, unsigned int* next) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned int s_tally[4];
+  constexpr int RF = tile_row_floats(D);
+  constexpr int KPV = 16 / (int)sizeof(K);  // keys per 16 bytes
   if (st->errors & (kErrTimeout | kErrSortRange | kErrLargeOverflow)) return;
   const unsigned int J = min(st->tile_jobs, job_cap);
   if (J == 0) return;
@@ -823,82 +842,109 @@ __global__ void __launch_bounds__(kTileWarps * 32) k_pairs_tiles(
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   unsigned char* ws = smem + (size_t)wib * warp_bytes;
   unsigned long long* w_emit = reinterpret_cast<unsigned long long*>(ws);
-  float* w_row = reinterpret_cast<float*>(ws + kWarpEmit * 8);
-  K* w_ka = reinterpret_cast<K*>(w_row + 32 * DPAD);  // fixed members' key rows
+  const int nbuf = tile_buffers<K>(m);
+  float* w_row = reinterpret_cast<float*>(ws + kWarpEmit * 8);  // nbuf x 32 rows
+  K* w_ka = reinterpret_cast<K*>(w_row + nbuf * 32 * RF);       // fixed members' key rows
   const int kst = staged_row_stride<K>(m);
-  K* w_kb = w_ka + (STAGE != 0 ? 32 * kst : 0);       // walked members' key rows
-  uint32_t* w_ia = reinterpret_cast<uint32_t*>(w_kb + (STAGE != 0 ? 32 * kst : 0));
-  uint32_t* w_ib = w_ia + 32;
-  unsigned short* w_q = reinterpret_cast<unsigned short*>(w_ib + 32);  // survivors of a tile
+  K* w_kb = w_ka + (STAGED ? 32 * kst : 0);                     // nbuf x 32 walked key rows
+  uint32_t* w_ia = reinterpret_cast<uint32_t*>(w_kb + (STAGED ? nbuf * 32 * kst : 0));
+  uint32_t* w_ib = w_ia + 32;                                   // nbuf x 32
+  unsigned short* w_q = reinterpret_cast<unsigned short*>(w_ib + nbuf * 32);  // survivors
+  const bool rows16 = (m * (int)sizeof(K)) % 16 == 0;  // key rows of whole 16-byte blocks
   unsigned int ecnt = 0;
   Tally tl;
   // copies the first t keys of member idx's key row to dst
   auto stage_keys = [&](K* dst, uint32_t idx, int t) {
     const K* kr = key_mat + (size_t)idx * m;
-    if (STAGE == 2) {
-      constexpr int kpv = 16 / (int)sizeof(K);
-      for (int u = 0; u < t; u += kpv) cp_async16(dst + u, kr + u);
-    } else if (STAGE == 1) {
+    if (rows16) {
+      for (int u = 0; u < t; u += KPV) cp_async16(dst + u, kr + u);
+    } else {
       for (int u = 0; u < t; ++u) cp_async_small<(int)sizeof(K)>(dst + u, kr + u);
     }
   };
-  // the next job is claimed while this one runs
-  unsigned int claim = 0;
+  // the next job is claimed, and its entry read, while this one runs
+  unsigned int claim = 0, job;
   if (lane == 0) claim = atomicAdd(next, 1u);
-  for (;;) {
-    const unsigned int job = __shfl_sync(full, claim, 0);
-    if (job >= J) break;
-    const TileJob jb = jobs[job];
+  job = __shfl_sync(full, claim, 0);
+  TileJob jb = jobs[min(job, J - 1)];
+  for (; job < J;) {
+    const LargeCell cell = cells[min(jb.cell, cell_cap - 1)];
+    const TileJob me = jb;
     if (lane == 0) claim = atomicAdd(next, 1u);
-    const int t = (int)jb.grid;
-    const unsigned int s = jb.size, T = (s + 31) / 32, r = T - 1 - jb.b;
-    if (jb.start + s > N || jb.b >= T || jb.inst >= nbt / m) {  // not a job of this build
-      if (lane == 0) atomicOr(&st->errors, kErrLargeOverflow);
+    const int t = (int)cell.grid;
+    const unsigned int s = cell.size, T = (s + 31) / 32, r = T - 1 - me.b;
+    if (cell.start + s > N || me.b >= T || t >= m || cell.inst >= nbt / m) {
+      if (lane == 0) atomicOr(&st->errors, kErrLargeOverflow);  // not a job of this build
+      job = __shfl_sync(full, claim, 0);
+      jb = jobs[min(job, J - 1)];
       continue;
     }
-    const uint32_t* members = svals + jb.start;
-    const float2 band = band_of(iplan[jb.inst]);
-    float y[D];
-    __syncwarp();  // the previous job's survivors are done with the staged rows
+    const uint32_t* members = svals + cell.start;
+    const float2 band = band_of(iplan[cell.inst]);
+    const Inst* I = inst + cell.inst;
+    const InstPlan* IP = iplan + cell.inst;
+    const unsigned int w0 = r + me.a0, w_end = r + min(me.a0 + tile_job_chunk(T), me.b + 1u);
+    auto member = [&](unsigned int w) { return members[min(32u * w + lane, s - 1)]; };
+    auto stage_tile = [&](unsigned int buf, uint32_t idx) {
+      w_ib[buf * 32 + lane] = idx;
+      const float* src = pf + (size_t)idx * DPAD;
+      float* dst = w_row + (buf * 32 + lane) * RF;
+#pragma unroll
+      for (int v = 0; v < RF / 4; ++v) cp_async16(dst + 4 * v, src + 4 * v);
+      if (STAGED) stage_keys(w_kb + (buf * 32 + lane) * kst, idx, t);
+    };
+    __syncwarp();  // the previous job's last tile is done with everything staged
+    float y[RF];
+    uint32_t idx1 = member(w0);
     {
-      const uint32_t idx = members[min(32u * r + lane, s - 1)];
+      const uint32_t idx = member(r);
       w_ia[lane] = idx;
-      if (STAGE != 0) stage_keys(w_ka + lane * kst, idx, t);
+      if (STAGED) stage_keys(w_ka + lane * kst, idx, t);
       const float4* src = reinterpret_cast<const float4*>(pf + (size_t)idx * DPAD);
 #pragma unroll
-      for (int v = 0; v < (D + 3) / 4; ++v) {
+      for (int v = 0; v < RF / 4; ++v) {
         const float4 q = __ldg(src + v);
         y[4 * v] = q.x;
-        if (4 * v + 1 < D) y[4 * v + 1] = q.y;
-        if (4 * v + 2 < D) y[4 * v + 2] = q.z;
-        if (4 * v + 3 < D) y[4 * v + 3] = q.w;
+        y[4 * v + 1] = q.y;
+        y[4 * v + 2] = q.z;
+        y[4 * v + 3] = q.w;
       }
     }
-    const unsigned int w_end = r + min(jb.a0 + tile_job_chunk(T), jb.b + 1u);
-    uint32_t idx_next = members[min(32u * (r + jb.a0) + lane, s - 1)];
-    for (unsigned int w = r + jb.a0; w < w_end; ++w) {
-      __syncwarp();  // the previous tile's survivors are done with the walked members
-      {
-        const uint32_t idx = idx_next;
-        w_ib[lane] = idx;
-        const float* src = pf + (size_t)idx * DPAD;
-#pragma unroll
-        for (int v = 0; v < (D + 3) / 4; ++v) cp_async16(w_row + lane * DPAD + 4 * v, src + 4 * v);
-        if (STAGE != 0) stage_keys(w_kb + lane * kst, idx, t);
-        if (w + 1 < w_end) idx_next = members[min(32u * (w + 1) + lane, s - 1)];
+    if (nbuf == 2) {
+      stage_tile(w0 & 1u, idx1);
+      cp_async_commit();
+      idx1 = member(w0 + 1);
+    }
+    for (unsigned int w = w0; w < w_end; ++w) {
+      const unsigned int buf = nbuf == 2 ? w & 1u : 0u;
+      if (nbuf == 2) {
+        const uint32_t idx2 = member(w + 2);
+        if (w + 1 < w_end) stage_tile(buf ^ 1u, idx1);  // (last read before the previous barrier)
+        cp_async_commit();
+        idx1 = idx2;
+        cp_async_wait<1>();  // this tile's copies have landed
+      } else {
+        stage_tile(0u, idx1);
+        idx1 = member(w + 1);
+        cp_async_wait_all();
       }
-      cp_async_wait_all();
+      if (w == w0) {
+        job = __shfl_sync(full, claim, 0);
+        jb = jobs[min(job, J - 1)];
+      }
       __syncwarp();
+      const float* rows = w_row + buf * 32 * RF;
+      const K* kb_rows = w_kb + (STAGED ? buf * 32 * kst : 0);
       const int nw = (int)min(32u, s - 32u * w);  // only the cell's last block is short
       unsigned int hits = 0, sure = 0;  // walked members not beyond r, certainly within r
       for (int x0 = 0; x0 < nw; x0 += 8) {
         unsigned int h8 = 0, s8 = 0;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-          const float* xr = w_row + (x0 + q) * DPAD;
+          const float* xr = rows + (x0 + q) * RF;
           float sf = 0.0f;
 #pragma unroll
-          for (int v = 0; v < (D + 3) / 4; ++v) {
+          for (int v = 0; v < RF / 4; ++v) {
             const float4 x = reinterpret_cast<const float4*>(xr)[v];
             float e = x.x - y[4 * v];
             sf = fmaf(e, e, sf);
@@ -923,6 +969,36 @@ __global__ void __launch_bounds__(kTileWarps * 32) k_pairs_tiles(
       }
       if (nw < 32) hits &= (1u << nw) - 1u;
       if (w == r) hits &= ~((2u << lane) - 1u);  // a block with itself: later members only
+      int t_left = t;  // earlier grids still to compare for each survivor
+      if (STAGED && MODE != kBits && t > 0 &&
+          __reduce_add_sync(full, (unsigned int)__popc(hits)) > (unsigned int)kWalkOwnerMin) {
+        unsigned int early = 0;  // walked members some earlier grid puts in the lane's cell
+        for (int u0 = 0; u0 < t; u0 += KPV) {
+          K o[KPV];
+          {
+            const uint4 v = *reinterpret_cast<const uint4*>(w_ka + lane * kst + u0);
+            const K* ok = reinterpret_cast<const K*>(&v);
+#pragma unroll
+            for (int z = 0; z < KPV; ++z) o[z] = ok[z];
+          }
+          const int left = t - u0;
+          for (int x0 = 0; x0 < nw; x0 += 8) {
+            unsigned int e8 = 0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              const uint4 v = *reinterpret_cast<const uint4*>(kb_rows + (x0 + q) * kst + u0);
+              const K* xk = reinterpret_cast<const K*>(&v);
+              bool same = xk[0] == o[0];
+#pragma unroll
+              for (int z = 1; z < KPV; ++z) same |= z < left && xk[z] == o[z];
+              if (same) e8 |= 1u << q;
+            }
+            early |= e8 << x0;
+          }
+        }
+        hits &= ~early;
+        t_left = 0;
+      }
       // list the survivors: (certain, walked member, fixed member)
       const int nh = __popc(hits);
       int incl = nh;
@@ -948,21 +1024,22 @@ __global__ void __launch_bounds__(kTileWarps * 32) k_pairs_tiles(
         unsigned int i = 0, j = 0;
         if (base + lane < total) {
           const unsigned int e = w_q[base + lane], x = (e >> 5) & 31u, c = e & 31u;
-          const uint32_t ia = w_ia[c], ib = w_ib[x];
+          const uint32_t ia = w_ia[c], ib = w_ib[buf * 32 + x];
           i = min(ia, ib);
           j = max(ia, ib);
-          const K* ka = STAGE != 0 ? w_ka + c * kst : key_mat + (size_t)ia * m;
-          const K* kb = STAGE != 0 ? w_kb + x * kst : key_mat + (size_t)ib * m;
-          keep = decide_survivor<K, MODE, STAGE != 0>((e >> 10) != 0u, i, j, t, ka, kb,
-                                                      inst + jb.inst, iplan + jb.inst, dtype, tl,
-                                                      sk.near_r);
+          const K* ka = STAGED ? w_ka + c * kst : key_mat + (size_t)ia * m;
+          const K* kb = STAGED ? kb_rows + x * kst : key_mat + (size_t)ib * m;
+          keep = decide_survivor<K, MODE, STAGED>((e >> 10) != 0u, i, j, t_left, ka, kb, I, IP,
+                                                  dtype, tl, sk.near_r);
         }
-        if (MODE == kBits) deliver_bits(keep, i, j, inst + jb.inst, sk);
+        if (MODE == kBits) deliver_bits(keep, i, j, I, sk);
         else if (MODE == kEmit) warp_emit_runs(keep, i, j, w_emit, ecnt, sk);
         else deliver<MODE>(keep, i, j, sk, tl);
       }
+      __syncwarp();  // everybody is done with this tile's buffer
     }
   }
+  cp_async_wait<0>();
   if (MODE == kEmit && ecnt) warp_flush(w_emit, ecnt, sk);
   __syncthreads();
   flush_tally<MODE>(tl, st, s_tally);
@@ -988,7 +1065,7 @@ __global__ void __launch_bounds__(kPairThreads) k_pairs_large(
   __shared__ unsigned long long s_emit[kPairThreads / 32][kWarpEmit];
   __shared__ unsigned int s_tally[4];
   if (threadIdx.x < 4) s_tally[threadIdx.x] = 0;
-  const unsigned long long L = min(st->dense_cells, (unsigned long long)cap);
+  const unsigned long long L = (unsigned long long)min(st->dense_cells, cap);
   const unsigned long long J = L ? job_off[L] : 0;
   unsigned long long* w_emit = s_emit[threadIdx.x >> 5];
   unsigned int ecnt = 0;
@@ -999,7 +1076,7 @@ __global__ void __launch_bounds__(kPairThreads) k_pairs_large(
       const long long mid = (el + eh + 1) >> 1;
       if (job_off[mid] <= job) el = mid; else eh = mid - 1;
     }
-    const LargeCell cell = large[el];
+    const LargeCell cell = large[cap - 1 - el];
     const float2 band = band_of(iplan[cell.inst]);
     const unsigned int s = cell.size;
     // tile pair (bi <= bj) of this cell
@@ -1108,7 +1185,7 @@ __global__ void __launch_bounds__(128) k_pairs_large_tc(
   __shared__ float s_thr, s_thr_in;
   __shared__ unsigned int s_mbits[4];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const unsigned long long L = min(st->dense_cells, (unsigned long long)cap);
+  const unsigned long long L = (unsigned long long)min(st->dense_cells, cap);
   const unsigned long long J = L ? job_off[L] : 0;
   if ((unsigned long long)blockIdx.x >= J) return;  // no job for this block: no TMEM either
   if (tid < 4) s_tally[tid] = 0;
@@ -1138,7 +1215,7 @@ __global__ void __launch_bounds__(128) k_pairs_large_tc(
       const long long mid = (el + eh + 1) >> 1;
       if (job_off[mid] <= job) el = mid; else eh = mid - 1;
     }
-    const LargeCell cell = large[el];
+    const LargeCell cell = large[cap - 1 - el];
     const Inst& I = inst[cell.inst];
     const int d = I.d;
     const float2 band = band_of(iplan[cell.inst]);
@@ -2026,10 +2103,10 @@ unsigned int tile_job_cap(const BuildArgs& a) {
   return (unsigned int)((size_t)a.n_total * a.m * sizeof(K) / sizeof(TileJob));
 }
 
-template <typename K, int DPAD, int D, int MODE, int STAGE>
+template <typename K, int DPAD, int D, int MODE, bool STAGED>
 void tiles_launch(const BuildArgs& a, int sorted_buf, cudaStream_t s) {
-  auto kern = k_pairs_tiles<K, DPAD, D, MODE, STAGE>;
-  const int wbytes = tile_region_bytes<K, DPAD>(a.m, STAGE != 0);
+  auto kern = k_pairs_tiles<K, DPAD, D, MODE, STAGED>;
+  const int wbytes = tile_region_bytes<K, D>(a.m, STAGED);
   const size_t smem = (size_t)wbytes * kTileWarps;
   // one wave of resident blocks (warps claim their jobs)
   static size_t attr_smem[64] = {};  // largest size granted so far, per device
@@ -2057,26 +2134,31 @@ void tiles_launch(const BuildArgs& a, int sorted_buf, cudaStream_t s) {
   }
   kern<<<(unsigned)(per * a.num_sms), kTileWarps * 32, smem, s>>>(
       a.vals[sorted_buf], a.pf, a.dtype, (const K*)a.key_mat, a.m, a.inst, a.iplan, a.st,
-      tile_jobs_of<K>(a, sorted_buf), tile_job_cap<K>(a),
+      a.large, a.large_cap, tile_jobs_of<K>(a, sorted_buf), tile_job_cap<K>(a),
       (unsigned int)(a.n_total * a.m), a.B * a.m, make_sink(a), wbytes, &a.st->tile_next[MODE == kWrite ? 1 : 0]);
 }
 
 template <typename K, int DPAD, int D, int MODE>
 void tiles_stage(const BuildArgs& a, int sorted_buf, cudaStream_t s) {
-  const int row = a.m * (int)sizeof(K);
-  if (row > kMaxStagedRow) tiles_launch<K, DPAD, D, MODE, 0>(a, sorted_buf, s);
-  else if (row % 16 == 0) tiles_launch<K, DPAD, D, MODE, 2>(a, sorted_buf, s);
-  else tiles_launch<K, DPAD, D, MODE, 1>(a, sorted_buf, s);
+  if (a.m * (int)sizeof(K) > kMaxStagedRow) tiles_launch<K, DPAD, D, MODE, false>(a, sorted_buf, s);
+  else tiles_launch<K, DPAD, D, MODE, true>(a, sorted_buf, s);
 }
 
-// Coordinates evaluated: the padded width, or less where the widest instance leaves half a
-// vector or more unused (d <= 6 of 8, d <= 12 of 16: the padding is zero).
+// Coordinates evaluated: the widest instance's d, rounded up to the compiled widths (the
+// padding is zero).
 template <typename K, int DPAD, int MODE>
 void tiles_dims(const BuildArgs& a, int sorted_buf, cudaStream_t s) {
-  if (DPAD == 8 && a.d_max <= 6) tiles_stage<K, DPAD, DPAD == 8 ? 6 : DPAD, MODE>(a, sorted_buf, s);
-  else if (DPAD == 16 && a.d_max <= 12)
-    tiles_stage<K, DPAD, DPAD == 16 ? 12 : DPAD, MODE>(a, sorted_buf, s);
-  else tiles_stage<K, DPAD, DPAD, MODE>(a, sorted_buf, s);
+  if constexpr (DPAD == 4) {
+    if (a.d_max <= 3) tiles_stage<K, 4, 3, MODE>(a, sorted_buf, s);
+    else tiles_stage<K, 4, 4, MODE>(a, sorted_buf, s);
+  } else if constexpr (DPAD == 8) {
+    if (a.d_max <= 6) tiles_stage<K, 8, 6, MODE>(a, sorted_buf, s);
+    else tiles_stage<K, 8, 8, MODE>(a, sorted_buf, s);
+  } else {
+    if (a.d_max <= 9) tiles_stage<K, 16, 9, MODE>(a, sorted_buf, s);
+    else if (a.d_max <= 12) tiles_stage<K, 16, 12, MODE>(a, sorted_buf, s);
+    else tiles_stage<K, 16, 16, MODE>(a, sorted_buf, s);
+  }
 }
 
 template <typename K, int DPAD, int MODE>
@@ -2169,6 +2251,7 @@ void reset_pairs_state(const BuildArgs& a, cudaStream_t s) {
   cudaMemsetAsync(&a.st->large_cells, 0, sizeof(a.st->large_cells), s);
   cudaMemsetAsync(&a.st->large_jobs, 0, sizeof(a.st->large_jobs), s);
   cudaMemsetAsync(&a.st->dense_cells, 0, sizeof(a.st->dense_cells), s);
+  cudaMemsetAsync(&a.st->tile_cells, 0, sizeof(a.st->tile_cells), s);
   cudaMemsetAsync(&a.st->tile_jobs, 0, sizeof(a.st->tile_jobs), s);
   cudaMemsetAsync(&a.st->tile_next[0], 0, sizeof(a.st->tile_next), s);
   cudaMemsetAsync(&a.st->span_next[0], 0, sizeof(a.st->span_next), s);
