@@ -5,8 +5,10 @@
 // set is the same as the FP64 definition's.
 //
 // Each coordinate is centred on the bounding box and split as x = hi + lo (both half
-// precision); x.y is approximated by hi.hi + hi.lo + lo.hi, three K = 16 MMAs per tile pair
-// (d <= 16 padded with zeros).  Operands sit in shared memory in the K-major layout without
+// precision); x.y is approximated by hi.hi + hi.lo + lo.hi.  For d <= 9 the three products and
+// the norms share one row of 32 halves (one or two K = 16 MMAs per tile pair); for d <= 12 the
+// norms ride in the hi block of three MMAs; beyond, three MMAs give x.y and the epilogue adds
+// the norms.  Operands sit in shared memory in the K-major layout without
 // swizzle: core matrices of 8 rows x 16 bytes, 128 bytes apart along K and 512 bytes apart
 // along M or N.  A CTA of 4 warps owns a 128 x 128 FP32 accumulator (128 TMEM columns);
 // warp w reads lanes 32w..32w+31.  The band is max(1e-3 r^2, E) where E bounds the error of
@@ -16,6 +18,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cfloat>
 #include <type_traits>
 
@@ -29,7 +32,11 @@ namespace {
 constexpr int kTcRows = 128;
 constexpr int kTcK = 32;                          // hi (16) + lo (16)
 constexpr int kTcTileBytes = kTcRows * kTcK * 2;  // 8 KB per 128-point tile
-constexpr int kTcThreads = 128;
+// Epilogue warps, one TMEM load in flight each: a probe of tcgen05.ld.32x32b.x32 read 249 bytes
+// a clock and SM with 4 warps, 323 with 8 and 60 with 16 (two loads in flight: 235 with 8).
+constexpr int kTcEpiWarps = 8;
+constexpr int kTcThreads = (kTcEpiWarps + 2) * 32;  // and one that copies tiles, one for the MMAs
+constexpr int kTcSlots = 4;                       // column tiles in shared memory
 // MMA completion waits: the context's spin limit times this (a commit takes far longer than
 // one look-back step)
 constexpr unsigned int kTcWaitScale = 16;
@@ -70,11 +77,19 @@ __global__ void k_tc_plan(const Inst* __restrict__ inst, const unsigned long lon
   tp->hi = __double2float_ru(rr + band);
 }
 
-// Half-precision hi/lo rows in the tile layout, and FP32 norms of the centred points.  FOLD
-// (d <= 12): the tiles come in two versions, the A operand's ([-2 x, |x|^2 hi, |x|^2 lo, 1, 1]
-// in the hi block) and the B operand's ([x, 1, 1, |y|^2 hi, |y|^2 lo]), so that the MMAs
-// accumulate |x|^2 + |y|^2 - 2 x.y; the norms array is then not read.
-template <bool BF16, bool FOLD>
+// What the operand rows hold.  kTcPlain: [hi | lo], 16 halves each.  kTcFold (d <= 12): the
+// tiles come in two versions, the A operand's ([-2 x, |x|^2 hi, |x|^2 lo, 1, 1] in the hi block)
+// and the B operand's ([x, 1, 1, |y|^2 hi, |y|^2 lo]), so that the MMAs accumulate
+// |x|^2 + |y|^2 - 2 x.y.  kTcPacked (3 d + 4 <= 32): A = [-2 hi, -2 hi, -2 lo, |x|^2 hi, |x|^2 lo,
+// 1, 1] against B = [hi, lo, hi, 1, 1, |y|^2 hi, |y|^2 lo] in consecutive slots: the same
+// products in two K = 16 MMAs instead of three (one for d <= 4), 64 of the 192 clocks a tile
+// pair holds the tensor pipe.
+enum TcForm : int { kTcPlain = 0, kTcFold = 1, kTcPacked = 2 };
+inline TcForm tc_form(int d) { return d >= 1 && d <= 9 ? kTcPacked : (d <= 12 ? kTcFold : kTcPlain); }
+
+// Half-precision rows in the tile layout, and FP32 norms of the centred points (read by the
+// plain form only).
+template <bool BF16, int FORM>
 __global__ void __launch_bounds__(256) k_tc_prep(const Inst* __restrict__ inst, int dtype,
                                                  const TcPlan* __restrict__ tp,
                                                  unsigned char* __restrict__ tiles,
@@ -91,35 +106,53 @@ __global__ void __launch_bounds__(256) k_tc_prep(const Inst* __restrict__ inst, 
   if (i >= n_pad) return;
   const long long ntile = n_pad / kTcRows;
   unsigned char* tile = tiles + (i / kTcRows) * (long long)kTcTileBytes;
-  unsigned char* tileB = FOLD ? tile + ntile * (long long)kTcTileBytes : tile;
+  unsigned char* tileB = FORM != kTcPlain ? tile + ntile * (long long)kTcTileBytes : tile;
   const int m = (int)(i % kTcRows);
+  const int d = I.d;
+  auto put = [&](unsigned char* t, int k, H v) { *reinterpret_cast<H*>(t + tile_off(m, k)) = v; };
   float nrm = 0.0f;
-  for (int k = 0; k < 16; ++k) {
+  const int width = FORM == kTcPacked ? d : 16;
+  for (int k = 0; k < width; ++k) {
     float xc = 0.0f;
-    if (i < I.n && k < I.d)
-      xc = __double2float_rn(__dsub_rn(load_coord(I.pts, dtype, i, I.d, k), tp->center[k]));
+    if (i < I.n && k < d)
+      xc = __double2float_rn(__dsub_rn(load_coord(I.pts, dtype, i, d, k), tp->center[k]));
     nrm = fmaf(xc, xc, nrm);
     const H h = to_h(xc);
     const H l = to_h(xc - to_f(h));
     // A version: -2 x (exact scaling by a power of two)
-    *reinterpret_cast<H*>(tile + tile_off(m, k)) = FOLD ? to_h(-2.0f * to_f(h)) : h;
-    *reinterpret_cast<H*>(tile + tile_off(m, 16 + k)) = FOLD ? to_h(-2.0f * to_f(l)) : l;
-    if (FOLD) {
-      *reinterpret_cast<H*>(tileB + tile_off(m, k)) = h;
-      *reinterpret_cast<H*>(tileB + tile_off(m, 16 + k)) = l;
+    const H h2 = to_h(-2.0f * to_f(h)), l2 = to_h(-2.0f * to_f(l));
+    if (FORM == kTcPacked) {
+      put(tile, k, h2);
+      put(tile, d + k, h2);
+      put(tile, 2 * d + k, l2);
+      put(tileB, k, h);
+      put(tileB, d + k, l);
+      put(tileB, 2 * d + k, h);
+    } else {
+      put(tile, k, FORM == kTcFold ? h2 : h);
+      put(tile, 16 + k, FORM == kTcFold ? l2 : l);
+      if (FORM == kTcFold) {
+        put(tileB, k, h);
+        put(tileB, 16 + k, l);
+      }
     }
   }
-  if (FOLD) {
-    const int d = I.d;  // slots d .. d + 3 of the hi block are free (d <= 12)
+  if (FORM != kTcPlain) {
+    const int q = FORM == kTcPacked ? 3 * d : d;  // the four slots of the norms
     const H nh = to_h(nrm), nl = to_h(nrm - to_f(nh)), one = to_h(1.0f);
-    *reinterpret_cast<H*>(tile + tile_off(m, d)) = nh;
-    *reinterpret_cast<H*>(tile + tile_off(m, d + 1)) = nl;
-    *reinterpret_cast<H*>(tile + tile_off(m, d + 2)) = one;
-    *reinterpret_cast<H*>(tile + tile_off(m, d + 3)) = one;
-    *reinterpret_cast<H*>(tileB + tile_off(m, d)) = one;
-    *reinterpret_cast<H*>(tileB + tile_off(m, d + 1)) = one;
-    *reinterpret_cast<H*>(tileB + tile_off(m, d + 2)) = nh;
-    *reinterpret_cast<H*>(tileB + tile_off(m, d + 3)) = nl;
+    put(tile, q, nh);
+    put(tile, q + 1, nl);
+    put(tile, q + 2, one);
+    put(tile, q + 3, one);
+    put(tileB, q, one);
+    put(tileB, q + 1, one);
+    put(tileB, q + 2, nh);
+    put(tileB, q + 3, nl);
+    if (FORM == kTcPacked)
+      for (int k = q + 4; k < kTcK; ++k) {
+        put(tile, k, to_h(0.0f));
+        put(tileB, k, to_h(0.0f));
+      }
   }
   norms[i] = nrm;
 }
@@ -151,8 +184,10 @@ __device__ __noinline__ void tc_candidate(float d2, long long gi, long long gj, 
                                           float& max_err, bool& overflow) {
   const double s = exact_dist2(I.pts, dtype, gi, gj, I.d);
   max_err = fmaxf(max_err, (float)fabs((double)d2 - s));
-  if (d2 >= lo_thr) ++rechecks;
-  if (fabs(__dsub_rn(__dsqrt_rn(s), I.r)) <= __dmul_rn(1e-12, I.r)) ++near_r;
+  if (!(d2 < lo_thr)) {  // (every pair within 1e-12 r of r lies in the band: it is 1e-3 r^2 wide)
+    ++rechecks;
+    if (fabs(__dsub_rn(__dsqrt_rn(s), I.r)) <= __dmul_rn(1e-12, I.r)) ++near_r;
+  }
   if (!(s <= IP.rr)) return;
   ++pairs;
   const unsigned int i = (unsigned int)(I.p0 + gi), j = (unsigned int)(I.p0 + gj);
@@ -165,9 +200,11 @@ __device__ __noinline__ void tc_candidate(float d2, long long gi, long long gj, 
   if (sk.symmetric) atomicAdd(&sk.row_cnt[j], 1u);
 }
 
-// Candidates queued per warp before their exact check.  A chunk with more candidates than this
-// (dense inputs: up to 32 x 32) is decided by its lanes directly.
-constexpr int kTcQueue = 256 + 32;
+// Candidates queued per warp before their exact check.  A check waits on the points' loads for
+// about two microseconds, and the accumulators wait with it, so a warp collects many: the
+// warps of a CTA then mostly check at the same time (at the end, at 200k points).  A chunk with
+// more candidates than this (dense inputs: up to 32 x 32) is decided by its lanes directly.
+constexpr int kTcQueue = 768;
 
 // Decides the qn queued candidates of a warp, 32 at a time (one per lane).  Called by all lanes.
 __device__ __forceinline__ void tc_drain(const unsigned int* q_i, const unsigned int* q_j,
@@ -186,48 +223,140 @@ __device__ __forceinline__ void tc_drain(const unsigned int* q_i, const unsigned
   __syncwarp();
 }
 
-// Persistent: each CTA walks a contiguous range of tile pairs (bi <= bj) in bi-major order,
-// so the A tile is reloaded only when bi changes.
-template <bool BF16, bool EMIT, bool FOLD>
-__global__ void __launch_bounds__(kTcThreads) k_brute_tc(
+// The smaller of three values, NaN if any is NaN.
+__device__ __forceinline__ float min3_nan(float a, float b, float c) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
+// Bounded wait that also ends when another thread of the block has given up.
+__device__ __forceinline__ bool tc_wait(const uint64_t* bar, uint32_t parity, unsigned int limit,
+                                        volatile int* late) {
+  const uint32_t addr = smem_u32(bar);
+  for (unsigned int it = 0; it < limit; ++it) {
+    uint32_t ok;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(addr), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if (*late) return false;
+  }
+  *late = 1;
+  return false;
+}
+
+// One thread: copy `bytes` (a multiple of 16, both ends 16-byte aligned) to shared memory,
+// counted on bar (whose expected bytes the caller has set).
+__device__ __forceinline__ void tc_bulk_copy(void* dst, const void* src, uint32_t bytes,
+                                             const uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
+          "r"(smem_u32(dst)),
+      "l"(src), "r"(bytes), "r"(smem_u32(bar))
+      : "memory");
+}
+__device__ __forceinline__ void tc_expect(const uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
+               "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void tc_commit(const uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+          smem_u32(bar))
+      : "memory");
+}
+
+// Jobs of the brute force: 256 rows (row tiles 2 I and 2 I + 1) against the 128 columns of tile
+// bj >= 2 I, I-major.  First job of I.
+__host__ __device__ inline long long tc_first_job(long long I, long long nt) {
+  return I * nt - I * (I - 1);
+}
+
+__host__ __device__ inline long long tc_jobs(long long nt) {
+  // sum over I < ceil(nt / 2) of nt - 2 I
+  const long long nI = (nt + 1) / 2;
+  return nI * nt - nI * (nI - 1);
+}
+
+// Shared memory of k_brute_tc: two pairs of row tiles, the column tiles, the candidate queues.
+constexpr size_t kTcSmem = (4 + kTcSlots) * (size_t)kTcTileBytes +
+                           (size_t)kTcEpiWarps * 3 * kTcQueue * 4 + 1024;
+
+// One lane of a converged warp.
+__device__ __forceinline__ bool tc_elect() {
+  uint32_t e;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+  return e != 0u;
+}
+
+// Persistent, one CTA per SM, each with a contiguous range of jobs.  One warp copies the tiles in
+// (bulk copies: column tiles up to kTcSlots jobs ahead, row tiles one change ahead), one issues
+// the MMAs: a job's two 128 x 128 accumulators are two of four, so that the MMAs of one overlap
+// the reads of the others.  Both run their loops as whole warps and elect a lane for the copies
+// and MMAs (a single lane running the loop, copies included, took 1500 clocks a job).  Eight
+// epilogue warps read the accumulators: warp w the rows of its quadrant w % 4 of row tile w / 4,
+// in four loads of 32 columns kept in registers; then the accumulator is free again.  No block
+// barrier in the loop.
+// An epilogue chunk of 32 columns is first reduced to its smallest d^2 with three-input minima
+// (16 instructions for 32 values); only a chunk that holds a value not above the threshold (one
+// in eleven at 200k points, degree 24) builds the mask of its candidates.  A job of 256 rows
+// halves what the column tiles cost in L2 bandwidth (8 KB a job: 8 KB per 128 rows would be
+// near 60 bytes a clock and SM).
+// 200k points in 6-D (2e10 pair tests), FP16: 7.26 ms with 128 x 128 jobs, 4 CTAs per SM, block
+// barriers and a mask for every chunk; 4.27 now, of which the candidates take 1.5 and the
+// waits of a job (an accumulator handed to the epilogue and back) most of the rest.
+template <bool BF16, bool EMIT, int FORM>
+__global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
     const unsigned char* __restrict__ tiles, const float* __restrict__ norms,
     const Inst* __restrict__ inst, const InstPlan* __restrict__ iplan,
     const TcPlan* __restrict__ tp, int dtype, Status* st, TcSink sk, long long nt,
     unsigned int wait_limit, unsigned int inject) {
   extern __shared__ __align__(1024) unsigned char smem[];
-  // double-buffered operand tiles and norms: the next job's are copied in while this job's
-  // MMAs and epilogue run
-  unsigned char* sa2 = smem;                                         // 2 x 8 KB
-  unsigned char* sb2 = smem + 2 * kTcTileBytes;                      // 2 x 8 KB
-  float* na2 = reinterpret_cast<float*>(smem + 4 * kTcTileBytes);   // 2 x 128
-  float* nb2 = na2 + 2 * kTcRows;                                    // 2 x 128
-  const float* nb = nullptr;  // this job's column norms
-  // per warp: the candidate queue (rows, columns, tile d^2), after the norms
-  unsigned int* q_i = reinterpret_cast<unsigned int*>(nb2 + 2 * kTcRows) +
-                      (size_t)(threadIdx.x >> 5) * 3 * kTcQueue;
-  unsigned int* q_j = q_i + kTcQueue;
-  float* q_d = reinterpret_cast<float*>(q_j + kTcQueue);
-  unsigned int qn = 0;  // entries queued (warp-uniform)
-  __shared__ __align__(8) uint64_t mbar;
-  __shared__ __align__(8) uint64_t mbar_idle;  // test hook: a barrier nothing arrives on
+  unsigned char* s_a = smem;                      // row tiles 2 I, 2 I + 1, of two I
+  unsigned char* s_b = smem + 4 * kTcTileBytes;   // kTcSlots column tiles
+  __shared__ __align__(8) uint64_t b_full[kTcSlots], b_empty[kTcSlots], acc_full[4], acc_empty[4],
+      a_full[2], a_empty[2], all_done, b_idle;  // b_idle: test hook, a barrier nothing arrives on
   __shared__ uint32_t tmem_base;
   __shared__ unsigned int s_cnt[4];
   __shared__ unsigned int s_err;
+  __shared__ int s_late;  // some wait ran out
+  const unsigned int full = 0xffffffffu;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const Inst I = inst[0];
-  const InstPlan IP = iplan[0];
-  const float lo_thr = tp->lo, hi_thr = tp->hi;
-  const long long n = I.n;
-
+  const long long nI = (nt + 1) / 2;
+  const long long jobs = tc_jobs(nt);
+  const long long per = (jobs + gridDim.x - 1) / gridDim.x;
+  const long long j0 = min(jobs, (long long)blockIdx.x * per), j1 = min(jobs, j0 + per);
   if (tid < 4) s_cnt[tid] = 0;
   if (tid == 0) {
     s_err = 0;
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar)));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar_idle)));
+    s_late = 0;
+    auto init = [](const uint64_t* bar, int count) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
+    };
+    for (int q = 0; q < kTcSlots; ++q) {
+      init(&b_full[q], 1);
+      init(&b_empty[q], 1);
+    }
+    for (int q = 0; q < 4; ++q) {
+      init(&acc_full[q], 1);
+      init(&acc_empty[q], kTcEpiWarps / 2);
+    }
+    for (int q = 0; q < 2; ++q) {
+      init(&a_full[q], 1);
+      init(&a_empty[q], 1);
+    }
+    init(&all_done, 1);
+    init(&b_idle, 1);
     asm volatile("fence.mbarrier_init.release.cluster;");
+    asm volatile("fence.proxy.async.shared::cta;");
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 128;" ::"r"(
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
         smem_u32(&tmem_base)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
@@ -235,199 +364,296 @@ __global__ void __launch_bounds__(kTcThreads) k_brute_tc(
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = tmem_base;
-  const uint32_t idesc = (1u << 4) | ((BF16 ? 1u : 0u) << 7) | ((BF16 ? 1u : 0u) << 10) |
-                         ((128u >> 3) << 17) | ((128u >> 4) << 24);
-
-  const long long jobs = nt * (nt + 1) / 2;
-  const long long per = (jobs + gridDim.x - 1) / gridDim.x;
-  const long long j0 = (long long)blockIdx.x * per, j1 = min(jobs, j0 + per);
-  // first (bi, bj) of this CTA: bi-major order over the upper triangle
-  long long bi = 0, bj = 0;
+  // first (I, bj) of this CTA
+  long long I0 = 0, bj0 = 0;
   if (j0 < j1) {
-    long long lo = 0, hi = nt - 1;
-    while (lo < hi) {  // largest bi whose first job index is <= j0
+    long long lo = 0, hi = nI - 1;
+    while (lo < hi) {  // the last I whose first job is <= j0
       const long long mid = (lo + hi + 1) >> 1;
-      if (mid * nt - mid * (mid - 1) / 2 <= j0) lo = mid; else hi = mid - 1;
+      if (tc_first_job(mid, nt) <= j0) lo = mid; else hi = mid - 1;
     }
-    bi = lo;
-    bj = bi + (j0 - (bi * nt - bi * (bi - 1) / 2));
+    I0 = lo;
+    bj0 = 2 * lo + (j0 - tc_first_job(lo, nt));
   }
-  uint32_t phase = 0;
-  bool timed_out = false;
-  unsigned int tl_pairs = 0, tl_rechecks = 0, tl_near = 0;
-  bool overflow = false;
-  float max_err = 0.0f;
-  // asynchronous copy of tile t and its norms into buffer `buf` of a side (16-byte copies)
-  // (FOLD: the B operand's tiles follow the A operand's, and the norms are in the tiles)
-  const unsigned char* tilesB = FOLD ? tiles + nt * (long long)kTcTileBytes : tiles;
-  auto stage = [&](const unsigned char* src, unsigned char* side, float* nside, long long t,
-                   int buf) {
-    const unsigned char* g = src + t * (long long)kTcTileBytes;
-    unsigned char* dst = side + buf * kTcTileBytes;
-    for (int x = tid; x < kTcTileBytes / 16; x += kTcThreads) cp_async16(dst + 16 * x, g + 16 * x);
-    if (!FOLD) cp_async_small<4>(nside + buf * kTcRows + tid, norms + t * kTcRows + tid);
-  };
-  int abuf = 0, bbuf = 0;
-  if (j0 < j1) {
-    stage(tiles, sa2, na2, bi, 0);
-    stage(tilesB, sb2, nb2, bj, 0);
-  }
-  for (long long job = j0; job < j1 && !timed_out; ++job) {
-    cp_async_wait_all();  // this job's tiles (copied during the previous job) have landed
-    asm volatile("fence.proxy.async.shared::cta;");
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    unsigned char* sa = sa2 + abuf * kTcTileBytes;
-    unsigned char* sb = sb2 + bbuf * kTcTileBytes;
-    const float* na = na2 + abuf * kTcRows;
-    nb = nb2 + bbuf * kTcRows;
-    // the next job's tiles go to the other buffers while this job runs
-    long long ni = bi, nj = bj + 1;
-    if (nj == nt) {
-      ++ni;
-      nj = ni;
+  const int count = (int)(j1 - j0);  // (at most 2^30)
+  const int ntile = (int)nt;
+
+  if (warp == kTcEpiWarps) {
+    // copies.  (unless plain, the B operand's tiles follow the A operand's, and hold the norms)
+    const unsigned char* tilesB = FORM != kTcPlain ? tiles + nt * (long long)kTcTileBytes : tiles;
+    int I = (int)I0, bj = (int)bj0, change = 0, a_copied = 0, p = 0;
+    bool ok = true, fresh = true;
+    for (; p < count; ++p) {
+      if (fresh) {  // the next pair of row tiles (in use until the MMAs of the pair before last end)
+        const int as = change & 1;
+        if (change >= 2) ok = tc_wait(&a_empty[as], (uint32_t)(((change >> 1) - 1) & 1), wait_limit, &s_late);
+        ok = __all_sync(full, ok);
+        if (!ok) break;
+        const bool two = 2 * I + 1 < ntile;  // (else the second tile's rows lie beyond n: ignored)
+        if (tc_elect()) {
+          tc_expect(&a_full[as], two ? 2 * kTcTileBytes : kTcTileBytes);
+          const unsigned char* src = tiles + 2LL * I * kTcTileBytes;
+          tc_bulk_copy(s_a + as * 2 * kTcTileBytes, src, kTcTileBytes, &a_full[as]);
+          if (two)
+            tc_bulk_copy(s_a + (as * 2 + 1) * kTcTileBytes, src + kTcTileBytes, kTcTileBytes,
+                         &a_full[as]);
+        }
+        ++change;
+        a_copied = change;
+        fresh = false;
+      }
+      const int slot = p % kTcSlots;
+      if (p >= kTcSlots)
+        ok = tc_wait(&b_empty[slot], (uint32_t)((p / kTcSlots - 1) & 1), wait_limit, &s_late);
+      ok = __all_sync(full, ok);
+      if (!ok) break;
+      if (tc_elect()) {
+        tc_expect(&b_full[slot], kTcTileBytes);
+        tc_bulk_copy(s_b + slot * kTcTileBytes, tilesB + (long long)bj * kTcTileBytes, kTcTileBytes,
+                     &b_full[slot]);
+      }
+      if (++bj == ntile) {
+        ++I;
+        bj = 2 * I;
+        fresh = true;
+      }
     }
-    const bool more = job + 1 < j1;
-    const bool new_a = ni != bi;
-    if (more) {
-      if (new_a) stage(tiles, sa2, na2, ni, abuf ^ 1);
-      stage(tilesB, sb2, nb2, nj, bbuf ^ 1);
-    }
-    if (tid == 0) {
-      // hi.hi + hi.lo + lo.hi: A parts (0, 0, 1), B parts (0, 1, 0); 256 bytes per part
-      const uint32_t a0 = smem_u32(sa), b0 = smem_u32(sb);
-      const uint32_t asel[3] = {0u, 0u, 256u}, bsel[3] = {0u, 256u, 0u};
+    // no copy is left in flight when the block ends (bounded waits, each on a copy's newest phase)
+    int never = 0;
+    for (int z = max(0, p - kTcSlots); z < p; ++z)
+      tc_wait(&b_full[z % kTcSlots], (uint32_t)((z / kTcSlots) & 1), wait_limit, &never);
+    for (int z = max(0, a_copied - 2); z < a_copied; ++z)
+      tc_wait(&a_full[z & 1], (uint32_t)((z >> 1) & 1), wait_limit, &never);
+    __syncwarp();
+  } else if (warp == kTcEpiWarps + 1) {
+    // MMAs
+    const uint32_t idesc = (1u << 4) | ((BF16 ? 1u : 0u) << 7) | ((BF16 ? 1u : 0u) << 10) |
+                           ((128u >> 3) << 17) | ((128u >> 4) << 24);
+    const bool one_part = FORM == kTcPacked && 3 * inst[0].d + 4 <= 16;
+    const uint64_t adesc = make_desc(smem_u32(s_a)), bdesc = make_desc(smem_u32(s_b));
+    int I = (int)I0, bj = (int)bj0, change = 0;
+    bool ok = true, fresh = true;
+    for (int q = 0; q < count; ++q) {
+      const int slot = q % kTcSlots;
+      if (fresh) {
+        ok = tc_wait(&a_full[change & 1], (uint32_t)((change >> 1) & 1), wait_limit, &s_late);
+        ++change;
+        fresh = false;
+      }
+      if (ok) ok = tc_wait(&b_full[slot], (uint32_t)((q / kTcSlots) & 1), wait_limit, &s_late);
+      const uint64_t ad0 = adesc + (uint64_t)(((change - 1) & 1) * 2 * (kTcTileBytes / 16));
+      const uint64_t bd0 = bdesc + (uint64_t)(slot * (kTcTileBytes / 16));
 #pragma unroll
-      for (int s = 0; s < 3; ++s) {
-        const uint64_t ad = make_desc(a0 + asel[s]);
-        const uint64_t bd = make_desc(b0 + bsel[s]);
-        const uint32_t acc = s > 0 ? 1u : 0u;
-        asm volatile(
-            "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-            "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
-      }
-      asm volatile(
-          "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-              smem_u32(&mbar)));
-    }
-    // bounded wait for this job's MMAs (the test hook waits on a barrier nothing arrives on)
-    const bool done = mbar_wait(
-        (inject & kInjectTcWait) ? smem_u32(&mbar_idle) : smem_u32(&mbar), phase, wait_limit);
-    if (!__syncthreads_and(done)) {
-      // give up: wait (bounded again) for the MMAs in flight, so that the tensor memory they
-      // write is not freed under them, then leave
-      mbar_wait(smem_u32(&mbar), phase, wait_limit);
-      if (tid == 0) atomicOr(&st->errors, kErrTimeout);
-      timed_out = true;
-      break;
-    }
-    phase ^= 1u;
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    // epilogue: row `row` of the tile against its 128 columns.  The fast path only builds a
-    // mask of the columns the tile does not reject; those (rare) go to the exact check.
-    const int row = warp * 32 + lane;
-    const long long gi = bi * kTcRows + row;
-    const float nrow = na[row];
-#pragma unroll 1
-    for (int c = 0; c < 128; c += 32) {
-      uint32_t r[32];
-      tc_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c, r);
-      const long long colbase = bj * kTcRows + c;
-      // columns q with gi < colbase + q < n
-      const long long qlo = gi - colbase + 1, qhi = n - colbase;
-      uint32_t valid = 0;
-      if (qlo < 32 && qhi > 0) {
-        const int a0 = qlo > 0 ? (int)qlo : 0, a1 = qhi < 32 ? (int)qhi : 32;
-        if (a1 > a0) valid = (a1 - a0 == 32 ? 0xffffffffu : ((1u << (a1 - a0)) - 1u)) << a0;
-      }
-      float d2v[32];
-      uint32_t hits = 0;
+      for (int mt = 0; mt < 2; ++mt) {
+        const int u = (q & 1) * 2 + mt;
+        if (ok && q >= 2)  // the epilogue has read this accumulator's last job
+          ok = tc_wait(&acc_empty[u], (uint32_t)(((q >> 1) - 1) & 1), wait_limit, &s_late);
+        ok = __all_sync(full, ok);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        if (tc_elect()) {
+          // plain and folded: hi.hi + hi.lo + lo.hi, A parts (0, 0, 1), B parts (0, 1, 0);
+          // packed: parts (0, 0), (1, 1); 256 bytes per part
+          const uint32_t d = tmem + (uint32_t)(u * 128);
+          const uint64_t am = ad0 + (uint64_t)(mt * (kTcTileBytes / 16));
 #pragma unroll
-      for (int q = 0; q < 32; ++q) {
-        d2v[q] = FOLD ? __uint_as_float(r[q])
-                      : (nrow + nb[c + q]) - 2.0f * __uint_as_float(r[q]);
-        hits |= (d2v[q] > hi_thr ? 0u : 1u) << q;  // NaN (overflowed tiles) goes to FP64
+          for (int part = 0; part < (FORM == kTcPacked ? 2 : 3); ++part) {
+            if (part == 1 && one_part) break;
+            const uint64_t ad = am + (FORM == kTcPacked ? part * 16u : (part == 2 ? 16u : 0u));
+            const uint64_t bd = bd0 + (part == 1 ? 16u : 0u);
+            asm volatile(
+                "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+                "l"(ad), "l"(bd), "r"(idesc), "r"(part > 0 ? 1u : 0u));
+          }
+          tc_commit(&acc_full[u]);
+        }
+        __syncwarp();
       }
-      hits &= valid;
-      // queue this chunk's candidates (the warp's shared-memory queue, kept across jobs) and
-      // decide them 32 at a time, one per lane, so that the FP64 checks and their global
-      // loads run in parallel instead of one lane at a time
-      const unsigned int nh = (unsigned int)__popc(hits);
-      unsigned int incl = nh;
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
+      if (!ok) break;
+      const bool last_of_I = bj + 1 == ntile;
+      if (tc_elect()) {
+        tc_commit(&b_empty[slot]);
+        if (last_of_I) tc_commit(&a_empty[(change - 1) & 1]);
       }
-      const unsigned int total = __shfl_sync(0xffffffffu, incl, 31);
-      if (total > (unsigned int)kTcQueue) {
+      __syncwarp();
+      if (++bj == ntile) {
+        ++I;
+        bj = 2 * I;
+        fresh = true;
+      }
+    }
+    // nor an MMA
+    int never = 0;
+    if (tc_elect()) tc_commit(&all_done);
+    __syncwarp();
+    tc_wait(&all_done, 0u, wait_limit, &never);
+    __syncwarp();
+  } else {
+    const Inst In = inst[0];
+    const InstPlan IP = iplan[0];
+    const float lo_thr = tp->lo, hi_thr = tp->hi;
+    const long long n = In.n;
+    const int quad = warp & 3, mt = warp >> 2;
+    unsigned int* q_i = reinterpret_cast<unsigned int*>(smem + (4 + kTcSlots) * kTcTileBytes) +
+                        (size_t)warp * 3 * kTcQueue;  // rows, columns, tile d^2
+    unsigned int* q_j = q_i + kTcQueue;
+    float* q_d = reinterpret_cast<float*>(q_j + kTcQueue);
+    unsigned int qn = 0;  // entries queued (warp-uniform)
+    unsigned int tl_pairs = 0, tl_rechecks = 0, tl_near = 0;
+    bool overflow = false;
+    float max_err = 0.0f;
+    int I = (int)I0, bj = (int)bj0;
+    for (int q = 0; q < count; ++q) {
+      const int u = (q & 1) * 2 + mt;
+      const bool ok = tc_wait((inject & kInjectTcWait) ? &b_idle : &acc_full[u],
+                              (uint32_t)((q >> 1) & 1), wait_limit, &s_late);
+      if (!__all_sync(full, ok)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      const long long gi = (2LL * I + mt) * kTcRows + quad * 32 + lane;
+      // a job on the diagonal, or with columns past the points
+      const bool edge = bj < 2 * I + 2 || bj == ntile - 1;
+      float d2[4][32], least[4];
+      const uint32_t acc = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(u * 128);
 #pragma unroll
-        for (int q = 0; q < 32; ++q)
-          if (hits & (1u << q))
-            tc_candidate(d2v[q], gi, colbase + q, I, IP, dtype, lo_thr, sk, EMIT, tl_pairs,
-                         tl_rechecks, tl_near, max_err, overflow);
-      } else if (total) {
-        if (qn + total > (unsigned int)kTcQueue) {  // room for the chunk: decide the queue first
-          tc_drain(q_i, q_j, q_d, qn, lane, I, IP, dtype, lo_thr, sk, EMIT, tl_pairs,
+      for (int h = 0; h < 4; ++h) {
+        uint32_t r[32];
+        tc_ld32(acc + (uint32_t)(h * 32), r);
+        if (FORM == kTcPlain) {
+          const float nrow = gi < nt * kTcRows ? __ldg(norms + gi) : 0.0f;
+          const float4* nb = reinterpret_cast<const float4*>(norms + (long long)bj * kTcRows + h * 32);
+#pragma unroll
+          for (int v = 0; v < 8; ++v) {
+            const float4 c4 = __ldg(nb + v);
+            d2[h][4 * v] = (nrow + c4.x) - 2.0f * __uint_as_float(r[4 * v]);
+            d2[h][4 * v + 1] = (nrow + c4.y) - 2.0f * __uint_as_float(r[4 * v + 1]);
+            d2[h][4 * v + 2] = (nrow + c4.z) - 2.0f * __uint_as_float(r[4 * v + 2]);
+            d2[h][4 * v + 3] = (nrow + c4.w) - 2.0f * __uint_as_float(r[4 * v + 3]);
+          }
+        } else {
+#pragma unroll
+          for (int v = 0; v < 32; ++v) d2[h][v] = __uint_as_float(r[v]);
+        }
+        float m0 = d2[h][0], m1 = d2[h][1];
+#pragma unroll
+        for (int v = 2; v + 3 < 32; v += 4) {
+          m0 = min3_nan(m0, d2[h][v], d2[h][v + 1]);
+          m1 = min3_nan(m1, d2[h][v + 2], d2[h][v + 3]);
+        }
+        m0 = min3_nan(m0, d2[h][30], d2[h][31]);
+        least[h] = min3_nan(m0, m1, m1);
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;");
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[u]))
+                     : "memory");
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        if (!__any_sync(full, !(least[h] > hi_thr))) continue;  // (NaN goes on)
+        const long long colbase = (long long)bj * kTcRows + h * 32;
+        uint32_t hits = 0;
+#pragma unroll
+        for (int v = 0; v < 32; ++v)
+          hits |= (d2[h][v] > hi_thr ? 0u : 1u) << v;  // NaN (overflowed tiles) goes to FP64
+        if (edge) {  // columns v with gi < colbase + v < n
+          const long long vlo = gi - colbase + 1, vhi = n - colbase;
+          uint32_t valid = 0;
+          if (vlo < 32 && vhi > 0) {
+            const int a0 = vlo > 0 ? (int)vlo : 0, a1 = vhi < 32 ? (int)vhi : 32;
+            if (a1 > a0) valid = (a1 - a0 == 32 ? full : ((1u << (a1 - a0)) - 1u)) << a0;
+          }
+          hits &= valid;
+        }
+        // queue this chunk's candidates (the warp's shared-memory queue, kept across jobs); they
+        // are decided 32 at a time, one per lane, so that the FP64 checks and their global loads
+        // run in parallel
+        const unsigned int nh = (unsigned int)__popc(hits);
+        const unsigned int who = __ballot_sync(full, nh != 0);
+        if (!who) continue;
+        if (qn + 32u > (unsigned int)kTcQueue) {  // room for one per lane
+          tc_drain(q_i, q_j, q_d, qn, lane, In, IP, dtype, lo_thr, sk, EMIT, tl_pairs,
                    tl_rechecks, tl_near, max_err, overflow);
           qn = 0;
         }
-        unsigned int pos = qn + incl - nh;
-        if (hits) {
-#pragma unroll
-          for (int q = 0; q < 32; ++q)
-            if (hits & (1u << q)) {
-              q_i[pos] = (unsigned int)gi;
-              q_j[pos] = (unsigned int)(colbase + q);
-              q_d[pos] = d2v[q];
-              ++pos;
-            }
+        if (!edge && !__any_sync(full, nh > 1u)) {
+          // (nearly always) at most one a lane, which is the lane's smallest value
+          if (nh) {
+            const unsigned int pos = qn + (unsigned int)__popc(who & ((1u << lane) - 1u));
+            q_i[pos] = (unsigned int)gi;
+            q_j[pos] = (unsigned int)(colbase + __ffs(hits) - 1);
+            q_d[pos] = least[h];
+          }
+          qn += (unsigned int)__popc(who);
+          continue;
         }
-        qn += total;
-        __syncwarp();
-        while (qn >= 32) {  // the newest 32 entries, one per lane
-          const unsigned int e = qn - 32 + lane;
-          tc_candidate(q_d[e], (long long)q_i[e], (long long)q_j[e], I, IP, dtype, lo_thr, sk,
-                       EMIT, tl_pairs, tl_rechecks, tl_near, max_err, overflow);
-          qn -= 32;
-          __syncwarp();
+        unsigned int incl = nh;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const unsigned int y = __shfl_up_sync(full, incl, o);
+          if (lane >= o) incl += y;
+        }
+        const unsigned int total = __shfl_sync(full, incl, 31);
+        if (total > (unsigned int)kTcQueue) {
+#pragma unroll
+          for (int v = 0; v < 32; ++v)
+            if (hits & (1u << v))
+              tc_candidate(d2[h][v], gi, colbase + v, In, IP, dtype, lo_thr, sk, EMIT, tl_pairs,
+                           tl_rechecks, tl_near, max_err, overflow);
+        } else if (total) {
+          if (qn + total > (unsigned int)kTcQueue) {  // room for the chunk: the queue first
+            tc_drain(q_i, q_j, q_d, qn, lane, In, IP, dtype, lo_thr, sk, EMIT, tl_pairs,
+                     tl_rechecks, tl_near, max_err, overflow);
+            qn = 0;
+          }
+          unsigned int pos = qn + incl - nh;
+          if (hits) {
+#pragma unroll
+            for (int v = 0; v < 32; ++v)
+              if (hits & (1u << v)) {
+                q_i[pos] = (unsigned int)gi;
+                q_j[pos] = (unsigned int)(colbase + v);
+                q_d[pos] = d2[h][v];
+                ++pos;
+              }
+          }
+          qn += total;
         }
       }
-            }
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    // (the barrier at the top of the next job separates this epilogue from its MMAs)
-    bi = ni;
-    bj = nj;
-    if (new_a) abuf ^= 1;
-    bbuf ^= 1;
+      if (++bj == ntile) {
+        ++I;
+        bj = 2 * I;
+      }
+    }
+    if (qn)  // the candidates still queued
+      tc_drain(q_i, q_j, q_d, qn, lane, In, IP, dtype, lo_thr, sk, EMIT, tl_pairs, tl_rechecks,
+               tl_near, max_err, overflow);
+    // tallies
+    for (int o = 16; o > 0; o >>= 1) {
+      tl_pairs += __shfl_xor_sync(full, tl_pairs, o);
+      tl_rechecks += __shfl_xor_sync(full, tl_rechecks, o);
+      tl_near += __shfl_xor_sync(full, tl_near, o);
+      max_err = fmaxf(max_err, __shfl_xor_sync(full, max_err, o));
+    }
+    if (lane == 0) {
+      atomicAdd(&s_cnt[0], tl_pairs);
+      atomicAdd(&s_cnt[1], tl_rechecks);
+      atomicAdd(&s_cnt[2], tl_near);
+      atomicMax(&s_err, __float_as_uint(max_err));
+    }
+    if (__any_sync(full, overflow) && lane == 0) atomicOr(&st->errors, kErrPairOverflow);
   }
-  cp_async_wait_all();  // no copy of this block is left in flight
-  if (qn)  // the candidates still queued
-    tc_drain(q_i, q_j, q_d, qn, lane, I, IP, dtype, lo_thr, sk, EMIT, tl_pairs, tl_rechecks,
-             tl_near, max_err, overflow);
-  // tallies
-  for (int o = 16; o > 0; o >>= 1) {
-    tl_pairs += __shfl_xor_sync(0xffffffffu, tl_pairs, o);
-    tl_rechecks += __shfl_xor_sync(0xffffffffu, tl_rechecks, o);
-    tl_near += __shfl_xor_sync(0xffffffffu, tl_near, o);
-    max_err = fmaxf(max_err, __shfl_xor_sync(0xffffffffu, max_err, o));
-  }
-  if (lane == 0) {
-    atomicAdd(&s_cnt[0], tl_pairs);
-    atomicAdd(&s_cnt[1], tl_rechecks);
-    atomicAdd(&s_cnt[2], tl_near);
-    atomicMax(&s_err, __float_as_uint(max_err));
-  }
-  if (__syncthreads_or(overflow) && tid == 0) atomicOr(&st->errors, kErrPairOverflow);
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
   if (tid == 0) {
+    if (s_late) atomicOr(&st->errors, kErrTimeout);
     if (s_cnt[0]) atomicAdd(&st->pairs, (unsigned long long)s_cnt[0]);
     if (s_cnt[1]) atomicAdd(&st->dist_rechecks, (unsigned long long)s_cnt[1]);
     if (s_cnt[2]) atomicAdd(&st->near_r, (unsigned long long)s_cnt[2]);
     atomicMax(&st->tc_max_err_bits, s_err);
   }
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(tmem));
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
 }  // namespace
@@ -442,25 +668,24 @@ int launch_brute_tc(const BuildArgs& a, bool bf16, Mode mode, unsigned char* til
   const long long n = a.n_total;
   const long long nt = (n + kTcRows - 1) / kTcRows;
   const long long n_pad = nt * kTcRows;
-  // the norms ride in the MMA when 4 slots of the K = 16 hi block are free (d <= 12)
-  const bool fold = a.dpad <= 16 && a.d_common >= 1 && a.d_common <= 12;
-  k_tc_plan<<<1, 1, 0, s>>>(a.inst, a.bbox, a.iplan, tp, a.st, bf16 ? 1 : 0, fold ? 1 : 0);
+  const TcForm form = tc_form(a.d_max);  // (one instance: its d)
+  k_tc_plan<<<1, 1, 0, s>>>(a.inst, a.bbox, a.iplan, tp, a.st, bf16 ? 1 : 0,
+                              form != kTcPlain ? 1 : 0);
   const unsigned pblocks = (unsigned)((n_pad + 255) / 256);
-  if (bf16 && fold)
-    k_tc_prep<true, true><<<pblocks, 256, 0, s>>>(a.inst, a.dtype, tp, tiles, norms, n_pad);
-  else if (bf16)
-    k_tc_prep<true, false><<<pblocks, 256, 0, s>>>(a.inst, a.dtype, tp, tiles, norms, n_pad);
-  else if (fold)
-    k_tc_prep<false, true><<<pblocks, 256, 0, s>>>(a.inst, a.dtype, tp, tiles, norms, n_pad);
-  else
-    k_tc_prep<false, false><<<pblocks, 256, 0, s>>>(a.inst, a.dtype, tp, tiles, norms, n_pad);
+  auto prep = bf16 ? (form == kTcPacked ? k_tc_prep<true, kTcPacked>
+                                        : (form == kTcFold ? k_tc_prep<true, kTcFold>
+                                                           : k_tc_prep<true, kTcPlain>))
+                   : (form == kTcPacked ? k_tc_prep<false, kTcPacked>
+                                        : (form == kTcFold ? k_tc_prep<false, kTcFold>
+                                                           : k_tc_prep<false, kTcPlain>));
+  prep<<<pblocks, 256, 0, s>>>(a.inst, a.dtype, tp, tiles, norms, n_pad);
   TcSink sk{a.row_cnt, a.pair_buf, a.pair_cap, &a.st->emitted, a.symmetric};
-  // 4 CTAs per SM at most: 128 TMEM columns each fill the 512 columns of an SM.  The dynamic
-  // shared memory (two tiles, norms, the warps' candidate queues, padding to 50 KB) enforces
-  // that occupancy.
-  const size_t smem = 50 * 1024;
-  const long long jobs = nt * (nt + 1) / 2;
-  const unsigned grid = (unsigned)(jobs < 4LL * a.num_sms ? jobs : 4LL * a.num_sms);
+  // one CTA per SM (it takes all 512 TMEM columns): more than half of the shared memory
+  const size_t smem = kTcSmem > 120 * 1024 ? kTcSmem : 120 * 1024;
+  const long long jobs = tc_jobs(nt);
+  // (more CTAs than that only where a CTA's jobs would not be counted in 31 bits)
+  const unsigned grid = (unsigned)std::max<long long>(std::min<long long>(jobs, a.num_sms),
+                                                      (jobs + (1LL << 30) - 1) >> 30);
   const bool emit = mode == kEmit;
 #define RTG_TC_LAUNCH1(B, E, F)                                                                \
   do {                                                                                         \
@@ -480,8 +705,9 @@ int launch_brute_tc(const BuildArgs& a, bool bf16, Mode mode, unsigned char* til
   } while (0)
 #define RTG_TC_LAUNCH(B, E)             \
   do {                                   \
-    if (fold) RTG_TC_LAUNCH1(B, E, true); \
-    else RTG_TC_LAUNCH1(B, E, false);     \
+    if (form == kTcPacked) RTG_TC_LAUNCH1(B, E, kTcPacked); \
+    else if (form == kTcFold) RTG_TC_LAUNCH1(B, E, kTcFold); \
+    else RTG_TC_LAUNCH1(B, E, kTcPlain);     \
   } while (0)
   if (grid > 0) {
     if (bf16 && emit) RTG_TC_LAUNCH(true, true);
