@@ -4,7 +4,7 @@
 // A build is one fixed sequence of kernels on the context's stream with a single host
 // synchronisation at the end.  Three launch decisions depend on the data: the key width
 // (32 or 64 bits), the number of radix passes and the size of the pair buffer.  They are
-// taken from the last build of the same shape; the device checks them (kErrKeyBits,
+// taken from the last builds of the same shape (ShapeGuess); the device checks them (kErrKeyBits,
 // kErrPairOverflow) and on a miss the build is run again with the values the device
 // reported.  The first build of a shape reads the key width back once before sorting.
 #include <cuda_runtime.h>
@@ -562,8 +562,15 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
     }
     bool two_pass = two_pass_flag || q.count_only || bitset;
     if (!two_pass) {
-      const size_t need = (size_t)g.pair_cap * 8;
-      if (c->budget && total_held(c) - c->pair_buf.cap + need + need / (sym ? 1 : 2) > c->budget) {
+      auto too_big = [&]() {
+        const size_t need = (size_t)g.pair_cap * 8;
+        return c->budget &&
+               total_held(c) - c->pair_buf.cap + need + need / (sym ? 1 : 2) > c->budget;
+      };
+      // room kept for a larger earlier input goes before the pair buffer does
+      if (too_big() && g.last_pairs >= 0)
+        g.pair_cap = std::min(g.pair_cap, ShapeGuess::tight_pairs(g.last_pairs));
+      if (too_big()) {
         two_pass = true;
         // the count-then-write form needs no pair buffer: a large one from an earlier build
         // would only crowd the columns out of the budget
@@ -630,10 +637,7 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
     if (!two_pass) {
       // kernels the last build of this shape gave nothing to do are left out; the kernels
       // before them flag any work that turns up, and the build runs again with them
-      if (m > 0 && known)
-        a.skip_tail =
-            (g.no_dense ? rtg::kSkipDense : 0) | (g.no_long_rows ? rtg::kSkipLongRows : 0) |
-            (g.no_rows_left ? rtg::kSkipRowsLeft : 0) | (g.no_bitmap ? rtg::kSkipBitmap : 0);
+      if (m > 0 && known) a.skip_tail = g.skip;
       if ((s = ensure(c, c->pair_buf, (size_t)g.pair_cap * 8)) != RTG_OK) return s;
       a.pair_buf = (unsigned long long*)c->pair_buf.p;
       a.pair_cap = g.pair_cap;
@@ -853,17 +857,9 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
     if (h.errors & retry) {
       // the launch assumptions were too small: take the device's values and run again
       release_out(c, out);
-      if (h.errors & rtg::kErrTailSkipped) {
-        g.no_dense = false;
-        g.no_long_rows = false;
-        g.no_rows_left = false;
-        g.no_bitmap = false;
-      }
-      if (h.errors & rtg::kErrKeyBits) {
-        g.key64 = h.sort_bits > 32;
-        g.key_bits = (int)h.sort_bits;
-        g.cell_bits = (int)h.cell_bits;
-      }
+      if (h.errors & rtg::kErrTailSkipped)
+        for (int w = 0; w < 4; ++w) g.settle_skip(w, false);
+      if (h.errors & rtg::kErrKeyBits) g.settle_bits((int)h.sort_bits, (int)h.cell_bits, false);
       if (h.errors & rtg::kErrPairOverflow)
         g.pair_cap = (long long)((double)h.emitted * 1.05) + 4096;
       continue;
@@ -873,19 +869,14 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
       return s;
     }
     // remember the launch decisions for the next build of this shape
-    if (m > 0) {
-      g.key64 = h.sort_bits > 32;
-      g.key_bits = (int)h.sort_bits;
-      g.cell_bits = (int)h.cell_bits;
-    }
-    if (!two_pass)
-      g.pair_cap = std::max<long long>((long long)((double)h.emitted * 1.05) + 4096, 4096);
+    if (m > 0) g.settle_bits((int)h.sort_bits, (int)h.cell_bits, !known);
+    if (!two_pass) g.settle_pairs((long long)h.emitted);
     if (m > 0 && !bitset) {
       // with a margin, so that new data of the same shape seldom brings such work back
-      g.no_dense = h.max_cell <= (unsigned long long)rtg::kSkipMargin;
-      g.no_long_rows = h.rows_over_margin == 0;
-      g.no_rows_left = h.rows_left == 0;
-      g.no_bitmap = h.long_rows == 0;
+      g.settle_skip(0, h.max_cell <= (unsigned long long)rtg::kSkipMargin);  // kSkipDense
+      g.settle_skip(1, h.rows_over_margin == 0);                             // kSkipLongRows
+      g.settle_skip(2, h.rows_left == 0);                                    // kSkipRowsLeft
+      g.settle_skip(3, h.long_rows == 0);                                    // kSkipBitmap
     }
     if (m > 0 && n_total > 0 && !q.count_only) {
       c->ppp_hint.put(maxd, (double)h.pairs / (double)n_total);

@@ -43,10 +43,57 @@ struct ShapeGuess {
   float cand_per_pos = -1.0f;  // in-cell candidates per sorted position at the last build
   bool pairs_tuned = false;    // enumeration knobs measured for this shape
   int spans_per_warp = 0;      // (tuned) spans per resident warp
-  bool no_dense = false;       // the last build had no cell of more than 32 points
-  bool no_long_rows = false;   // the last build had no row of more than 32 entries
-  bool no_bitmap = false;      // the last build had no row of more than 256 entries
-  bool no_rows_left = false;   // the last build left no row to the block row sort
+  // Kernels left out of the shape's builds (rtg::kSkip* bits), with for each the builds in a row
+  // that had nothing for it.  A decision that follows every build changes the launch sequence
+  // with every other input near a margin, and each change captures the graph again (60 to 110
+  // us): so a kernel that had work comes back at once and goes only after kCalmBuilds.
+  int skip = 0;
+  int calm[4] = {kCalmBuilds, kCalmBuilds, kCalmBuilds, kCalmBuilds};
+  // Builds in a row whose keys needed fewer bits than key_bits / cell_bits hold, and the widest
+  // of them (too few bits cost a second build, one pass too many a few per cent).
+  int narrow = 0, narrow_key = 0, narrow_cell = 0;
+  static constexpr int kCalmBuilds = 16;
+
+  // After a build: bit `which` (0..3) stands for a kernel that found no work (idle) or some.
+  void settle_skip(int which, bool idle) {
+    int& n = calm[which];
+    if (!idle) {
+      n = 0;
+      skip &= ~(1 << which);
+    } else if (n >= kCalmBuilds || ++n >= kCalmBuilds) {
+      skip |= 1 << which;
+    }
+  }
+  // After a build whose keys took kb bits (the widest cell index cb).
+  void settle_bits(int kb, int cb, bool first) {
+    if (first || kb > key_bits || cb > cell_bits) {
+      key_bits = first ? kb : std::max(kb, key_bits);
+      cell_bits = first ? cb : std::max(cb, cell_bits);
+      narrow = narrow_key = narrow_cell = 0;
+    } else if (kb == key_bits && cb == cell_bits) {
+      narrow = narrow_key = narrow_cell = 0;
+    } else {
+      narrow_key = std::max(narrow_key, kb);
+      narrow_cell = std::max(narrow_cell, cb);
+      if (++narrow >= kCalmBuilds) {
+        key_bits = narrow_key;
+        cell_bits = narrow_cell;
+        narrow = narrow_key = narrow_cell = 0;
+      }
+    }
+    key64 = key_bits > 32;
+  }
+  // Pair-buffer entries after a build that emitted e pairs: kept while they hold 6% more than e
+  // and no more than four times that, so that inputs of one shape whose pair counts differ
+  // neither overflow the buffer (a second enumeration: twice the time on clustered points) nor
+  // change the launch sequence.
+  static long long tight_pairs(long long e) { return e + e / 16 + 4096; }
+  void settle_pairs(long long e) {
+    last_pairs = e;
+    if (pair_cap < tight_pairs(e) || pair_cap > 4 * tight_pairs(e))
+      pair_cap = (e + e / 4 + 4096 + 4095) / 4096 * 4096;
+  }
+  long long last_pairs = -1;  // pairs of the shape's last build (-1: none)
 };
 
 // A build's launch sequence captured once and replayed for later builds of the same shape.

@@ -115,3 +115,22 @@ def test_overflow_after_a_replay_with_an_even_pass_count():
         ref = oracle.rtg(pts, r, T, r).csr
         assert np.array_equal(rp, ref.row_ptr) and np.array_equal(col, ref.col), k
     ctx.close()
+
+
+def test_inputs_that_alternate_settle():
+    # two inputs of one shape whose pair counts, cells and rows differ: once both were built, no
+    # build runs twice, and each still equals the oracle's
+    d, n, m, r = 3, 4000, 6, 0.06
+    a = gen.points_uniform(31, n, d)  # light cells and short rows
+    b = gen.points_mixture(31, n, d, k=8, sigma=0.05, dtype=np.float64)
+    T = gen.transforms(31, d, m, r)
+    refs = [oracle.rtg(p, r, T, r).csr for p in (a, b)]
+    ctx = rtg.Context(0)
+    for k in range(10):
+        which = k % 2
+        res = ctx.all_pairs((a, b)[which], r, T, r)
+        st, (rp, col) = res.stats, res.download()
+        res.release()
+        assert np.array_equal(rp, refs[which].row_ptr) and np.array_equal(col, refs[which].col), k
+        assert k < 4 or st["attempts"] == 1, (k, st["attempts"])
+    ctx.close()
