@@ -84,13 +84,13 @@ struct ShapeGuess {
     key64 = key_bits > 32;
   }
   // Pair-buffer entries after a build that emitted e pairs: kept while they hold 6% more than e
-  // and no more than four times that, so that inputs of one shape whose pair counts differ
+  // and no more than four times that (and 2^20, 8 MB), so that inputs of one shape whose pair counts differ
   // neither overflow the buffer (a second enumeration: twice the time on clustered points) nor
   // change the launch sequence.
   static long long tight_pairs(long long e) { return e + e / 16 + 4096; }
   void settle_pairs(long long e) {
     last_pairs = e;
-    if (pair_cap < tight_pairs(e) || pair_cap > 4 * tight_pairs(e))
+    if (pair_cap < tight_pairs(e) || pair_cap > 4 * tight_pairs(e) + (1 << 20))
       pair_cap = (e + e / 4 + 4096 + 4095) / 4096 * 4096;
   }
   long long last_pairs = -1;  // pairs of the shape's last build (-1: none)
