@@ -621,7 +621,8 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
     };
     auto pairs = [&](rtg::Mode mode) {
       if (m > 0) return rtg::launch_pairs(a, sorted, mode, st);
-      if (tc)
+      // (the tensor-core kernel counts and emits; columns are written by the other one)
+      if (tc && mode != rtg::kWrite)
         return rtg::launch_brute_tc(a, (q.flags & RTG_FLAG_TC_BF16) != 0, mode,
                                     (unsigned char*)c->tc_tiles.p, (float*)c->tc_norms.p,
                                     (rtg::TcPlan*)c->tc_plan.p, st);

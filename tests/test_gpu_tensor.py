@@ -64,3 +64,22 @@ def test_dense_cells_on_tensor_cores_match_oracle(ctx, tensor, sigma, n, d, dtyp
     assert np.array_equal(rp, ref.csr.row_ptr) and np.array_equal(col, ref.csr.col)
     assert st["candidates"] == [s["candidates"] for s in ref.stats]
     assert st["large_cells"] > 0 and st["max_cell"] > 256
+
+
+@pytest.mark.parametrize("two_pass_by_overflow", [True, False])
+def test_tc_brute_writes_columns_of_dense_graphs(ctx, two_pass_by_overflow):
+    # more pairs than a first build's buffer holds (16 a point): the columns come from a second
+    # enumeration; the shape's next build holds them all
+    n, d = (1500, 3) if two_pass_by_overflow else (400, 2)
+    pts = gen.points_uniform(77, n, d, np.float32)
+    r = gen.radius_for_degree(n, d, 150.0)
+    ex = oracle.brute(pts, r)
+    assert ex.nnz > 16 * n
+    own = rtg.Context(0)
+    for k in range(2):
+        res = own.brute_force(pts, r, tensor="fp16")
+        rp, col = res.download()
+        assert res.stats["attempts"] == (2 if k == 0 else 1)
+        res.release()
+        assert np.array_equal(rp, ex.row_ptr) and np.array_equal(col, ex.col)
+    own.close()
