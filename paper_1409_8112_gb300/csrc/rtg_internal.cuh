@@ -154,6 +154,7 @@ struct TcPlan {
   double center[kMaxDim];
   double band, bound;
   float lo, hi;  // FP32 d^2 below hi goes to the FP64 check; lo bounds the band from below
+  int use;       // the tiles decide (always when asked for; else when the band is narrow)
 };
 
 // One roadmap of a batch (filled on the host).
@@ -284,6 +285,8 @@ struct BuildArgs {
   int passes;          // radix passes launched
   unsigned int* sort_epoch;  // device counter: look-back epoch base, advanced by every sort
   int num_sms;
+  const TcPlan* tc_auto;    // brute force: the CUDA-core kernel leaves the pairs to the tiles when
+                            // this plan (of launch_brute_tc) says so; null: it takes them
   int tc_cells;             // cells of more than 256 points on the tensor cores: 0 off,
                             // 1 FP16 halves, 2 BF16 halves
   unsigned int spin_limit;  // bounded waits: iterations before giving up (0: the default)
@@ -463,9 +466,10 @@ size_t sort_tiles_for(long long N, int items);
 // Whether the single-launch sort can run this variant: every tile's block resident at once.
 bool sort_coop_fits(long long N, int bits, int items, int num_sms, bool key64);
 size_t tc_tiles_bytes(long long n);
-// tensor-core brute force (instance 0 only); returns kernels launched
+// tensor-core brute force (instance 0 only); returns kernels launched.  always: whatever the
+// error bound; else only where the plan finds the band narrow (TcPlan::use).
 int launch_brute_tc(const BuildArgs& a, bool bf16, Mode mode, unsigned char* tiles, float* norms,
-                    TcPlan* tp, cudaStream_t s);
+                    TcPlan* tp, bool always, cudaStream_t s);
 
 // Text returned by rtg_last_error(NULL) on this thread.
 void set_last_error(const char* msg);

@@ -1418,7 +1418,9 @@ template <int DPAD, int MODE>
 __global__ void __launch_bounds__(kPairThreads) k_brute(const float* __restrict__ pf, int dtype,
                                                         const Inst* __restrict__ inst,
                                                         const InstPlan* __restrict__ iplan,
-                                                        Status* st, Sink sk) {
+                                                        Status* st, Sink sk,
+                                                        const TcPlan* tc_auto) {
+  if (tc_auto && tc_auto->use) return;  // the tensor-core tiles have taken the pairs
   __shared__ __align__(16) float sa[kBT * DPAD];
   __shared__ __align__(16) float sb[kBT * DPAD];
   __shared__ unsigned int s_tally[4];
@@ -2067,7 +2069,7 @@ template <int DPAD, int MODE>
 void brute_impl(const BuildArgs& a, cudaStream_t s) {
   const unsigned blocks = (unsigned)(8 * a.num_sms);
   k_brute<DPAD, MODE><<<blocks, kPairThreads, 0, s>>>(a.pf, a.dtype, a.inst, a.iplan, a.st,
-                                                      make_sink(a));
+                                                      make_sink(a), a.tc_auto);
 }
 
 // The dense-cell jobs on the tensor cores (FP16 or BF16 halves), 4 blocks of 128 threads per

@@ -50,7 +50,7 @@ __device__ __forceinline__ double load_coord(const void* pts, int dtype, long lo
 // Band, thresholds and centre for instance 0 (one thread).
 __global__ void k_tc_plan(const Inst* __restrict__ inst, const unsigned long long* bbox,
                           const InstPlan* __restrict__ iplan, TcPlan* tp, Status* st, int bf16,
-                          int fold) {
+                          int fold, int always) {
   const Inst I = inst[0];
   const int d = I.d;
   double M = 0.0;
@@ -72,7 +72,12 @@ __global__ void k_tc_plan(const Inst* __restrict__ inst, const unsigned long lon
   const double band = fmax(1e-3 * rr, 1.25 * E);
   tp->band = band;
   tp->bound = E;
-  st->tc_band = band;
+  // Unasked, the tiles are taken when the FP64 band they need stays below an eighth of r^2 (so
+  // few pairs fall inside it) and nothing overflows a half (coordinates doubled, norms).
+  const double most = bf16 ? 1e30 : 60000.0;
+  const bool use = always || (band <= 0.125 * rr && 2.0 * M < most && (double)d * M * M < most);
+  tp->use = use ? 1 : 0;
+  if (use) st->tc_band = band;
   tp->lo = __double2float_rd(rr - band);
   tp->hi = __double2float_ru(rr + band);
 }
@@ -103,7 +108,7 @@ __global__ void __launch_bounds__(256) k_tc_prep(const Inst* __restrict__ inst, 
   };
   const Inst I = inst[0];
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= n_pad) return;
+  if (i >= n_pad || !tp->use) return;
   const long long ntile = n_pad / kTcRows;
   unsigned char* tile = tiles + (i / kTcRows) * (long long)kTcTileBytes;
   unsigned char* tileB = FORM != kTcPlain ? tile + ntile * (long long)kTcTileBytes : tile;
@@ -327,6 +332,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
   __shared__ int s_late;  // some wait ran out
   const unsigned int full = 0xffffffffu;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (!tp->use) return;  // the CUDA-core kernel takes the pairs
   const long long nI = (nt + 1) / 2;
   const long long jobs = tc_jobs(nt);
   const long long per = (jobs + gridDim.x - 1) / gridDim.x;
@@ -664,13 +670,13 @@ size_t tc_tiles_bytes(long long n) {
 }
 
 int launch_brute_tc(const BuildArgs& a, bool bf16, Mode mode, unsigned char* tiles, float* norms,
-                    TcPlan* tp, cudaStream_t s) {
+                    TcPlan* tp, bool always, cudaStream_t s) {
   const long long n = a.n_total;
   const long long nt = (n + kTcRows - 1) / kTcRows;
   const long long n_pad = nt * kTcRows;
   const TcForm form = tc_form(a.d_max);  // (one instance: its d)
   k_tc_plan<<<1, 1, 0, s>>>(a.inst, a.bbox, a.iplan, tp, a.st, bf16 ? 1 : 0,
-                              form != kTcPlain ? 1 : 0);
+                              form != kTcPlain ? 1 : 0, always ? 1 : 0);
   const unsigned pblocks = (unsigned)((n_pad + 255) / 256);
   auto prep = bf16 ? (form == kTcPacked ? k_tc_prep<true, kTcPacked>
                                         : (form == kTcFold ? k_tc_prep<true, kTcFold>

@@ -83,3 +83,36 @@ def test_tc_brute_writes_columns_of_dense_graphs(ctx, two_pass_by_overflow):
         res.release()
         assert np.array_equal(rp, ex.row_ptr) and np.array_equal(col, ex.col)
     own.close()
+
+
+@pytest.mark.parametrize("n,d,dtype,scale,shift,degree,tiles", [
+    (4095, 6, np.float64, 1.0, 0.0, 20.0, False),   # below the size rule
+    (4096, 6, np.float64, 1.0, 0.0, 20.0, True),
+    (4223, 1, np.float32, 1.0, 0.0, 9.0, None),
+    (4225, 4, np.float32, 1.0, 0.0, 12.0, True),    # one K = 16 part
+    (4099, 5, np.float64, 1.0, 0.0, 12.0, True),    # two parts
+    (5000, 9, np.float32, 1.0, 0.0, 12.0, True),
+    (4500, 10, np.float64, 1.0, 0.0, 12.0, True),   # norms in the hi block
+    (4300, 13, np.float32, 1.0, 0.0, 12.0, True),   # norms added afterwards
+    (4111, 3, np.float64, 1e-3, 0.0, 12.0, None),
+    (4111, 3, np.float64, 1e-7, 0.0, 12.0, False),  # the halves cannot resolve such points
+    (4111, 6, np.float32, 1e3, 0.0, 12.0, False),   # norms beyond the half range
+    (4111, 6, np.float64, 1.0, 1e4, 12.0, True),    # far from the origin: the tiles are centred
+    (4111, 2, np.float64, 1.0, 0.0, 0.02, False),   # r far below the points' extent
+])
+def test_default_brute_force_by_either_kernel(ctx, n, d, dtype, scale, shift, degree, tiles):
+    # the default brute force takes tensor-core tiles where their error bound is narrow against
+    # r^2; the set is the oracle's whichever kernel decided it
+    pts = (gen.points_uniform(n + d, n, d) * scale + shift).astype(dtype)
+    r = gen.radius_for_degree(n, d, degree) * scale
+    ex = oracle.brute(pts, r)
+    for kw in ({}, {"count_only": True}, {"symmetric": True}):
+        res = ctx.brute_force(pts, r, **kw)
+        st = res.stats
+        assert st["pairs"] == ex.nnz
+        if tiles is not None:
+            assert (st["band"] > 0) == tiles
+        if not kw:
+            rp, col = res.download()
+            assert np.array_equal(rp, ex.row_ptr) and np.array_equal(col, ex.col)
+        res.release()
