@@ -1080,7 +1080,8 @@ void trim_workspace(rtg_ctx* c) {
   if (c->stream) cudaStreamSynchronize(c->stream);
   DevBuf* bufs[] = {&c->pts,      &c->pf,        &c->key_mat, &c->keys0,    &c->keys1,
                     &c->vals0,    &c->vals1,     &c->lookback, &c->row_cnt, &c->scan_lb,
-                    &c->large,    &c->large_job, &c->pair_buf, &c->tc_tiles, &c->tc_norms};
+                    &c->large,    &c->large_job, &c->pair_buf, &c->tc_tiles, &c->tc_norms,
+                    &c->q_slots};
   for (DevBuf* b : bufs) free_buf(c, *b);
   // captured graphs name the freed buffers (a replay needs the same pointers, so none would
   // replay; they go now rather than when their shape comes back)
@@ -1101,6 +1102,7 @@ void destroy_ctx(rtg_ctx* c) {
   while (!c->graphs.empty()) drop_graph(c, c->graphs.begin()->first);
   free_buf(c, c->out_slot);
   free_buf(c, c->q_idx);
+  free_buf(c, c->q_slots);
   free_buf(c, c->bits);
   free_buf(c, c->sort_epoch);
   if (c->h_slot) cudaFreeHost(c->h_slot);

@@ -155,7 +155,7 @@ struct rtg_ctx {
   std::string err;
   rtghost::DevBuf status, inst, iplan, gplan, bases, T64, pts, pf, key_mat, keys0, keys1,
       vals0, vals1, lookback, hist, digit_off, row_cnt, scan_lb, large, large_job, pair_buf,
-      tc_tiles, tc_norms, tc_plan, out_slot, sort_epoch, q_idx, bits;
+      tc_tiles, tc_norms, tc_plan, out_slot, sort_epoch, q_idx, q_slots, bits;
   rtg::Status* h_status = nullptr;  // pinned
   rtg::OutSlot* h_slot = nullptr;   // pinned; copied to out_slot before the output kernels
   bool use_graphs = true;           // RTG_GRAPHS=0 launches every kernel directly

@@ -17,14 +17,17 @@
 //     on the original coordinates (the band likewise only inside the bounding box);
 //   * j is reported by the first grid that puts it in the query's cell (the dedupe of
 //     Sec. III-B by key rows), so every answer appears once.
-// One thread per query for indexes of light cells, one warp per query (32 candidates at a time)
-// for dense ones.  Two passes: count the answers, scan the counts into row pointers, write the
-// answers, then sort each row (the pair path's row sort).
+// Indexes of light cells give each (query, grid) a thread, which collects the answers of a query in
+// 32 slots; after the scan of the counts the rows are sorted on their way to their places.  Only
+// queries with more answers than slots are searched again, one thread per query.  Indexes of
+// dense cells give each query a warp (32 candidates at a time) and search twice: count the
+// answers, scan, write them, then sort each row (the pair path's row sort).
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <string>
 
 #include "rtg_host.h"
@@ -310,7 +313,7 @@ __global__ void __launch_bounds__(kIndexThreads) k_index_query(
 
 // One thread per query, for indexes whose cells hold few points (a warp per query would leave
 // most lanes idle): the thread walks the m grids in order, keeping the query's keys for the
-// first-grid rule, and writes its own row.
+// first-grid rule, and writes its own row.  WRITE: rows of at least min_len answers.
 template <typename K, int DPAD, bool WRITE>
 __global__ void __launch_bounds__(kIndexThreads) k_index_query_thread(
     const Inst* __restrict__ inst, const InstPlan* __restrict__ iplan,
@@ -319,13 +322,14 @@ __global__ void __launch_bounds__(kIndexThreads) k_index_query_thread(
     const unsigned long long* __restrict__ table, long long cap,
     const K* __restrict__ key_mat, int m, const float* __restrict__ pf,
     const void* __restrict__ queries, int dtype, long long nq, QueryBox box,
-    unsigned int* row_cnt, const OutSlot* out, Status* st) {
+    unsigned int* row_cnt, const OutSlot* out, Status* st, int min_len) {
   const Inst I = inst[0];
   const InstPlan IP = iplan[0];
   const int d = I.d, tstride = d * d + d;
   unsigned int rechecks = 0;
   for (long long kq = blockIdx.x * (long long)blockDim.x + threadIdx.x; kq < nq;
        kq += (long long)gridDim.x * blockDim.x) {
+    if (WRITE && out->row_ptr[kq + 1] - out->row_ptr[kq] < min_len) continue;
     float qf[DPAD];
     bool in_box = true, finite = true;
 #pragma unroll
@@ -401,10 +405,184 @@ __global__ void __launch_bounds__(kIndexThreads) k_index_query_thread(
     atomicAdd(&st->dist_rechecks, (unsigned long long)rechecks);
 }
 
+// One thread per (query, grid), for indexes whose cells hold few points: 256 / m queries per block
+// and step, thread slot m + t taking grid t.  The grids' FP32 rotations sit in shared memory,
+// axis by axis with the grids next to each other, and so do the step's query keys (read by the
+// first-grid rule).  A query's answers go to its kRowSlots slots in the order found, counted in
+// row_cnt; st->max_cell receives the largest count.
+// Bound by the latency of its chains (table, run head, members, rows, key rows), which is why
+// the grids of a query are spread over threads: 100,000 queries by one thread each left 21
+// warps per SM and took 187 us to count and as long again to write (query call 424 us, now 218).
+template <typename K, int DPAD>
+__global__ void __launch_bounds__(kIndexThreads) k_index_query_lanes(
+    const Inst* __restrict__ inst, const InstPlan* __restrict__ iplan,
+    const GridPlan* __restrict__ gplan, const double* __restrict__ T64,
+    const K* __restrict__ skeys, const uint32_t* __restrict__ svals,
+    const unsigned long long* __restrict__ table, long long cap,
+    const K* __restrict__ key_mat, int m, const float* __restrict__ pf,
+    const void* __restrict__ queries, int dtype, long long nq, QueryBox box,
+    unsigned int* row_cnt, int* __restrict__ slots, Status* st) {
+  extern __shared__ float s_rot[];  // [axis][l][grid], then the shifts [axis][grid]
+  __shared__ K s_key[kIndexThreads];
+  __shared__ unsigned char s_has[kIndexThreads];
+  __shared__ unsigned int s_found[kIndexThreads];
+  __shared__ unsigned int s_most;
+  const Inst I = inst[0];
+  const InstPlan IP = iplan[0];
+  const int d = I.d;
+  float* s_sh = s_rot + d * d * m;
+  for (int x = threadIdx.x; x < d * d * m; x += blockDim.x) {
+    const int g = x % m, kl = x / m;
+    s_rot[x] = gplan[g].Rf[(kl / d) * kMaxDim + kl % d];
+  }
+  for (int x = threadIdx.x; x < d * m; x += blockDim.x) s_sh[x] = gplan[x % m].sf[x / m];
+  if (threadIdx.x == 0) s_most = 0;
+  s_found[threadIdx.x] = 0;
+  __syncthreads();
+  const int P = kIndexThreads / m;  // queries per step
+  const int t = (int)threadIdx.x % m, slot = (int)threadIdx.x / m;
+  const GridPlan& G = gplan[t];
+  const double* Tt = T64 + I.T0 + (size_t)t * (d * d + d);
+  const unsigned long long* tab = table + (long long)t * cap;
+  const float inv_cf = I.inv_cf;
+  unsigned int rechecks = 0, most = 0;
+  for (long long q0 = (long long)blockIdx.x * P; q0 < nq; q0 += (long long)gridDim.x * P) {
+    const long long kq = q0 + slot;
+    const bool on = slot < P && kq < nq;
+    float qf[DPAD];
+    bool in_box = true, finite = true;
+    if (on) {
+#pragma unroll
+      for (int l = 0; l < DPAD; ++l) {
+        qf[l] = 0.0f;
+        if (l < d) {
+          const double x = coord(queries, dtype, kq, d, l);
+          finite &= isfinite(x);
+          in_box &= x >= box.lo[l] && x <= box.hi[l];
+          qf[l] = dtype == 0 ? __double2float_rn(x) : (float)x;
+          finite &= isfinite(qf[l]);
+        }
+      }
+    }
+    if (on && !finite && t == 0) atomicOr(&st->errors, kErrNonFinite);
+    bool has = on && finite;
+    K key = (K)G.base;
+    if (has) {
+      for (int k = 0; k < d; ++k) {  // as query_key, from shared memory
+        long long cell = 0;
+        bool certain = false;
+        if (in_box) {
+          float y = s_sh[k * m + t];
+#pragma unroll
+          for (int l = 0; l < DPAD; ++l)
+            if (l < d) y = fmaf(s_rot[(k * d + l) * m + t], qf[l], y);
+          const float u = y * inv_cf;
+          const float f = floorf(u), e = G.E[k];
+          certain = __fsub_rd(u, e) >= f && __fadd_ru(u, e) < f + 1.0f;
+          cell = (long long)(int)f;
+        }
+        if (!certain && !exact_axis(queries, dtype, kq, d, Tt, k, I.c, &cell)) {
+          has = false;
+          continue;
+        }
+        const long long off = cell - G.qlo[k];
+        if ((unsigned long long)off >= G.ext[k]) has = false;
+        else key += (K)off * (K)G.stride[k];
+      }
+    }
+    s_key[threadIdx.x] = key;
+    s_has[threadIdx.x] = has ? 1 : 0;
+    __syncthreads();  // the step's keys; s_found is zero
+    if (has) {
+      const float2 band = IP.filter_on && in_box ? make_float2(IP.s_lo, IP.s_hi)
+                                                 : make_float2(-1.0f, __int_as_float(0x7f800000));
+      long long lo, hi;
+      find_run(skeys, tab, cap, key, &lo, &hi);
+      const int first = slot * m;
+      for (long long pos = lo; pos < hi; ++pos) {
+        const unsigned int j = svals[pos];
+        float sf = 0.0f;
+        const float4* pj = reinterpret_cast<const float4*>(pf + (size_t)j * DPAD);
+#pragma unroll
+        for (int v = 0; v < DPAD / 4; ++v) {
+          const float4 y = __ldg(pj + v);
+          float e = qf[4 * v] - y.x;
+          sf = fmaf(e, e, sf);
+          e = qf[4 * v + 1] - y.y;
+          sf = fmaf(e, e, sf);
+          e = qf[4 * v + 2] - y.z;
+          sf = fmaf(e, e, sf);
+          e = qf[4 * v + 3] - y.w;
+          sf = fmaf(e, e, sf);
+        }
+        if (sf > band.y) continue;
+        if (!(sf < band.x)) {
+          double s2 = 0.0;
+          for (int l = 0; l < d; ++l) {
+            const double e = __dsub_rn(coord(queries, dtype, kq, d, l),
+                                       coord(I.pts, dtype, (long long)j, d, l));
+            s2 = __fma_rn(e, e, s2);
+          }
+          ++rechecks;
+          if (!(s2 <= IP.rr)) continue;
+        }
+        // reported by the first grid that puts j in the query's cell
+        const K* kj = key_mat + (size_t)j * m;
+        bool earlier = false;
+        for (int u0 = 0; u0 < t && !earlier; u0 += 4) {
+#pragma unroll
+          for (int z = 0; z < 4; ++z)
+            if (u0 + z < t)
+              earlier |= s_has[first + u0 + z] && __ldg(kj + u0 + z) == s_key[first + u0 + z];
+        }
+        if (earlier) continue;
+        const unsigned int at = atomicAdd(&s_found[slot], 1u);
+        if (at < (unsigned int)kRowSlots) slots[kq * kRowSlots + at] = (int)j;
+      }
+    }
+    __syncthreads();
+    if (on && t == 0) {
+      const unsigned int c = s_found[slot];
+      row_cnt[kq] = c;
+      most = max(most, c);
+      s_found[slot] = 0;
+    }
+    // (the next step's first barrier comes before s_found is used again)
+  }
+  if (most) atomicMax(&s_most, most);
+  for (int o = 16; o > 0; o >>= 1) rechecks += __shfl_xor_sync(0xffffffffu, rechecks, o);
+  if ((threadIdx.x & 31) == 0 && rechecks)
+    atomicAdd(&st->dist_rechecks, (unsigned long long)rechecks);
+  __syncthreads();
+  if (threadIdx.x == 0 && s_most) atomicMax(&st->max_cell, (unsigned long long)s_most);
+}
+
 template <typename K, int DPAD, bool WRITE>
 void query_launch(const rtg_index* ix, const void* q, long long nq, const QueryBox& box,
                   unsigned int* row_cnt, const OutSlot* out, Status* st, int num_sms,
-                  cudaStream_t s) {
+                  int* slots, int min_len, cudaStream_t s) {
+  if (!WRITE && slots) {
+    const int P = kIndexThreads / ix->m;
+    long long blocks = (nq + P - 1) / P;
+    if (blocks > 6LL * num_sms) blocks = 6LL * num_sms;
+    const size_t smem = (size_t)ix->m * ix->d * (ix->d + 1) * sizeof(float);
+    static size_t attr_smem[64] = {};  // largest size granted so far, per device
+    int dev = 0;
+    cudaGetDevice(&dev);
+    {
+      std::lock_guard<std::mutex> lk(launch_attr_mutex());
+      if (dev < 0 || dev >= 64 || smem > attr_smem[dev]) {
+        cudaFuncSetAttribute(k_index_query_lanes<K, DPAD>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (dev >= 0 && dev < 64) attr_smem[dev] = smem;
+      }
+    }
+    k_index_query_lanes<K, DPAD><<<(unsigned)blocks, kIndexThreads, smem, s>>>(
+        ix->inst, ix->iplan, ix->gplan, ix->T64, (const K*)ix->skeys, ix->svals, ix->table,
+        ix->table_cap, (const K*)ix->key_mat, ix->m, ix->pf, q, ix->dtype, nq, box, row_cnt, slots,
+        st);
+    return;
+  }
   if (ix->thread_queries) {
     long long blocks = (nq + kIndexThreads - 1) / kIndexThreads;
     if (blocks > 8LL * num_sms) blocks = 8LL * num_sms;
@@ -412,7 +590,7 @@ void query_launch(const rtg_index* ix, const void* q, long long nq, const QueryB
     k_index_query_thread<K, DPAD, WRITE><<<(unsigned)blocks, kIndexThreads, 0, s>>>(
         ix->inst, ix->iplan, ix->gplan, ix->T64, (const K*)ix->skeys, ix->svals, ix->table,
         ix->table_cap, (const K*)ix->key_mat, ix->m, ix->pf, q, ix->dtype, nq, box, row_cnt,
-        out, st);
+        out, st, min_len);
     return;
   }
   long long blocks = (nq + kIndexThreads / 32 - 1) / (kIndexThreads / 32);
@@ -427,8 +605,9 @@ void query_launch(const rtg_index* ix, const void* q, long long nq, const QueryB
 template <bool WRITE>
 void launch_index_query(const rtg_index* ix, const void* q, long long nq, const QueryBox& box,
                         unsigned int* row_cnt, const OutSlot* out, Status* st, int num_sms,
-                        cudaStream_t s) {
-#define RTG_IQ(K, P) query_launch<K, P, WRITE>(ix, q, nq, box, row_cnt, out, st, num_sms, s)
+                        int* slots, int min_len, cudaStream_t s) {
+#define RTG_IQ(K, P) \
+  query_launch<K, P, WRITE>(ix, q, nq, box, row_cnt, out, st, num_sms, slots, min_len, s)
   if (ix->key64) {
     if (ix->dpad == 4) RTG_IQ(unsigned long long, 4);
     else if (ix->dpad == 8) RTG_IQ(unsigned long long, 8);
@@ -622,6 +801,16 @@ rtg_status index_query(rtg_ctx* c, const rtg_index* ix, const void* queries, int
     release_out(c, out);
     return s;
   }
+  // slots for the answers of light cells' queries (without room for them: two searches)
+  int* slots = nullptr;
+  if (ix->thread_queries) {
+    if (ensure(c, c->q_slots, (size_t)nq * rtg::kRowSlots * sizeof(int)) == RTG_OK) {
+      slots = (int*)c->q_slots.p;
+    } else {
+      c->err.clear();
+      cudaGetLastError();
+    }
+  }
   const void* q = queries;
   if (!on_device) {
     if ((s = cuda_ok(c, cudaMemcpyAsync(c->pts.p, queries, (size_t)nq * ix->d * esz,
@@ -649,7 +838,7 @@ rtg_status index_query(rtg_ctx* c, const rtg_index* ix, const void* queries, int
   c->h_slot->col_cap = 0;
   cudaMemsetAsync(a.st, 0, sizeof(rtg::Status), st);
   cudaMemcpyAsync(c->out_slot.p, c->h_slot, sizeof(rtg::OutSlot), cudaMemcpyHostToDevice, st);
-  rtg::launch_index_query<false>(ix, q, nq, box, a.row_cnt, a.out, a.st, c->num_sms, st);
+  rtg::launch_index_query<false>(ix, q, nq, box, a.row_cnt, a.out, a.st, c->num_sms, slots, 0, st);
   rtg::launch_scan(a, st);
   if ((s = cuda_ok(c, cudaGetLastError(), "index query")) != RTG_OK ||
       (s = read_status(c)) != RTG_OK) {
@@ -675,8 +864,13 @@ rtg_status index_query(rtg_ctx* c, const rtg_index* ix, const void* queries, int
     c->h_slot->col = (int*)cp;
     c->h_slot->col_cap = nnz;
     cudaMemcpyAsync(c->out_slot.p, c->h_slot, sizeof(rtg::OutSlot), cudaMemcpyHostToDevice, st);
-    rtg::launch_index_query<true>(ix, q, nq, box, a.row_cnt, a.out, a.st, c->num_sms, st);
-    rtg::launch_rowsort(a, st, ix->n);  // answers are indexed-point indices
+    const bool all_in_slots = slots && c->h_status->max_cell <= (unsigned long long)rtg::kRowSlots;
+    if (slots) rtg::launch_rows_from_slots(a.out, nq, slots, st);
+    if (!all_in_slots) {
+      rtg::launch_index_query<true>(ix, q, nq, box, a.row_cnt, a.out, a.st, c->num_sms, nullptr,
+                                    slots ? rtg::kRowSlots + 1 : 0, st);
+      rtg::launch_rowsort(a, st, ix->n);  // answers are indexed-point indices
+    }
   }
   if ((s = cuda_ok(c, cudaGetLastError(), "index query")) != RTG_OK ||
       (s = read_status(c)) != RTG_OK || (s = check_errors(c, ~0u)) != RTG_OK) {

@@ -457,6 +457,11 @@ int launch_rowsort(const BuildArgs& a, cudaStream_t s, long long col_bound = -1)
 // cleared so that the enumeration can be run again (the autotuner's trials).
 void reset_pairs_state(const BuildArgs& a, cudaStream_t s);
 
+// Rows collected unordered in slots of kRowSlots entries each (row k at slots + k kRowSlots):
+// every row of at most kRowSlots entries goes to its place in the output CSR in ascending order.
+constexpr int kRowSlots = 32;
+void launch_rows_from_slots(const OutSlot* out, long long n, const int* slots, cudaStream_t s);
+
 // Guards the per-device caches of kernel attributes (shared-memory limits, occupancy) that
 // the launch code keeps in statics: builds of several contexts may launch from several host
 // threads at once (the serving lanes).

@@ -1718,6 +1718,48 @@ __global__ void __launch_bounds__(256) k_rowsort_thread(const OutSlot* out, long
   }
 }
 
+// Rows of at most kRowSlots entries from their slots to their places, one thread per row (the
+// register network of k_rowsort_thread between a 16-byte load per four entries and the store).
+__global__ void __launch_bounds__(128) k_rows_from_slots(const OutSlot* out, long long n,
+                                                         const int* __restrict__ slots) {
+  const long long* __restrict__ row_ptr = out->row_ptr;
+  int* col = out->col;
+  const long long row = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (row >= n) return;
+  const long long b = row_ptr[row];
+  const int len = (int)min(row_ptr[row + 1] - b, (long long)kRowSlots + 1);
+  if (len == 0 || len > kRowSlots || b + len > out->col_cap) return;
+  const int4* src = reinterpret_cast<const int4*>(slots + row * kRowSlots);
+  auto load = [&](int* v, int words) {
+#pragma unroll
+    for (int q = 0; q < kRowSlots / 4; ++q)
+      if (q < words) {
+        const int4 x = 4 * q < len ? __ldg(src + q) : make_int4(INT_MAX, INT_MAX, INT_MAX, INT_MAX);
+        v[4 * q] = x.x;
+        v[4 * q + 1] = 4 * q + 1 < len ? x.y : INT_MAX;
+        v[4 * q + 2] = 4 * q + 2 < len ? x.z : INT_MAX;
+        v[4 * q + 3] = 4 * q + 3 < len ? x.w : INT_MAX;
+      }
+  };
+  if (len <= 16) {
+    int v[16];
+    load(v, 4);
+    if (len <= 4) bitonic_regs<4>(v);
+    else if (len <= 8) bitonic_regs<8>(v);
+    else bitonic_regs<16>(v);
+#pragma unroll
+    for (int q = 0; q < 16; ++q)
+      if (q < len) col[b + q] = v[q];
+  } else {
+    int v[32];
+    load(v, 8);
+    bitonic_regs<32>(v);
+#pragma unroll
+    for (int q = 0; q < 32; ++q)
+      if (q < len) col[b + q] = v[q];
+  }
+}
+
 // One row of at most 32 V entries sorted by one warp: lane l holds entries l V .. l V + V - 1
 // in registers (+infinity padding); bitonic network, exchanges across lanes by shuffles.
 template <int V>
@@ -2420,6 +2462,10 @@ int launch_rowsort(const BuildArgs& a, cudaStream_t s, long long col_bound) {
   k_rowsort_queued<<<(unsigned)(3 * a.num_sms), kRowSortThreads, smem, s>>>(
       a.out, a.n_total, a.row_cnt, long_count, bits);
   return 3;
+}
+
+void launch_rows_from_slots(const OutSlot* out, long long n, const int* slots, cudaStream_t s) {
+  if (n > 0) k_rows_from_slots<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(out, n, slots);
 }
 
 }  // namespace rtg

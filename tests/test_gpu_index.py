@@ -128,3 +128,28 @@ def test_empty_cases_and_errors(ctx):
     assert res.nnz == 0 and np.array_equal(rp, np.zeros(6, dtype=np.int64))
     res.release()
     ix0.close()
+
+
+@pytest.mark.parametrize("n,d,m,nq,dtype", [(6000, 3, 1, 1, np.float64), (6000, 4, 7, 37, np.float32),
+                                            (9000, 6, 8, 33, np.float64), (3000, 2, 64, 5, np.float32),
+                                            (4000, 9, 3, 86, np.float64)])
+def test_more_answers_than_slots(ctx, n, d, m, nq, dtype):
+    # light cells but for one spot of 33 and one of 32 points: queries there have more answers
+    # than are collected in slots, or just as many, next to queries with few and none
+    rng = np.random.default_rng(n + m)
+    pts = rng.random((n, d))
+    r = gen.radius_for_degree(n, d, 4.0)
+    spots = np.full(d, 0.5), np.full(d, 3.0)
+    for k, (spot, many) in enumerate(zip(spots, (33, 32))):
+        pts[100 * k:100 * k + many] = spot + rng.normal(0.0, 1e-3 * r, (many, d))
+    pts = pts.astype(dtype)
+    q = np.vstack([spots[0], spots[1], rng.random((max(nq - 2, 0), d))])[:nq].astype(dtype)
+    T = gen.transforms(n + m, d, m, r)
+    ix = ctx.index(pts, r, T, r)
+    for queries in (q, q[::-1].copy()):
+        res = ix.query(queries)
+        ref = oracle.rtg_query(pts, r, T, r, queries)
+        _compare(res, ref)
+        assert np.diff(ref.row_ptr).max() >= 33
+        res.release()
+    ix.close()
