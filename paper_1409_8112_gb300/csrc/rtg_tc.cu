@@ -170,7 +170,7 @@ struct TcSink {
   int symmetric;
 };
 
-__device__ __noinline__ double exact_dist2(const void* pts, int dtype, long long i, long long j,
+__device__ __forceinline__ double exact_dist2(const void* pts, int dtype, long long i, long long j,
                                            int d) {
   double s = 0.0;
   for (int l = 0; l < d; ++l) {
@@ -182,18 +182,19 @@ __device__ __noinline__ double exact_dist2(const void* pts, int dtype, long long
 
 // A pair the tile did not reject: decided with the FP64 reference sequence (only rejections
 // rely on the error bound); [lo, hi] is where the tile alone could not decide.
-__device__ __noinline__ void tc_candidate(float d2, long long gi, long long gj, const Inst& I,
-                                          const InstPlan& IP, int dtype, float lo_thr,
+__device__ __forceinline__ void tc_candidate(float d2, long long gi, long long gj, const Inst* Ip,
+                                             const InstPlan* IPp, int dtype, float lo_thr,
                                           const TcSink& sk, bool emit, unsigned int& pairs,
                                           unsigned int& rechecks, unsigned int& near_r,
                                           float& max_err, bool& overflow) {
+  const Inst& I = *Ip;  // (read where it is used: the epilogue has no registers to spare)
   const double s = exact_dist2(I.pts, dtype, gi, gj, I.d);
   max_err = fmaxf(max_err, (float)fabs((double)d2 - s));
   if (!(d2 < lo_thr)) {  // (every pair within 1e-12 r of r lies in the band: it is 1e-3 r^2 wide)
     ++rechecks;
     if (fabs(__dsub_rn(__dsqrt_rn(s), I.r)) <= __dmul_rn(1e-12, I.r)) ++near_r;
   }
-  if (!(s <= IP.rr)) return;
+  if (!(s <= IPp->rr)) return;
   ++pairs;
   const unsigned int i = (unsigned int)(I.p0 + gi), j = (unsigned int)(I.p0 + gj);
   if (emit) {
@@ -207,14 +208,14 @@ __device__ __noinline__ void tc_candidate(float d2, long long gi, long long gj, 
 
 // Candidates queued per warp before their exact check.  A check waits on the points' loads for
 // about two microseconds, and the accumulators wait with it, so a warp collects many: the
-// warps of a CTA then mostly check at the same time (at the end, at 200k points).  A chunk with
-// more candidates than this (dense inputs: up to 32 x 32) is decided by its lanes directly.
+// warps of a CTA then mostly check at the same time (at the end, at 200k points).  The check is
+// inlined: a call makes the compiler keep the accumulators a warp holds in local memory.
 constexpr int kTcQueue = 768;
 
 // Decides the qn queued candidates of a warp, 32 at a time (one per lane).  Called by all lanes.
 __device__ __forceinline__ void tc_drain(const unsigned int* q_i, const unsigned int* q_j,
                                          const float* q_d, unsigned int qn, int lane,
-                                         const Inst& I, const InstPlan& IP, int dtype,
+                                         const Inst* I, const InstPlan* IP, int dtype,
                                          float lo_thr, const TcSink& sk, bool emit,
                                          unsigned int& pairs, unsigned int& rechecks,
                                          unsigned int& near_r, float& max_err, bool& overflow) {
@@ -305,7 +306,7 @@ __device__ __forceinline__ bool tc_elect() {
 // the reads of the others.  Both run their loops as whole warps and elect a lane for the copies
 // and MMAs (a single lane running the loop, copies included, took 1500 clocks a job).  Eight
 // epilogue warps read the accumulators: warp w the rows of its quadrant w % 4 of row tile w / 4,
-// in four loads of 32 columns kept in registers; then the accumulator is free again.  No block
+// in four loads of 32 columns, two at a time; then the accumulator is free again.  No block
 // barrier in the loop.
 // An epilogue chunk of 32 columns is first reduced to its smallest d^2 with three-input minima
 // (16 instructions for 32 values); only a chunk that holds a value not above the threshold (one
@@ -313,8 +314,10 @@ __device__ __forceinline__ bool tc_elect() {
 // halves what the column tiles cost in L2 bandwidth (8 KB a job: 8 KB per 128 rows would be
 // near 60 bytes a clock and SM).
 // 200k points in 6-D (2e10 pair tests), FP16: 7.26 ms with 128 x 128 jobs, 4 CTAs per SM, block
-// barriers and a mask for every chunk; 4.27 now, of which the candidates take 1.5 and the
-// waits of a job (an accumulator handed to the epilogue and back) most of the rest.
+// barriers and a mask for every chunk; 4.27 with the warps above but the candidates' check in a
+// call (the warps' 128 accumulator values then lived in local memory); 3.47 now, most of it the
+// waits of a job (an accumulator handed to the epilogue and back); the TMEM reads alone would
+// take 0.8 ms, the MMAs 0.5.
 template <bool BF16, bool EMIT, int FORM>
 __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
     const unsigned char* __restrict__ tiles, const float* __restrict__ norms,
@@ -473,16 +476,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
                 "l"(ad), "l"(bd), "r"(idesc), "r"(part > 0 ? 1u : 0u));
           }
           tc_commit(&acc_full[u]);
+          if (mt == 1) {
+            tc_commit(&b_empty[slot]);
+            if (bj + 1 == ntile) tc_commit(&a_empty[(change - 1) & 1]);
+          }
         }
         __syncwarp();
       }
       if (!ok) break;
-      const bool last_of_I = bj + 1 == ntile;
-      if (tc_elect()) {
-        tc_commit(&b_empty[slot]);
-        if (last_of_I) tc_commit(&a_empty[(change - 1) & 1]);
-      }
-      __syncwarp();
       if (++bj == ntile) {
         ++I;
         bj = 2 * I;
@@ -496,10 +497,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
     tc_wait(&all_done, 0u, wait_limit, &never);
     __syncwarp();
   } else {
-    const Inst In = inst[0];
-    const InstPlan IP = iplan[0];
-    const float lo_thr = tp->lo, hi_thr = tp->hi;
-    const long long n = In.n;
+    const float hi_thr = tp->hi;
     const int quad = warp & 3, mt = warp >> 2;
     unsigned int* q_i = reinterpret_cast<unsigned int*>(smem + (4 + kTcSlots) * kTcTileBytes) +
                         (size_t)warp * 3 * kTcQueue;  // rows, columns, tile d^2
@@ -519,111 +517,101 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
       const long long gi = (2LL * I + mt) * kTcRows + quad * 32 + lane;
       // a job on the diagonal, or with columns past the points
       const bool edge = bj < 2 * I + 2 || bj == ntile - 1;
-      float d2[4][32], least[4];
       const uint32_t acc = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(u * 128);
+      // 64 columns at a time: a warp that held all 128 would spill
 #pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        uint32_t r[32];
-        tc_ld32(acc + (uint32_t)(h * 32), r);
-        if (FORM == kTcPlain) {
-          const float nrow = gi < nt * kTcRows ? __ldg(norms + gi) : 0.0f;
-          const float4* nb = reinterpret_cast<const float4*>(norms + (long long)bj * kTcRows + h * 32);
+      for (int g = 0; g < 2; ++g) {
+        float d2[2][32], least[2];
 #pragma unroll
-          for (int v = 0; v < 8; ++v) {
-            const float4 c4 = __ldg(nb + v);
-            d2[h][4 * v] = (nrow + c4.x) - 2.0f * __uint_as_float(r[4 * v]);
-            d2[h][4 * v + 1] = (nrow + c4.y) - 2.0f * __uint_as_float(r[4 * v + 1]);
-            d2[h][4 * v + 2] = (nrow + c4.z) - 2.0f * __uint_as_float(r[4 * v + 2]);
-            d2[h][4 * v + 3] = (nrow + c4.w) - 2.0f * __uint_as_float(r[4 * v + 3]);
+        for (int h = 0; h < 2; ++h) {
+          uint32_t r[32];
+          tc_ld32(acc + (uint32_t)(g * 64 + h * 32), r);
+          if (FORM == kTcPlain) {
+            const float nrow = gi < nt * kTcRows ? __ldg(norms + gi) : 0.0f;
+            const float4* nb = reinterpret_cast<const float4*>(norms + (long long)bj * kTcRows + g * 64 + h * 32);
+#pragma unroll
+            for (int v = 0; v < 8; ++v) {
+              const float4 c4 = __ldg(nb + v);
+              d2[h][4 * v] = (nrow + c4.x) - 2.0f * __uint_as_float(r[4 * v]);
+              d2[h][4 * v + 1] = (nrow + c4.y) - 2.0f * __uint_as_float(r[4 * v + 1]);
+              d2[h][4 * v + 2] = (nrow + c4.z) - 2.0f * __uint_as_float(r[4 * v + 2]);
+              d2[h][4 * v + 3] = (nrow + c4.w) - 2.0f * __uint_as_float(r[4 * v + 3]);
+            }
+          } else {
+#pragma unroll
+            for (int v = 0; v < 32; ++v) d2[h][v] = __uint_as_float(r[v]);
           }
-        } else {
+          float m0 = d2[h][0], m1 = d2[h][1];
 #pragma unroll
-          for (int v = 0; v < 32; ++v) d2[h][v] = __uint_as_float(r[v]);
-        }
-        float m0 = d2[h][0], m1 = d2[h][1];
-#pragma unroll
-        for (int v = 2; v + 3 < 32; v += 4) {
-          m0 = min3_nan(m0, d2[h][v], d2[h][v + 1]);
-          m1 = min3_nan(m1, d2[h][v + 2], d2[h][v + 3]);
-        }
-        m0 = min3_nan(m0, d2[h][30], d2[h][31]);
-        least[h] = min3_nan(m0, m1, m1);
-      }
-      asm volatile("tcgen05.fence::before_thread_sync;");
-      __syncwarp();
-      if (lane == 0)
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[u]))
-                     : "memory");
-#pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        if (!__any_sync(full, !(least[h] > hi_thr))) continue;  // (NaN goes on)
-        const long long colbase = (long long)bj * kTcRows + h * 32;
-        uint32_t hits = 0;
-#pragma unroll
-        for (int v = 0; v < 32; ++v)
-          hits |= (d2[h][v] > hi_thr ? 0u : 1u) << v;  // NaN (overflowed tiles) goes to FP64
-        if (edge) {  // columns v with gi < colbase + v < n
-          const long long vlo = gi - colbase + 1, vhi = n - colbase;
-          uint32_t valid = 0;
-          if (vlo < 32 && vhi > 0) {
-            const int a0 = vlo > 0 ? (int)vlo : 0, a1 = vhi < 32 ? (int)vhi : 32;
-            if (a1 > a0) valid = (a1 - a0 == 32 ? full : ((1u << (a1 - a0)) - 1u)) << a0;
+          for (int v = 2; v + 3 < 32; v += 4) {
+            m0 = min3_nan(m0, d2[h][v], d2[h][v + 1]);
+            m1 = min3_nan(m1, d2[h][v + 2], d2[h][v + 3]);
           }
-          hits &= valid;
+          m0 = min3_nan(m0, d2[h][30], d2[h][31]);
+          least[h] = min3_nan(m0, m1, m1);
         }
-        // queue this chunk's candidates (the warp's shared-memory queue, kept across jobs); they
-        // are decided 32 at a time, one per lane, so that the FP64 checks and their global loads
-        // run in parallel
-        const unsigned int nh = (unsigned int)__popc(hits);
-        const unsigned int who = __ballot_sync(full, nh != 0);
-        if (!who) continue;
-        if (qn + 32u > (unsigned int)kTcQueue) {  // room for one per lane
-          tc_drain(q_i, q_j, q_d, qn, lane, In, IP, dtype, lo_thr, sk, EMIT, tl_pairs,
-                   tl_rechecks, tl_near, max_err, overflow);
-          qn = 0;
+        if (g == 1) {  // read: the accumulator is free
+          asm volatile("tcgen05.fence::before_thread_sync;");
+          __syncwarp();
+          if (lane == 0)
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[u]))
+                         : "memory");
         }
-        if (!edge && !__any_sync(full, nh > 1u)) {
-          // (nearly always) at most one a lane, which is the lane's smallest value
-          if (nh) {
-            const unsigned int pos = qn + (unsigned int)__popc(who & ((1u << lane) - 1u));
-            q_i[pos] = (unsigned int)gi;
-            q_j[pos] = (unsigned int)(colbase + __ffs(hits) - 1);
-            q_d[pos] = least[h];
-          }
-          qn += (unsigned int)__popc(who);
-          continue;
-        }
-        unsigned int incl = nh;
+        // Candidates go to the warp's shared-memory queue, kept across jobs, and are decided 32 at
+        // a time, one per lane, so that the FP64 checks and their global loads run in parallel.
+        const bool found = __any_sync(
+            full, !(min3_nan(least[0], least[1], least[1]) > hi_thr));
+        if (found) {  // (NaN too)
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const unsigned int y = __shfl_up_sync(full, incl, o);
-          if (lane >= o) incl += y;
-        }
-        const unsigned int total = __shfl_sync(full, incl, 31);
-        if (total > (unsigned int)kTcQueue) {
+          for (int h = 0; h < 2; ++h) {
+            if (!__any_sync(full, !(least[h] > hi_thr))) continue;
+            const unsigned int col0 = (unsigned int)bj * kTcRows + g * 64 + h * 32;
+            // NaN (overflowed tiles) goes to FP64; four chains, for the latency
+            uint32_t m0 = 0, m1 = 0, m2 = 0, m3 = 0;
 #pragma unroll
-          for (int v = 0; v < 32; ++v)
-            if (hits & (1u << v))
-              tc_candidate(d2[h][v], gi, colbase + v, In, IP, dtype, lo_thr, sk, EMIT, tl_pairs,
-                           tl_rechecks, tl_near, max_err, overflow);
-        } else if (total) {
-          if (qn + total > (unsigned int)kTcQueue) {  // room for the chunk: the queue first
-            tc_drain(q_i, q_j, q_d, qn, lane, In, IP, dtype, lo_thr, sk, EMIT, tl_pairs,
-                     tl_rechecks, tl_near, max_err, overflow);
-            qn = 0;
-          }
-          unsigned int pos = qn + incl - nh;
-          if (hits) {
-#pragma unroll
-            for (int v = 0; v < 32; ++v)
-              if (hits & (1u << v)) {
-                q_i[pos] = (unsigned int)gi;
-                q_j[pos] = (unsigned int)(colbase + v);
-                q_d[pos] = d2[h][v];
-                ++pos;
+            for (int v = 0; v < 8; ++v) {
+              if (!(d2[h][v] > hi_thr)) m0 |= 1u << v;
+              if (!(d2[h][8 + v] > hi_thr)) m1 |= 1u << (8 + v);
+              if (!(d2[h][16 + v] > hi_thr)) m2 |= 1u << (16 + v);
+              if (!(d2[h][24 + v] > hi_thr)) m3 |= 1u << (24 + v);
+            }
+            uint32_t hits = (m0 | m1) | (m2 | m3);
+            if (edge) {  // columns v with gi < col0 + v < n
+              const long long vlo = gi - (long long)col0 + 1, vhi = (long long)inst->n - (long long)col0;
+              uint32_t valid = 0;
+              if (vlo < 32 && vhi > 0) {
+                const int a0 = vlo > 0 ? (int)vlo : 0, a1 = vhi < 32 ? (int)vhi : 32;
+                if (a1 > a0) valid = (a1 - a0 == 32 ? full : ((1u << (a1 - a0)) - 1u)) << a0;
               }
+              hits &= valid;
+            }
+            // one candidate a lane and round: a lane's only one is its smallest value (the usual
+            // round), others are picked out of the registers
+            uint32_t who = __ballot_sync(full, hits != 0u);
+            bool only = !edge && (hits & (hits - 1u)) == 0u;
+            while (who) {
+              if (qn + 32u > (unsigned int)kTcQueue) {
+                tc_drain(q_i, q_j, q_d, qn, lane, inst, iplan, dtype, tp->lo, sk, EMIT, tl_pairs,
+                         tl_rechecks, tl_near, max_err, overflow);
+                qn = 0;
+              }
+              if (hits) {
+                const int v = __ffs(hits) - 1;
+                float x = least[h];
+                if (!only) {
+#pragma unroll
+                  for (int z = 0; z < 32; ++z) x = z == v ? d2[h][z] : x;
+                }
+                const unsigned int pos = qn + (unsigned int)__popc(who & ((1u << lane) - 1u));
+                q_i[pos] = (unsigned int)gi;
+                q_j[pos] = col0 + (unsigned int)v;
+                q_d[pos] = x;
+                hits &= hits - 1u;
+              }
+              qn += (unsigned int)__popc(who);
+              who = __ballot_sync(full, hits != 0u);
+            }
           }
-          qn += total;
         }
       }
       if (++bj == ntile) {
@@ -632,7 +620,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
       }
     }
     if (qn)  // the candidates still queued
-      tc_drain(q_i, q_j, q_d, qn, lane, In, IP, dtype, lo_thr, sk, EMIT, tl_pairs, tl_rechecks,
+      tc_drain(q_i, q_j, q_d, qn, lane, inst, iplan, dtype, tp->lo, sk, EMIT, tl_pairs, tl_rechecks,
                tl_near, max_err, overflow);
     // tallies
     for (int o = 16; o > 0; o >>= 1) {
