@@ -8,10 +8,17 @@
 // same expression in FP32 and proves, per coordinate, that floor() of the FP64 value equals
 // floor() of the FP32 estimate: with A = |s_k| + sum_l |R_kl| max|p_l| the FP32 estimate of
 // y_k / c is within E = (d + 6) 2^-24 A / c of the FP64 quotient (rounding of R, s and p to
-// FP32, d rounded fmas, the rounded reciprocal and product; the FP64 chain's own error is
-// below 2^-29 of that).  When [u - E, u + E] holds no integer the FP32 floor is exact;
-// otherwise the coordinate is recomputed with the FP64 sequence.  E is widened by 3e-12 / c
-// so every coordinate within 1e-12 of a wall takes the FP64 path, where it is counted.
+// FP32, the rounded reciprocal of c and its product with R and s, d rounded fmas; the FP64
+// chain's own error is below 2^-29 of that).  When [u - E, u + E] holds no integer the FP32
+// floor is exact; otherwise the coordinate is recomputed with the FP64 sequence.  E is widened
+// by 3e-12 / c so every coordinate within 1e-12 of a wall takes the FP64 path, where it is
+// counted.
+//
+// The floor takes no conversion instruction (a quarter of a warp's issue rate or less): for
+// |u| < 2^22 the sum u + 1.5 2^23, rounded down, is 1.5 2^23 + floor(u) exactly, its low bits
+// hold floor(u), and the distance to the cell's walls follows from u - floor(u), which is exact
+// but for a rounding of at most 2^-25 when u is just below zero.  |u - floor(u) - 1/2| <= 1/2 - E
+// - 2^-23 (cell_slack) then proves the floor; at |u| >= 2^22 E exceeds 1/2 and nothing is proved.
 #include <cuda_runtime.h>
 
 #include <cfloat>
@@ -391,13 +398,21 @@ __device__ __noinline__ long long exact_cell(const void* pts, int dtype, long lo
   return (long long)floor(u);
 }
 
+constexpr float kFloorBias = 12582912.0f;              // 1.5 2^23
+constexpr unsigned int kFloorBits = 0x4B400000u;       // its bit pattern
+// What |u - floor(u) - 1/2| may be at most for floor(u) to be certain, given E: below
+// 1/2 - E by more than the rounding of that expression (2^-25 + 2^-26).
+__device__ __forceinline__ float cell_slack(float E) {
+  return __fsub_rd(__fsub_rd(0.5f, E), 0x1.0p-23f);
+}
+
 // One (grid, axis) row of the key computation, 16-byte aligned in shared memory so that a
-// thread reads it with a few vector loads: the FP32 rotation row, the FP32 shift and error
-// bound, and the axis's cell range and key stride.
+// thread reads it with a few vector loads: the FP32 rotation row and shift in units of the cell
+// side, the slack (cell_slack), and the axis's cell range and key stride.
 template <int DPAD>
 struct __align__(16) AxisRow {
   float R[DPAD];
-  float s, E;
+  float s, slack;
   float pad0, pad1;
   long long qlo;
   unsigned long long ext;
@@ -433,16 +448,15 @@ __global__ void __launch_bounds__(kPointBlock) k_keys(
     const int t = x / d, k = x - t * d;
     AxisRow<DPAD>& A = rows[x];
 #pragma unroll
-    for (int l = 0; l < DPAD; ++l) A.R[l] = Gb[t].Rf[k * kMaxDim + l];
-    A.s = Gb[t].sf[k];
-    A.E = Gb[t].E[k];
+    for (int l = 0; l < DPAD; ++l) A.R[l] = __fmul_rn(Gb[t].Rf[k * kMaxDim + l], I.inv_cf);
+    A.s = __fmul_rn(Gb[t].sf[k], I.inv_cf);
+    A.slack = cell_slack(Gb[t].E[k]);
     A.qlo = Gb[t].qlo[k];
     A.ext = Gb[t].ext[k];
     A.stride = Gb[t].stride[k];
   }
   for (int t = threadIdx.x; t < m; t += blockDim.x) sbase[t] = Gb[t].base;
   __syncthreads();
-  const float inv_c = I.inv_cf;
   if (threadIdx.x == 0 && blockIdx.x == I.blk0) plan_band(b, I, dtype, bbox, iplan);
   const double c = I.c;
   const long long i = (blockIdx.x - I.blk0) * (long long)kPointBlock + threadIdx.x;
@@ -472,23 +486,20 @@ __global__ void __launch_bounds__(kPointBlock) k_keys(
       unsigned int redo = 0;  // axes whose FP32 index is not certain
       for (int k = 0; k < dv; ++k) {
         const float2 se = *reinterpret_cast<const float2*>(&A[k].s);
-        float y = se.x;
+        float u = se.x;
 #pragma unroll
         for (int v = 0; v < DPAD / 4; ++v) {
+          if (4 * v >= d) break;  // (block-uniform: a mixed batch is padded to its widest d)
           const float4 r = reinterpret_cast<const float4*>(A[k].R)[v];
-          y = fmaf(r.x, p[4 * v], y);
-          y = fmaf(r.y, p[4 * v + 1], y);
-          y = fmaf(r.z, p[4 * v + 2], y);
-          y = fmaf(r.w, p[4 * v + 3], y);
+          u = fmaf(r.x, p[4 * v], u);
+          u = fmaf(r.y, p[4 * v + 1], u);
+          u = fmaf(r.z, p[4 * v + 2], u);
+          u = fmaf(r.w, p[4 * v + 3], u);
         }
-        const float u = y * inv_c;
-        // the FP32 index is certain when [u - E, u + E] holds no cell wall: both ends (rounded
-        // outwards) lie in [floor(u), floor(u) + 1).  |u| >= 2^23 always fails (u is then an
-        // integer and u - E < u), so floor(u) is exact in 32-bit integers here.
-        const float f = floorf(u);
-        const bool certain = __fsub_rd(u, se.y) >= f && __fadd_ru(u, se.y) < f + 1.0f;
+        const float w = __fadd_rd(u, kFloorBias);
+        const bool certain = fabsf(u - (w - kFloorBias) - 0.5f) <= se.y;
         const longlong2 qe = *reinterpret_cast<const longlong2*>(&A[k].qlo);
-        long long off = (long long)(int)f - qe.x;
+        long long off = (long long)(int)(__float_as_uint(w) - kFloorBits) - qe.x;
         const bool out = (unsigned long long)off >= (unsigned long long)qe.y;
         if (!certain) redo |= 1u << k;
         if (certain && out) range_err = true;
@@ -605,13 +616,13 @@ constexpr int kKeyLaneThreads = 256;
 // Per (axis, grid) record of k_keys_lanes.
 template <typename K>
 struct __align__(16) LaneAxis {
-  float E;
+  float slack;
   unsigned int pad;
   K qlo, ext, stride;
 };
 template <>
 struct __align__(16) LaneAxis<uint32_t> {
-  float E;
+  float slack;
   uint32_t qlo, ext, stride;
 };
 
@@ -727,7 +738,7 @@ __global__ void __launch_bounds__(kKeyLaneThreads, 2) k_keys_lanes(
       for (int x = threadIdx.x; x < D * m; x += blockDim.x) {
         const int a = x / m, g = x - a * m;
         LaneAxis<K> r;
-        r.E = Gb[g].E[a];
+        r.slack = cell_slack(Gb[g].E[a]);
         r.qlo = (K)Gb[g].qlo[a];
         r.ext = (K)Gb[g].ext[a];
         r.stride = (K)Gb[g].stride[a];
@@ -738,8 +749,8 @@ __global__ void __launch_bounds__(kKeyLaneThreads, 2) k_keys_lanes(
 #pragma unroll
       for (int a = 0; a < D; ++a) {
 #pragma unroll
-        for (int l = 0; l < D; ++l) R[a][l] = G->Rf[a * kMaxDim + l];
-        sf[a] = G->sf[a];
+        for (int l = 0; l < D; ++l) R[a][l] = __fmul_rn(G->Rf[a * kMaxDim + l], I.inv_cf);
+        sf[a] = __fmul_rn(G->sf[a], I.inv_cf);
       }
       base = (K)G->base;
       cur_b = ci.b;
@@ -754,7 +765,6 @@ __global__ void __launch_bounds__(kKeyLaneThreads, 2) k_keys_lanes(
     }
     phase ^= 1u << buf;
     pending &= ~(1u << buf);
-    const float inv_c = I.inv_cf;
     const float* rows = s_rows[buf];
     K* out = key_mat + ci.g0 * m + (long long)(slot * m + t);  // this thread's first word
     for (int p0 = 0; p0 < ci.npts; p0 += P, out += P * m) {  // block-uniform
@@ -774,15 +784,13 @@ __global__ void __launch_bounds__(kKeyLaneThreads, 2) k_keys_lanes(
       unsigned int redo = 0;
 #pragma unroll
       for (int a = 0; a < D; ++a) {
-        float y = sf[a];
+        float u = sf[a];
 #pragma unroll
-        for (int l = 0; l < D; ++l) y = fmaf(R[a][l], x[l], y);
+        for (int l = 0; l < D; ++l) u = fmaf(R[a][l], x[l], u);
         const LaneAxis<K> ax = s_ax[a * m + t];
-        const float u = y * inv_c;
-        const float f = floorf(u);
-        // certain when [u - E, u + E], rounded outwards, holds no cell wall (as in k_keys)
-        const bool certain = __fsub_rd(u, ax.E) >= f && __fadd_ru(u, ax.E) < f + 1.0f;
-        const K off = (K)(long long)(int)f - ax.qlo;
+        const float w = __fadd_rd(u, kFloorBias);
+        const bool certain = fabsf(u - (w - kFloorBias) - 0.5f) <= ax.slack;
+        const K off = (K)(long long)(int)(__float_as_uint(w) - kFloorBits) - ax.qlo;
         const bool out = off >= ax.ext;
         if (!certain) redo |= 1u << a;
         if (certain && out) range_err = true;
