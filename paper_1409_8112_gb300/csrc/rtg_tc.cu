@@ -36,7 +36,7 @@ constexpr int kTcTileBytes = kTcRows * kTcK * 2;  // 8 KB per 128-point tile
 // a clock and SM with 4 warps, 323 with 8 and 60 with 16 (two loads in flight: 235 with 8).
 constexpr int kTcEpiWarps = 8;
 constexpr int kTcThreads = (kTcEpiWarps + 2) * 32;  // and one that copies tiles, one for the MMAs
-constexpr int kTcSlots = 4;                       // column tiles in shared memory
+constexpr int kTcSlots = 3;                       // pairs of column tiles in shared memory
 // MMA completion waits: the context's spin limit times this (a commit takes far longer than
 // one look-back step)
 constexpr unsigned int kTcWaitScale = 16;
@@ -277,20 +277,14 @@ __device__ __forceinline__ void tc_commit(const uint64_t* bar) {
       : "memory");
 }
 
-// Jobs of the brute force: 256 rows (row tiles 2 I and 2 I + 1) against the 128 columns of tile
-// bj >= 2 I, I-major.  First job of I.
-__host__ __device__ inline long long tc_first_job(long long I, long long nt) {
-  return I * nt - I * (I - 1);
-}
-
-__host__ __device__ inline long long tc_jobs(long long nt) {
-  // sum over I < ceil(nt / 2) of nt - 2 I
-  const long long nI = (nt + 1) / 2;
-  return nI * nt - nI * (nI - 1);
+// Jobs of the brute force: blocks of 256 rows (row tiles 2 I and 2 I + 1) against blocks of 256
+// columns, J >= I, I-major.  First job of I among nb blocks.
+__host__ __device__ inline long long tc_first_job(long long I, long long nb) {
+  return I * nb - I * (I - 1) / 2;
 }
 
 // Shared memory of k_brute_tc: two pairs of row tiles, the column tiles, the candidate queues.
-constexpr size_t kTcSmem = (4 + kTcSlots) * (size_t)kTcTileBytes +
+constexpr size_t kTcSmem = (4 + 2 * kTcSlots) * (size_t)kTcTileBytes +
                            (size_t)kTcEpiWarps * 3 * kTcQueue * 4 + 1024;
 
 // One lane of a converged warp.
@@ -302,22 +296,21 @@ __device__ __forceinline__ bool tc_elect() {
 
 // Persistent, one CTA per SM, each with a contiguous range of jobs.  One warp copies the tiles in
 // (bulk copies: column tiles up to kTcSlots jobs ahead, row tiles one change ahead), one issues
-// the MMAs: a job's two 128 x 128 accumulators are two of four, so that the MMAs of one overlap
-// the reads of the others.  Both run their loops as whole warps and elect a lane for the copies
-// and MMAs (a single lane running the loop, copies included, took 1500 clocks a job).  Eight
-// epilogue warps read the accumulators: warp w the rows of its quadrant w % 4 of row tile w / 4,
-// in four loads of 32 columns, two at a time; then the accumulator is free again.  No block
-// barrier in the loop.
+// the MMAs, 128 x 256 each: a job's two row tiles are the two accumulators of 256 columns, so
+// that the MMAs of one overlap the reads of the other.  Both run their loops as whole warps and
+// elect a lane for the copies and MMAs (a single lane running the loop, copies included, took
+// 1500 clocks a 256 x 128 job).  Eight epilogue warps read the accumulators in turn: warp w the
+// rows of its quadrant w % 4, columns 128 (w / 4) on, in four loads of 32 columns, two at a
+// time; then the accumulator is free again.  No block barrier in the loop.
 // An epilogue chunk of 32 columns is first reduced to its smallest d^2 with three-input minima
 // (16 instructions for 32 values); only a chunk that holds a value not above the threshold (one
-// in eleven at 200k points, degree 24) builds the mask of its candidates.  A job of 256 rows
-// halves what the column tiles cost in L2 bandwidth (8 KB a job: 8 KB per 128 rows would be
-// near 60 bytes a clock and SM).
+// in eleven at 200k points, degree 24) builds the mask of its candidates.  A job of 256 x 256
+// costs 16 KB of column tiles for four tile pairs (8 KB for each would be near 60 bytes a clock
+// and SM of L2 bandwidth).
 // 200k points in 6-D (2e10 pair tests), FP16: 7.26 ms with 128 x 128 jobs, 4 CTAs per SM, block
-// barriers and a mask for every chunk; 4.27 with the warps above but the candidates' check in a
-// call (the warps' 128 accumulator values then lived in local memory); 3.47 now, most of it the
-// waits of a job (an accumulator handed to the epilogue and back); the TMEM reads alone would
-// take 0.8 ms, the MMAs 0.5.
+// barriers and a mask for every chunk; 3.37 now: 1.84 without candidates (the TMEM reads alone
+// would take 0.8, the MMAs 0.5), the rest for the 1.8 million candidates, for each of which a
+// warp stops about 800 clocks and the others wait for its accumulator.
 template <bool BF16, bool EMIT, int FORM>
 __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
     const unsigned char* __restrict__ tiles, const float* __restrict__ norms,
@@ -326,8 +319,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
     unsigned int wait_limit, unsigned int inject) {
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* s_a = smem;                      // row tiles 2 I, 2 I + 1, of two I
-  unsigned char* s_b = smem + 4 * kTcTileBytes;   // kTcSlots column tiles
-  __shared__ __align__(8) uint64_t b_full[kTcSlots], b_empty[kTcSlots], acc_full[4], acc_empty[4],
+  unsigned char* s_b = smem + 4 * kTcTileBytes;   // kTcSlots pairs of column tiles
+  __shared__ __align__(8) uint64_t b_full[kTcSlots], b_empty[kTcSlots], acc_full[2], acc_empty[2],
       a_full[2], a_empty[2], all_done, b_idle;  // b_idle: test hook, a barrier nothing arrives on
   __shared__ uint32_t tmem_base;
   __shared__ unsigned int s_cnt[4];
@@ -336,8 +329,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
   const unsigned int full = 0xffffffffu;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (!tp->use) return;  // the CUDA-core kernel takes the pairs
-  const long long nI = (nt + 1) / 2;
-  const long long jobs = tc_jobs(nt);
+  const long long nb = (nt + 1) / 2;  // blocks of 256 points
+  const long long jobs = tc_first_job(nb, nb);
   const long long per = (jobs + gridDim.x - 1) / gridDim.x;
   const long long j0 = min(jobs, (long long)blockIdx.x * per), j1 = min(jobs, j0 + per);
   if (tid < 4) s_cnt[tid] = 0;
@@ -351,11 +344,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
       init(&b_full[q], 1);
       init(&b_empty[q], 1);
     }
-    for (int q = 0; q < 4; ++q) {
-      init(&acc_full[q], 1);
-      init(&acc_empty[q], kTcEpiWarps / 2);
-    }
     for (int q = 0; q < 2; ++q) {
+      init(&acc_full[q], 1);
+      init(&acc_empty[q], kTcEpiWarps);
       init(&a_full[q], 1);
       init(&a_empty[q], 1);
     }
@@ -373,24 +364,24 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = tmem_base;
-  // first (I, bj) of this CTA
-  long long I0 = 0, bj0 = 0;
+  // first (I, J) of this CTA
+  long long I0 = 0, J0 = 0;
   if (j0 < j1) {
-    long long lo = 0, hi = nI - 1;
+    long long lo = 0, hi = nb - 1;
     while (lo < hi) {  // the last I whose first job is <= j0
       const long long mid = (lo + hi + 1) >> 1;
-      if (tc_first_job(mid, nt) <= j0) lo = mid; else hi = mid - 1;
+      if (tc_first_job(mid, nb) <= j0) lo = mid; else hi = mid - 1;
     }
     I0 = lo;
-    bj0 = 2 * lo + (j0 - tc_first_job(lo, nt));
+    J0 = lo + (j0 - tc_first_job(lo, nb));
   }
   const int count = (int)(j1 - j0);  // (at most 2^30)
-  const int ntile = (int)nt;
+  const int ntile = (int)nt, nblk = (int)nb;
 
   if (warp == kTcEpiWarps) {
     // copies.  (unless plain, the B operand's tiles follow the A operand's, and hold the norms)
     const unsigned char* tilesB = FORM != kTcPlain ? tiles + nt * (long long)kTcTileBytes : tiles;
-    int I = (int)I0, bj = (int)bj0, change = 0, a_copied = 0, p = 0;
+    int I = (int)I0, J = (int)J0, change = 0, a_copied = 0, p = 0;
     bool ok = true, fresh = true;
     for (; p < count; ++p) {
       if (fresh) {  // the next pair of row tiles (in use until the MMAs of the pair before last end)
@@ -398,7 +389,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
         if (change >= 2) ok = tc_wait(&a_empty[as], (uint32_t)(((change >> 1) - 1) & 1), wait_limit, &s_late);
         ok = __all_sync(full, ok);
         if (!ok) break;
-        const bool two = 2 * I + 1 < ntile;  // (else the second tile's rows lie beyond n: ignored)
+        const bool two = 2 * I + 1 < ntile;  // (else the second tile lies beyond n: ignored)
         if (tc_elect()) {
           tc_expect(&a_full[as], two ? 2 * kTcTileBytes : kTcTileBytes);
           const unsigned char* src = tiles + 2LL * I * kTcTileBytes;
@@ -417,13 +408,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
       ok = __all_sync(full, ok);
       if (!ok) break;
       if (tc_elect()) {
-        tc_expect(&b_full[slot], kTcTileBytes);
-        tc_bulk_copy(s_b + slot * kTcTileBytes, tilesB + (long long)bj * kTcTileBytes, kTcTileBytes,
-                     &b_full[slot]);
+        const bool two = 2 * J + 1 < ntile;
+        tc_expect(&b_full[slot], two ? 2 * kTcTileBytes : kTcTileBytes);
+        tc_bulk_copy(s_b + slot * 2 * kTcTileBytes, tilesB + 2LL * J * kTcTileBytes,
+                     two ? 2 * kTcTileBytes : kTcTileBytes, &b_full[slot]);
       }
-      if (++bj == ntile) {
-        ++I;
-        bj = 2 * I;
+      if (++J == nblk) {
+        J = ++I;
         fresh = true;
       }
     }
@@ -437,10 +428,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
   } else if (warp == kTcEpiWarps + 1) {
     // MMAs
     const uint32_t idesc = (1u << 4) | ((BF16 ? 1u : 0u) << 7) | ((BF16 ? 1u : 0u) << 10) |
-                           ((128u >> 3) << 17) | ((128u >> 4) << 24);
+                           ((256u >> 3) << 17) | ((128u >> 4) << 24);
     const bool one_part = FORM == kTcPacked && 3 * inst[0].d + 4 <= 16;
     const uint64_t adesc = make_desc(smem_u32(s_a)), bdesc = make_desc(smem_u32(s_b));
-    int I = (int)I0, bj = (int)bj0, change = 0;
+    int I = (int)I0, J = (int)J0, change = 0;
     bool ok = true, fresh = true;
     for (int q = 0; q < count; ++q) {
       const int slot = q % kTcSlots;
@@ -451,19 +442,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
       }
       if (ok) ok = tc_wait(&b_full[slot], (uint32_t)((q / kTcSlots) & 1), wait_limit, &s_late);
       const uint64_t ad0 = adesc + (uint64_t)(((change - 1) & 1) * 2 * (kTcTileBytes / 16));
-      const uint64_t bd0 = bdesc + (uint64_t)(slot * (kTcTileBytes / 16));
+      const uint64_t bd0 = bdesc + (uint64_t)(slot * 2 * (kTcTileBytes / 16));
 #pragma unroll
       for (int mt = 0; mt < 2; ++mt) {
-        const int u = (q & 1) * 2 + mt;
-        if (ok && q >= 2)  // the epilogue has read this accumulator's last job
-          ok = tc_wait(&acc_empty[u], (uint32_t)(((q >> 1) - 1) & 1), wait_limit, &s_late);
+        if (ok && q >= 1)  // the epilogue has read this accumulator's last job
+          ok = tc_wait(&acc_empty[mt], (uint32_t)((q - 1) & 1), wait_limit, &s_late);
         ok = __all_sync(full, ok);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;");
         if (tc_elect()) {
           // plain and folded: hi.hi + hi.lo + lo.hi, A parts (0, 0, 1), B parts (0, 1, 0);
           // packed: parts (0, 0), (1, 1); 256 bytes per part
-          const uint32_t d = tmem + (uint32_t)(u * 128);
+          const uint32_t d = tmem + (uint32_t)(mt * 256);
           const uint64_t am = ad0 + (uint64_t)(mt * (kTcTileBytes / 16));
 #pragma unroll
           for (int part = 0; part < (FORM == kTcPacked ? 2 : 3); ++part) {
@@ -475,18 +465,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
                 "l"(ad), "l"(bd), "r"(idesc), "r"(part > 0 ? 1u : 0u));
           }
-          tc_commit(&acc_full[u]);
+          tc_commit(&acc_full[mt]);
           if (mt == 1) {
             tc_commit(&b_empty[slot]);
-            if (bj + 1 == ntile) tc_commit(&a_empty[(change - 1) & 1]);
+            if (J + 1 == nblk) tc_commit(&a_empty[(change - 1) & 1]);
           }
         }
         __syncwarp();
       }
       if (!ok) break;
-      if (++bj == ntile) {
-        ++I;
-        bj = 2 * I;
+      if (++J == nblk) {
+        J = ++I;
         fresh = true;
       }
     }
@@ -498,8 +487,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
     __syncwarp();
   } else {
     const float hi_thr = tp->hi;
-    const int quad = warp & 3, mt = warp >> 2;
-    unsigned int* q_i = reinterpret_cast<unsigned int*>(smem + (4 + kTcSlots) * kTcTileBytes) +
+    const int quad = warp & 3, half = warp >> 2;
+    unsigned int* q_i = reinterpret_cast<unsigned int*>(smem + (4 + 2 * kTcSlots) * kTcTileBytes) +
                         (size_t)warp * 3 * kTcQueue;  // rows, columns, tile d^2
     unsigned int* q_j = q_i + kTcQueue;
     float* q_d = reinterpret_cast<float*>(q_j + kTcQueue);
@@ -507,17 +496,19 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
     unsigned int tl_pairs = 0, tl_rechecks = 0, tl_near = 0;
     bool overflow = false;
     float max_err = 0.0f;
-    int I = (int)I0, bj = (int)bj0;
-    for (int q = 0; q < count; ++q) {
-      const int u = (q & 1) * 2 + mt;
-      const bool ok = tc_wait((inject & kInjectTcWait) ? &b_idle : &acc_full[u],
-                              (uint32_t)((q >> 1) & 1), wait_limit, &s_late);
+    int I = (int)I0, J = (int)J0;
+    for (int unit = 0; unit < 2 * count; ++unit) {
+      const int q = unit >> 1, mt = unit & 1;
+      const bool ok = tc_wait((inject & kInjectTcWait) ? &b_idle : &acc_full[mt],
+                              (uint32_t)(q & 1), wait_limit, &s_late);
       if (!__all_sync(full, ok)) break;
       asm volatile("tcgen05.fence::after_thread_sync;");
       const long long gi = (2LL * I + mt) * kTcRows + quad * 32 + lane;
+      const unsigned int cbase = (unsigned int)(2 * J + half) * kTcRows;  // first column
       // a job on the diagonal, or with columns past the points
-      const bool edge = bj < 2 * I + 2 || bj == ntile - 1;
-      const uint32_t acc = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(u * 128);
+      const bool edge = J == I || J == nblk - 1;
+      const uint32_t acc =
+          tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(mt * 256 + half * 128);
       // 64 columns at a time: a warp that held all 128 would spill
 #pragma unroll
       for (int g = 0; g < 2; ++g) {
@@ -528,7 +519,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
           tc_ld32(acc + (uint32_t)(g * 64 + h * 32), r);
           if (FORM == kTcPlain) {
             const float nrow = gi < nt * kTcRows ? __ldg(norms + gi) : 0.0f;
-            const float4* nb = reinterpret_cast<const float4*>(norms + (long long)bj * kTcRows + g * 64 + h * 32);
+            const float4* nb = reinterpret_cast<const float4*>(
+                norms + min((long long)cbase, (nt - 1) * kTcRows) + g * 64 + h * 32);
 #pragma unroll
             for (int v = 0; v < 8; ++v) {
               const float4 c4 = __ldg(nb + v);
@@ -554,7 +546,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
           asm volatile("tcgen05.fence::before_thread_sync;");
           __syncwarp();
           if (lane == 0)
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[u]))
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[mt]))
                          : "memory");
         }
         // Candidates go to the warp's shared-memory queue, kept across jobs, and are decided 32 at
@@ -565,7 +557,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             if (!__any_sync(full, !(least[h] > hi_thr))) continue;
-            const unsigned int col0 = (unsigned int)bj * kTcRows + g * 64 + h * 32;
+            const unsigned int col0 = cbase + g * 64 + h * 32;
             // NaN (overflowed tiles) goes to FP64; four chains, for the latency
             uint32_t m0 = 0, m1 = 0, m2 = 0, m3 = 0;
 #pragma unroll
@@ -614,10 +606,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
           }
         }
       }
-      if (++bj == ntile) {
-        ++I;
-        bj = 2 * I;
-      }
+      if (mt == 1 && ++J == nblk) J = ++I;
     }
     if (qn)  // the candidates still queued
       tc_drain(q_i, q_j, q_d, qn, lane, inst, iplan, dtype, tp->lo, sk, EMIT, tl_pairs, tl_rechecks,
@@ -676,7 +665,7 @@ int launch_brute_tc(const BuildArgs& a, bool bf16, Mode mode, unsigned char* til
   TcSink sk{a.row_cnt, a.pair_buf, a.pair_cap, &a.st->emitted, a.symmetric};
   // one CTA per SM (it takes all 512 TMEM columns): more than half of the shared memory
   const size_t smem = kTcSmem > 120 * 1024 ? kTcSmem : 120 * 1024;
-  const long long jobs = tc_jobs(nt);
+  const long long nb = (nt + 1) / 2, jobs = tc_first_job(nb, nb);
   // (more CTAs than that only where a CTA's jobs would not be counted in 31 bits)
   const unsigned grid = (unsigned)std::max<long long>(std::min<long long>(jobs, a.num_sms),
                                                       (jobs + (1LL << 30) - 1) >> 30);
