@@ -1662,6 +1662,7 @@ __device__ __forceinline__ void bitonic_regs(int* v) {
 constexpr int kWarpRowMax = 256;  // rows up to this length are sorted in a warp's registers
 constexpr int kBitmapWords = 4096;   // 16 KB of shared memory per warp at most
 constexpr int kBitmapWarps = 4;      // warps per block of k_rowsort_bitmap
+constexpr int kHeld = 16;            // entries of a row a lane holds in registers there
 constexpr unsigned int kRowDone = 0xffffffffu;  // a queue entry whose row is sorted
 
 // One thread per row: rows of at most 32 entries are sorted in registers (bitonic network
@@ -1869,7 +1870,7 @@ __device__ void block_radix_row(int* row, int* sm, unsigned short* cnt, unsigned
 // counted; a sorted one is marked.  Rows of kSmallCell + 1 .. kWarpRowMax entries are sorted in a
 // warp's registers.  A block per row with the same bitmap spent its time in eight barriers a row:
 // row sort of 100k clustered points in 3-D (2.1e7 pairs) 749 us, of 50k in 9-D (1.3e8) 1283 us;
-// now 376 and 818 us (bound by the 4-byte stores of the columns).
+// now 372 and 707 us.
 __global__ void __launch_bounds__(kBitmapWarps * 32) k_rowsort_bitmap(
     const OutSlot* out, long long n, unsigned int* row_queue, const unsigned int* long_count,
     const unsigned int* mid_count, int per_max, unsigned int* rows_left, unsigned int* errors,
@@ -1883,15 +1884,37 @@ __global__ void __launch_bounds__(kBitmapWarps * 32) k_rowsort_bitmap(
   unsigned int* bm = bitmap + (size_t)wib * 32 * per_max;
   const unsigned int cnt = *long_count;
   const unsigned int warps = gridDim.x * kBitmapWarps;
-  for (unsigned int k = blockIdx.x * kBitmapWarps + wib; k < cnt; k += warps) {
-    const unsigned int row = row_queue[n - 1 - k];
-    const long long b = row_ptr[row], len = row_ptr[row + 1] - b;
+  const unsigned int k0 = blockIdx.x * kBitmapWarps + wib;
+  // the next row's entry and bounds are read while this one is sorted
+  unsigned int next_row = k0 < cnt ? row_queue[n - 1 - (long long)k0] : 0u;
+  long long next_b = row_ptr[next_row], next_e = row_ptr[next_row + 1];
+  for (unsigned int k = k0; k < cnt; k += warps) {
+    const long long b = next_b, len = next_e - next_b;
+    {
+      const unsigned long long kn = (unsigned long long)k + warps;
+      if (kn < cnt) next_row = row_queue[n - 1 - (long long)kn];
+      next_b = row_ptr[next_row];
+      next_e = row_ptr[next_row + 1];
+    }
     if (b + len > col_cap) continue;
     int lo = INT_MAX, hi = -1;
-    for (long long x = lane; x < len; x += 32) {
-      const int v = col[b + x];
-      lo = min(lo, v);
-      hi = max(hi, v);
+    // rows of up to 512 entries are read once, into registers
+    int held[kHeld];
+    if (len <= 32 * kHeld) {
+#pragma unroll
+      for (int q = 0; q < kHeld; ++q) held[q] = q * 32 + lane < len ? col[b + q * 32 + lane] : -1;
+#pragma unroll
+      for (int q = 0; q < kHeld; ++q)
+        if (q * 32 + lane < len) {
+          lo = min(lo, held[q]);
+          hi = max(hi, held[q]);
+        }
+    } else {
+      for (long long x = lane; x < len; x += 32) {
+        const int v = col[b + x];
+        lo = min(lo, v);
+        hi = max(hi, v);
+      }
     }
     lo = __reduce_min_sync(full, lo);
     hi = __reduce_max_sync(full, hi);
@@ -1908,9 +1931,18 @@ __global__ void __launch_bounds__(kBitmapWarps * 32) k_rowsort_bitmap(
     const int P = (int)per;
     for (int w = lane; w < 32 * P; w += 32) bm[w] = 0u;
     __syncwarp();
-    for (long long x = lane; x < len; x += 32) {
-      const int v = col[b + x] - lo;
-      atomicOr(&bm[v >> 5], 1u << (v & 31));
+    if (len <= 32 * kHeld) {
+#pragma unroll
+      for (int q = 0; q < kHeld; ++q)
+        if (q * 32 + lane < len) {
+          const int v = held[q] - lo;
+          atomicOr(&bm[v >> 5], 1u << (v & 31));
+        }
+    } else {
+      for (long long x = lane; x < len; x += 32) {
+        const int v = col[b + x] - lo;
+        atomicOr(&bm[v >> 5], 1u << (v & 31));
+      }
     }
     __syncwarp();
     const unsigned int* mine = bm + lane * P;
@@ -1922,14 +1954,48 @@ __global__ void __launch_bounds__(kBitmapWarps * 32) k_rowsort_bitmap(
       const int z = __shfl_up_sync(full, incl, o);
       if (lane >= o) incl += z;
     }
-    int* dst = col + b + (incl - c);
+    // a lane's columns are consecutive in the row
     const int base = lo + lane * P * 32;
-    for (int w = 0; w < P; ++w) {
-      unsigned int word = mine[w];
-      while (word) {
-        const int bit = __ffs(word) - 1;
-        word &= word - 1;
-        *dst++ = base + w * 32 + bit;
+    if (len < words) {  // few columns a word
+      int* dst = col + b + (incl - c);
+      for (int w = 0; w < P; ++w) {
+        unsigned int word = mine[w];
+        while (word) {
+          const int bit = __ffs(word) - 1;
+          word &= word - 1;
+          *dst++ = base + w * 32 + bit;
+        }
+      }
+    } else {
+      // dense rows: four at a time leave in one 16-byte store (single ones made the L2's store
+      // sectors the bound: 818 against 707 us at 50k points in 9-D)
+      const long long first = b + (incl - c);
+      long long pos = first;
+      int4 four = make_int4(0, 0, 0, 0);
+      auto single = [&](int z) { return z == 0 ? four.x : (z == 1 ? four.y : (z == 2 ? four.z : four.w)); };
+      for (int w = 0; w < P; ++w) {
+        unsigned int word = mine[w];
+        while (word) {
+          const int v = base + w * 32 + __ffs(word) - 1;
+          word &= word - 1;
+          const int z = (int)(pos & 3);
+          four.x = z == 0 ? v : four.x;
+          four.y = z == 1 ? v : four.y;
+          four.z = z == 2 ? v : four.z;
+          four.w = v;
+          if (z == 3) {
+            if (pos - 3 >= first) {
+              *reinterpret_cast<int4*>(col + pos - 3) = four;
+            } else {
+              for (long long x = first; x <= pos; ++x) col[x] = single((int)(x & 3));
+            }
+          }
+          ++pos;
+        }
+      }
+      for (long long x = max(first, pos - (pos & 3)); x < pos; ++x) {
+        const int z = (int)(x & 3);  // (the last one of an unfinished four sits in .w)
+        col[x] = x == pos - 1 ? four.w : single(z);
       }
     }
     if (lane == 0) row_queue[n - 1 - k] = kRowDone;
