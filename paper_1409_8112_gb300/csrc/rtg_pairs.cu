@@ -209,10 +209,13 @@ __device__ __forceinline__ bool decide_pair(unsigned int i, unsigned int j, int 
                                             const float* pb, const K* ki, const K* kj,
                                             const Inst* __restrict__ Ip,
                                             const InstPlan* __restrict__ IPp, float2 band,
-                                            int dtype, Tally& tl, unsigned long long* near_r) {
+                                            int dtype, Tally& tl, unsigned long long* near_r,
+                                            int nv = DPAD / 4) {
+  // nv: the row's 16-byte vectors that hold coordinates (the others are zero)
   float sf = 0.0f;
 #pragma unroll
   for (int v = 0; v < DPAD / 4; ++v) {
+    if (v > 0 && v >= nv) break;
     const float4 x = reinterpret_cast<const float4*>(pa)[v];
     const float4 y = reinterpret_cast<const float4*>(pb)[v];
     float e = x.x - y.x;
@@ -537,6 +540,10 @@ __global__ void __launch_bounds__(kPairThreads, RTG_PAIRS_MIN_BLOCKS) k_pairs_wa
     const int inst_lo = bt_lo / m;
     const bool one_inst = inst_lo == bt_hi / m;
     const float2 span_band = band_of(iplan[inst_lo]);
+    // vectors of a row that hold coordinates: a batch of mixed d is padded to its widest (rows of
+    // 64 bytes for d = 3 next to d = 9: 1054 us of pairs phase for 128 roadmaps of d = 3, 6
+    // and 9 with every vector gathered and compared, 911 with the used ones)
+    const int nv = DPAD > 4 && one_inst ? (inst[inst_lo].d + 3) >> 2 : DPAD / 4;
     const K* kspan = skeys + P0;
     const uint32_t* vspan = svals + P0;
     int P = 0;
@@ -623,7 +630,8 @@ __global__ void __launch_bounds__(kPairThreads, RTG_PAIRS_MIN_BLOCKS) k_pairs_wa
         const float* src = pf + (size_t)vc * DPAD;
         float* dst = w_pt + slot * DPAD;
 #pragma unroll
-        for (int v = 0; v < DPAD / 4; ++v) cp_async16(dst + 4 * v, src + 4 * v);
+        for (int v = 0; v < DPAD / 4; ++v)
+          if (v < nv) cp_async16(dst + 4 * v, src + 4 * v);
         if (STAGE == 2) {
           // 16-byte copies covering the first t keys (key rows and staged rows start on 16-byte
           // boundaries and hold a multiple of 16 bytes, so the copies stay inside both)
@@ -689,7 +697,7 @@ __global__ void __launch_bounds__(kPairThreads, RTG_PAIRS_MIN_BLOCKS) k_pairs_wa
             keep = decide_pair<K, DPAD, MODE, STAGE != 0>(i, j, t, w_pt + sa * DPAD,
                                                           w_pt + sb * DPAD, ka, kb, inst + ib_,
                                                           iplan + ib_, band, dtype, tl,
-                                                          sk.near_r);
+                                                          sk.near_r, nv);
           }
           if (MODE == kBits) {
             deliver_bits(keep, i, j, inst + pinst, sk);
