@@ -322,7 +322,7 @@ def measure_build(ctx, stream, flush, args, pts, T, r, dtype_name, ws, rank, clo
     traffic = ncu_traffic(n, dtype_name, dom, sort_cfg)
     kernels = {"sort": "one k_sort_pass per radix pass (look-back), upsweep + scan + downsweep "
                        "per pass, or one k_sort_coop launch (autotuned variant)",
-               "pairs": "k_pairs_warp + k_pairs_medium + k_large_setup + k_pairs_large"}[dom]
+               "pairs": "k_pairs_warp + k_pairs_tiles + k_large_setup + k_pairs_large"}[dom]
     roofline = {"bound": "hbm", "kernel": dom, "kernels": kernels, "achieved": round(achieved, 1),
                 "peak": peak, "peak_kind": peak_kind, "unit": "GB/s",
                 "frac": round(achieved / peak, 4), "traffic": traffic,
