@@ -247,8 +247,9 @@ rtg_status rtg_batch_all_pairs(rtg_ctx* ctx, const rtg_instance* items, int coun
  * errors as rtg_all_pairs (no transforms).  With count_only != 0 only out->nnz and
  * out->stats.pairs are set (no device memory is returned beyond the row pointers).
  * With RTG_FLAG_TC_FP16 or RTG_FLAG_TC_BF16 the distances come from tensor-core tiles; without
- * either flag FP16 tiles are taken for n >= 4096 where their error bound is below r^2 / 8 (and
- * there is room for them), CUDA cores otherwise; the set is the same.  The tiles' distances
+ * either flag FP16 tiles are taken for n >= 4096 where their error bound is below r^2 / 8 (there
+ * is room for them and the context has no budget), CUDA cores otherwise; the set is the same.
+ * The tiles' distances
  * (|x|^2 + |y|^2 - 2 x.y, x.y as hi.hi + hi.lo + lo.hi of a half-precision split of the
  * centred coordinates, FP32 accumulation); a pair is rejected on the tile only when its d^2
  * exceeds r^2 + band, band = max(1e-3 r^2, proven error bound), and every other pair is

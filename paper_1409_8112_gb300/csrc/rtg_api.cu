@@ -582,7 +582,8 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
       }
     }
     const bool tc = m == 0 && (q.flags & (RTG_FLAG_TC_FP16 | RTG_FLAG_TC_BF16)) != 0;
-    bool tc_auto = m == 0 && !tc && n_total >= kBruteTcMin;
+    // (not under a memory budget, whose room is for the pairs)
+    bool tc_auto = m == 0 && !tc && n_total >= kBruteTcMin && c->budget == 0;
     if (tc || tc_auto) {
       if ((s = ensure(c, c->tc_tiles, rtg::tc_tiles_bytes(n_total))) != RTG_OK ||
           (s = ensure(c, c->tc_norms, (size_t)(n_total + 128) * 4)) != RTG_OK ||

@@ -20,6 +20,7 @@
 
 #include <algorithm>
 #include <cfloat>
+#include <mutex>
 #include <type_traits>
 
 #include "rtg_internal.cuh"
@@ -675,6 +676,7 @@ int launch_brute_tc(const BuildArgs& a, bool bf16, Mode mode, unsigned char* til
     static size_t attr[64] = {};                                                               \
     int dev = 0;                                                                               \
     cudaGetDevice(&dev);                                                                       \
+    std::lock_guard<std::mutex> lk(launch_attr_mutex());                                       \
     if (dev < 0 || dev >= 64 || attr[dev] < smem) {                                            \
       cudaFuncSetAttribute(k_brute_tc<B, E, F>, cudaFuncAttributeMaxDynamicSharedMemorySize,    \
                            (int)smem);                                                         \
