@@ -18,7 +18,7 @@
 //   * j is reported by the first grid that puts it in the query's cell (the dedupe of
 //     Sec. III-B by key rows), so every answer appears once.
 // Indexes of light cells give each (query, grid) a thread, which collects the answers of a query in
-// 32 slots; after the scan of the counts the rows are sorted on their way to their places.  Only
+// 64 slots; after the scan of the counts the rows are sorted on their way to their places.  Only
 // queries with more answers than slots are searched again, one thread per query.  Indexes of
 // dense cells give each query a warp (32 candidates at a time) and search twice: count the
 // answers, scan, write them, then sort each row (the pair path's row sort).
@@ -412,7 +412,8 @@ __global__ void __launch_bounds__(kIndexThreads) k_index_query_thread(
 // row_cnt; st->max_cell receives the largest count.
 // Bound by the latency of its chains (table, run head, members, rows, key rows), which is why
 // the grids of a query are spread over threads: 100,000 queries by one thread each left 21
-// warps per SM and took 187 us to count and as long again to write (query call 424 us, now 218).
+// warps per SM and took 187 us to count and as long again to write (query call with its copy out
+// 485 us, now 293; with 32 slots 274, but one query in 100,000 with more answers cost 70 us).
 template <typename K, int DPAD>
 __global__ void __launch_bounds__(kIndexThreads) k_index_query_lanes(
     const Inst* __restrict__ inst, const InstPlan* __restrict__ iplan,
@@ -801,9 +802,10 @@ rtg_status index_query(rtg_ctx* c, const rtg_index* ix, const void* queries, int
     release_out(c, out);
     return s;
   }
-  // slots for the answers of light cells' queries (without room for them: two searches)
+  // slots for the answers of light cells' queries (two searches without room for them, under a
+  // memory budget, whose room is for the answers, and for more than 2^23 queries: 2 GB)
   int* slots = nullptr;
-  if (ix->thread_queries) {
+  if (ix->thread_queries && c->budget == 0 && nq <= (int64_t(1) << 23)) {
     if (ensure(c, c->q_slots, (size_t)nq * rtg::kRowSlots * sizeof(int)) == RTG_OK) {
       slots = (int*)c->q_slots.p;
     } else {

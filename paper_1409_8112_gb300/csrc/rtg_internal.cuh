@@ -459,7 +459,7 @@ void reset_pairs_state(const BuildArgs& a, cudaStream_t s);
 
 // Rows collected unordered in slots of kRowSlots entries each (row k at slots + k kRowSlots):
 // every row of at most kRowSlots entries goes to its place in the output CSR in ascending order.
-constexpr int kRowSlots = 32;
+constexpr int kRowSlots = 64;
 void launch_rows_from_slots(const OutSlot* out, long long n, const int* slots, cudaStream_t s);
 
 // Guards the per-device caches of kernel attributes (shared-memory limits, occupancy) that

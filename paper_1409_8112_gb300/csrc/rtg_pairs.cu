@@ -1727,48 +1727,6 @@ __global__ void __launch_bounds__(256) k_rowsort_thread(const OutSlot* out, long
   }
 }
 
-// Rows of at most kRowSlots entries from their slots to their places, one thread per row (the
-// register network of k_rowsort_thread between a 16-byte load per four entries and the store).
-__global__ void __launch_bounds__(128) k_rows_from_slots(const OutSlot* out, long long n,
-                                                         const int* __restrict__ slots) {
-  const long long* __restrict__ row_ptr = out->row_ptr;
-  int* col = out->col;
-  const long long row = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (row >= n) return;
-  const long long b = row_ptr[row];
-  const int len = (int)min(row_ptr[row + 1] - b, (long long)kRowSlots + 1);
-  if (len == 0 || len > kRowSlots || b + len > out->col_cap) return;
-  const int4* src = reinterpret_cast<const int4*>(slots + row * kRowSlots);
-  auto load = [&](int* v, int words) {
-#pragma unroll
-    for (int q = 0; q < kRowSlots / 4; ++q)
-      if (q < words) {
-        const int4 x = 4 * q < len ? __ldg(src + q) : make_int4(INT_MAX, INT_MAX, INT_MAX, INT_MAX);
-        v[4 * q] = x.x;
-        v[4 * q + 1] = 4 * q + 1 < len ? x.y : INT_MAX;
-        v[4 * q + 2] = 4 * q + 2 < len ? x.z : INT_MAX;
-        v[4 * q + 3] = 4 * q + 3 < len ? x.w : INT_MAX;
-      }
-  };
-  if (len <= 16) {
-    int v[16];
-    load(v, 4);
-    if (len <= 4) bitonic_regs<4>(v);
-    else if (len <= 8) bitonic_regs<8>(v);
-    else bitonic_regs<16>(v);
-#pragma unroll
-    for (int q = 0; q < 16; ++q)
-      if (q < len) col[b + q] = v[q];
-  } else {
-    int v[32];
-    load(v, 8);
-    bitonic_regs<32>(v);
-#pragma unroll
-    for (int q = 0; q < 32; ++q)
-      if (q < len) col[b + q] = v[q];
-  }
-}
-
 // One row of at most 32 V entries sorted by one warp: lane l holds entries l V .. l V + V - 1
 // in registers (+infinity padding); bitonic network, exchanges across lanes by shuffles.
 template <int V>
@@ -1814,6 +1772,61 @@ __device__ __forceinline__ void warp_sort_row(int* a, int len) {
   for (int q = 0; q < V; ++q) {
     const int e = lane * V + q;
     if (e < len) a[e] = v[q];
+  }
+}
+
+// Rows of at most kRowSlots entries from their slots to their places: up to 32 entries by one
+// thread (the register network of k_rowsort_thread between a 16-byte load per four entries and
+// the store), longer ones by their warp.
+__global__ void __launch_bounds__(128) k_rows_from_slots(const OutSlot* out, long long n,
+                                                         const int* __restrict__ slots) {
+  const long long* __restrict__ row_ptr = out->row_ptr;
+  int* col = out->col;
+  const long long row = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const unsigned int full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const long long b = row < n ? row_ptr[row] : 0;
+  int len = row < n ? (int)min(row_ptr[row + 1] - b, (long long)kRowSlots + 1) : 0;
+  if (len > kRowSlots || b + len > out->col_cap) len = 0;
+  static_assert(kRowSlots == 64, "two entries a lane below");
+  for (unsigned int big = __ballot_sync(full, len > 32); big; big &= big - 1) {
+    const int L = __ffs(big) - 1, l2 = __shfl_sync(full, len, L);
+    const long long b2 = __shfl_sync(full, b, L);
+    const int* from = slots + (row - lane + L) * kRowSlots;
+    col[b2 + lane] = from[lane];
+    if (lane + 32 < l2) col[b2 + 32 + lane] = from[32 + lane];
+    __syncwarp();
+    warp_sort_row<2>(col + b2, l2);
+  }
+  if (len == 0 || len > 32) return;
+  const int4* src = reinterpret_cast<const int4*>(slots + row * kRowSlots);
+  auto load = [&](int* v, int words) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      if (q < words) {
+        const int4 x = 4 * q < len ? __ldg(src + q) : make_int4(INT_MAX, INT_MAX, INT_MAX, INT_MAX);
+        v[4 * q] = x.x;
+        v[4 * q + 1] = 4 * q + 1 < len ? x.y : INT_MAX;
+        v[4 * q + 2] = 4 * q + 2 < len ? x.z : INT_MAX;
+        v[4 * q + 3] = 4 * q + 3 < len ? x.w : INT_MAX;
+      }
+  };
+  if (len <= 16) {
+    int v[16];
+    load(v, 4);
+    if (len <= 4) bitonic_regs<4>(v);
+    else if (len <= 8) bitonic_regs<8>(v);
+    else bitonic_regs<16>(v);
+#pragma unroll
+    for (int q = 0; q < 16; ++q)
+      if (q < len) col[b + q] = v[q];
+  } else {
+    int v[32];
+    load(v, 8);
+    bitonic_regs<32>(v);
+#pragma unroll
+    for (int q = 0; q < 32; ++q)
+      if (q < len) col[b + q] = v[q];
   }
 }
 

@@ -134,22 +134,23 @@ def test_empty_cases_and_errors(ctx):
                                             (9000, 6, 8, 33, np.float64), (3000, 2, 64, 5, np.float32),
                                             (4000, 9, 3, 86, np.float64)])
 def test_more_answers_than_slots(ctx, n, d, m, nq, dtype):
-    # light cells but for one spot of 33 and one of 32 points: queries there have more answers
-    # than are collected in slots, or just as many, next to queries with few and none
+    # light cells but for spots of 65, 64 and 33 points: queries there have more answers than the
+    # 64 that are collected in slots, just as many, or more than one thread sorts, next to
+    # queries with few and none
     rng = np.random.default_rng(n + m)
     pts = rng.random((n, d))
     r = gen.radius_for_degree(n, d, 4.0)
-    spots = np.full(d, 0.5), np.full(d, 3.0)
-    for k, (spot, many) in enumerate(zip(spots, (33, 32))):
+    spots = np.full(d, 0.5), np.full(d, 3.0), np.full(d, -2.0)
+    for k, (spot, many) in enumerate(zip(spots, (65, 64, 33))):
         pts[100 * k:100 * k + many] = spot + rng.normal(0.0, 1e-3 * r, (many, d))
     pts = pts.astype(dtype)
-    q = np.vstack([spots[0], spots[1], rng.random((max(nq - 2, 0), d))])[:nq].astype(dtype)
+    q = np.vstack([*spots, rng.random((max(nq - 3, 0), d))])[:nq].astype(dtype)
     T = gen.transforms(n + m, d, m, r)
     ix = ctx.index(pts, r, T, r)
     for queries in (q, q[::-1].copy()):
         res = ix.query(queries)
         ref = oracle.rtg_query(pts, r, T, r, queries)
         _compare(res, ref)
-        assert np.diff(ref.row_ptr).max() >= 33
+        assert np.diff(ref.row_ptr).max() >= 65
         res.release()
     ix.close()
