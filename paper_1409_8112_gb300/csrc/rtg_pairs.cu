@@ -1626,8 +1626,14 @@ __global__ void __launch_bounds__(256) k_scatter(const unsigned long long* __res
         const bool has = pr[u] != ~0ull;
         const unsigned int row =
             has ? (side == 0 ? (unsigned int)(pr[u] >> 32) : (unsigned int)pr[u]) : 0xffffffffu;
-        const unsigned int peers = __match_any_sync(full, row);
-        const int leader = __ffs(peers) - 1;
+        // neighbouring lanes with the same row form a run (a shuffle and a ballot instead of
+        // __match_any_sync: 1M 77.8 -> 73.7 us, clustered 50k in 9-D 558 -> 533)
+        const unsigned int prev = __shfl_up_sync(full, row, 1);
+        const unsigned int heads = __ballot_sync(full, lane == 0 || row != prev);
+        const int leader = 31 - __clz(heads & (lt | (1u << lane)));
+        const unsigned int later = heads & ~(lt | (1u << lane));
+        const unsigned int peers =
+            (later ? (later & (0u - later)) - 1u : full) & ~((1u << leader) - 1u);
         unsigned int b0 = 0;
         if (has && lane == leader) b0 = atomicAdd(&row_cnt[row], (unsigned int)__popc(peers));
         b0 = __shfl_sync(full, b0, leader);
