@@ -907,6 +907,7 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
     }
     c->guesses[key] = g;
     c->last_sorted = sorted;
+    c->last_key64 = a.key64;
 
     out->n = n_total;
     out->symmetric = sym;

@@ -193,6 +193,9 @@ struct rtg_ctx {
   rtghost::Upload up_inst, up_T;
   rtghost::Server* server = nullptr;  // created by the first rtg_submit
   int last_sorted = 0;  // keys/vals buffer (0 or 1) that holds the last build's sorted keys
+  // Width of the keys the last build left there and in key_mat: the width its shape was guessed
+  // to need, which stays at 64 bits for a while after a build that needed more than 32.
+  bool last_key64 = false;
   // Failure-path hooks (rtg_set_test_hooks): the bounded device waits' iteration limit (0:
   // the default), waits made to wait for something that never happens (rtg::kInject*), and
   // the number of the device allocation that is made to fail (0: none).

@@ -663,7 +663,6 @@ rtg_status index_create(rtg_ctx* c, const rtg_instance& it, int m, int dtype, in
   const Request q{&it, 1, m, dtype, on_device, 0u, true, true};  // grid t at [t n, (t + 1) n)
   rtg_status s = build(c, q, &tmp);
   if (s != RTG_OK) return s;
-  const int key_bits = tmp.stats.key_bits;
   // candidates per sorted position: about how many points share a cell with a query
   const double cand_per_pos =
       it.n > 0 ? (double)tmp.stats.total_candidates / ((double)it.n * m) : 0.0;
@@ -675,7 +674,7 @@ rtg_status index_create(rtg_ctx* c, const rtg_instance& it, int m, int dtype, in
   ix->m = m;
   ix->dtype = dtype;
   ix->dpad = rtg::dpad_for(it.d);
-  ix->key64 = key_bits > 32;
+  ix->key64 = it.n > 0 && c->last_key64;  // (an empty build leaves no keys)
   ix->N = (long long)it.n * m;
   ix->thread_queries = cand_per_pos < 4.0;
   if (it.n == 0) {  // nothing was planned: every query has an empty answer

@@ -154,3 +154,30 @@ def test_more_answers_than_slots(ctx, n, d, m, nq, dtype):
         assert np.diff(ref.row_ptr).max() >= 65
         res.release()
     ix.close()
+
+
+@pytest.mark.parametrize("n,d,m,dtype", [(4000, 6, 8, np.float64), (3001, 5, 7, np.float32)])
+def test_key_width_alternates_between_indexes_of_a_shape(n, d, m, dtype):
+    # small cells need keys of more than 32 bits, wide ones of the same points do not: the grids of
+    # an index are stored in the width its build used, whatever that build's keys needed, also
+    # after the count-only builds of tune_params on the same context
+    pts = gen.points_uniform(31, n, d, dtype)
+    q = _queries(32, pts, 200, d, dtype)
+    bits = set()
+    with rtg.Context(0) as own:
+        def check(r):
+            T = gen.transforms(33, d, m, r)
+            res = own.all_pairs(pts, r, T, r)
+            bits.add(res.stats["key_bits"] > 32)
+            res.release()
+            ix = own.index(pts, r, T, r)
+            res = ix.query(q)
+            _compare(res, oracle.rtg_query(pts, r, T, r, q))
+            res.release()
+            ix.close()
+        small, wide = (0.03, 0.3) if d == 6 else (0.012, 0.2)
+        for r in (small, wide, wide, small, wide, small, wide):
+            check(r)
+        own.tune_params(pts, small, 0.5, seed=1)
+        check(wide)
+    assert bits == {False, True}
