@@ -20,6 +20,7 @@
 
 #include <algorithm>
 #include <cfloat>
+#include <limits>
 #include <mutex>
 #include <type_traits>
 
@@ -181,30 +182,25 @@ __device__ __forceinline__ double exact_dist2(const void* pts, int dtype, long l
   return s;
 }
 
-// A pair the tile did not reject: decided with the FP64 reference sequence (only rejections
-// rely on the error bound); [lo, hi] is where the tile alone could not decide.
-__device__ __forceinline__ void tc_candidate(float d2, long long gi, long long gj, const Inst* Ip,
-                                             const InstPlan* IPp, int dtype, float lo_thr,
-                                          const TcSink& sk, bool emit, unsigned int& pairs,
-                                          unsigned int& rechecks, unsigned int& near_r,
-                                          float& max_err, bool& overflow) {
+// What a warp's candidates add up to in one drain.
+struct TcTally {
+  unsigned int pairs = 0, rechecks = 0, near_r = 0;
+  float max_err = 0.0f;
+};
+
+// Whether a pair the tile did not reject lies within r, by the FP64 reference sequence (only
+// rejections rely on the error bound); [lo, hi] is where the tile alone could not decide.
+__device__ __forceinline__ bool tc_decide(float d2, unsigned int gi, unsigned int gj, const Inst* Ip,
+                                          const InstPlan* IPp, int dtype, float lo_thr,
+                                          TcTally& tl) {
   const Inst& I = *Ip;  // (read where it is used: the epilogue has no registers to spare)
   const double s = exact_dist2(I.pts, dtype, gi, gj, I.d);
-  max_err = fmaxf(max_err, (float)fabs((double)d2 - s));
+  tl.max_err = fmaxf(tl.max_err, (float)fabs((double)d2 - s));
   if (!(d2 < lo_thr)) {  // (every pair within 1e-12 r of r lies in the band: it is 1e-3 r^2 wide)
-    ++rechecks;
-    if (fabs(__dsub_rn(__dsqrt_rn(s), I.r)) <= __dmul_rn(1e-12, I.r)) ++near_r;
+    ++tl.rechecks;
+    if (fabs(__dsub_rn(__dsqrt_rn(s), I.r)) <= __dmul_rn(1e-12, I.r)) ++tl.near_r;
   }
-  if (!(s <= IPp->rr)) return;
-  ++pairs;
-  const unsigned int i = (unsigned int)(I.p0 + gi), j = (unsigned int)(I.p0 + gj);
-  if (emit) {
-    const unsigned long long slot = atomicAdd(sk.emitted, 1ull);
-    if ((long long)slot < sk.pair_cap) sk.pair_buf[slot] = ((unsigned long long)i << 32) | j;
-    else overflow = true;
-  }
-  atomicAdd(&sk.row_cnt[i], 1u);
-  if (sk.symmetric) atomicAdd(&sk.row_cnt[j], 1u);
+  return s <= IPp->rr;
 }
 
 // Candidates queued per warp before their exact check.  A check waits on the points' loads for
@@ -212,22 +208,65 @@ __device__ __forceinline__ void tc_candidate(float d2, long long gi, long long g
 // warps of a CTA then mostly check at the same time (at the end, at 200k points).  The check is
 // inlined: a call makes the compiler keep the accumulators a warp holds in local memory.
 constexpr int kTcQueue = 768;
+static_assert(kTcQueue <= 32 * 32, "a bit per 32 candidates");
 
-// Decides the qn queued candidates of a warp, 32 at a time (one per lane).  Called by all lanes.
+// A CTA's sums.  64 bits: a CTA takes up to 2^30 jobs of 2^16 pairs (1.2 million points with every
+// pair within r pass 2^32 on 152 CTAs).
+using TcCount = unsigned long long;
+constexpr int kTcJobPairs = 256 * 256;
+constexpr long long kTcMaxJobs = 1LL << 30;
+static_assert(std::numeric_limits<TcCount>::max() / kTcJobPairs >= (TcCount)kTcMaxJobs,
+              "a CTA's pairs must be countable");
+struct TcCounts {
+  TcCount pairs, rechecks, near_r;
+  unsigned int max_err;  // float bits
+};
+
+// Decides the qn queued candidates of a warp, 32 at a time (one per lane), delivers the pairs and
+// adds up in cnt (shared memory).  Called by all lanes.
 __device__ __forceinline__ void tc_drain(const unsigned int* q_i, const unsigned int* q_j,
                                          const float* q_d, unsigned int qn, int lane,
                                          const Inst* I, const InstPlan* IP, int dtype,
                                          float lo_thr, const TcSink& sk, bool emit,
-                                         unsigned int& pairs, unsigned int& rechecks,
-                                         unsigned int& near_r, float& max_err, bool& overflow) {
+                                         TcCounts* cnt, unsigned int* errors) {
+  const unsigned int full = 0xffffffffu;
   __syncwarp();
-  for (unsigned int b = 0; b < qn; b += 32) {
-    const unsigned int e = b + lane;
-    if (e < qn)
-      tc_candidate(q_d[e], (long long)q_i[e], (long long)q_j[e], I, IP, dtype, lo_thr, sk, emit,
-                   pairs, rechecks, near_r, max_err, overflow);
+  TcTally tl;
+  const unsigned int p0 = (unsigned int)I->p0;
+  unsigned int kept = 0;  // bit k: this lane's candidate of the k-th 32 is a pair
+  for (unsigned int k = 0; 32 * k < qn; ++k) {
+    const unsigned int e = 32 * k + lane;
+    if (e < qn && tc_decide(q_d[e], q_i[e], q_j[e], I, IP, dtype, lo_thr, tl)) {
+      kept |= 1u << k;
+      atomicAdd(&sk.row_cnt[p0 + q_i[e]], 1u);
+      if (sk.symmetric) atomicAdd(&sk.row_cnt[p0 + q_j[e]], 1u);
+    }
   }
-  __syncwarp();
+  tl.pairs = __reduce_add_sync(full, (unsigned int)__popc(kept));
+  tl.rechecks = __reduce_add_sync(full, tl.rechecks);
+  tl.near_r = __reduce_add_sync(full, tl.near_r);
+  if (emit && tl.pairs) {  // one reservation for the drain
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(sk.emitted, (unsigned long long)tl.pairs);
+    long long slot = (long long)__shfl_sync(full, base, 0);
+    if (lane == 0 && slot + tl.pairs > sk.pair_cap) atomicOr(errors, kErrPairOverflow);
+    for (unsigned int k = 0; 32 * k < qn; ++k) {
+      const unsigned int mask = __ballot_sync(full, (kept >> k) & 1u);
+      const long long at = slot + __popc(mask & ((1u << lane) - 1u));
+      if (((kept >> k) & 1u) && at < sk.pair_cap)
+        sk.pair_buf[at] = ((unsigned long long)(p0 + q_i[32 * k + lane]) << 32) |
+                          (p0 + q_j[32 * k + lane]);
+      slot += __popc(mask);
+    }
+  }
+  const unsigned int err = __reduce_max_sync(full, __float_as_uint(tl.max_err));
+  if (lane == 0) {
+    atomicAdd(&cnt->pairs, (TcCount)tl.pairs);
+    atomicAdd(&cnt->rechecks, (TcCount)tl.rechecks);
+    if (tl.near_r) atomicAdd(&cnt->near_r, (TcCount)tl.near_r);
+    atomicMax(&cnt->max_err, err);
+  }
+  __syncwarp();  // the queue may be filled again
 }
 
 // The smaller of three values, NaN if any is NaN.
@@ -324,8 +363,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
   __shared__ __align__(8) uint64_t b_full[kTcSlots], b_empty[kTcSlots], acc_full[2], acc_empty[2],
       a_full[2], a_empty[2], all_done, b_idle;  // b_idle: test hook, a barrier nothing arrives on
   __shared__ uint32_t tmem_base;
-  __shared__ unsigned int s_cnt[4];
-  __shared__ unsigned int s_err;
+  __shared__ TcCounts s_cnt;
   __shared__ int s_late;  // some wait ran out
   const unsigned int full = 0xffffffffu;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -334,9 +372,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
   const long long jobs = tc_first_job(nb, nb);
   const long long per = (jobs + gridDim.x - 1) / gridDim.x;
   const long long j0 = min(jobs, (long long)blockIdx.x * per), j1 = min(jobs, j0 + per);
-  if (tid < 4) s_cnt[tid] = 0;
   if (tid == 0) {
-    s_err = 0;
+    s_cnt = TcCounts{};
     s_late = 0;
     auto init = [](const uint64_t* bar, int count) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
@@ -494,9 +531,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
     unsigned int* q_j = q_i + kTcQueue;
     float* q_d = reinterpret_cast<float*>(q_j + kTcQueue);
     unsigned int qn = 0;  // entries queued (warp-uniform)
-    unsigned int tl_pairs = 0, tl_rechecks = 0, tl_near = 0;
-    bool overflow = false;
-    float max_err = 0.0f;
     int I = (int)I0, J = (int)J0;
     for (int unit = 0; unit < 2 * count; ++unit) {
       const int q = unit >> 1, mt = unit & 1;
@@ -584,8 +618,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
             bool only = !edge && (hits & (hits - 1u)) == 0u;
             while (who) {
               if (qn + 32u > (unsigned int)kTcQueue) {
-                tc_drain(q_i, q_j, q_d, qn, lane, inst, iplan, dtype, tp->lo, sk, EMIT, tl_pairs,
-                         tl_rechecks, tl_near, max_err, overflow);
+                tc_drain(q_i, q_j, q_d, qn, lane, inst, iplan, dtype, tp->lo, sk, EMIT, &s_cnt,
+                         &st->errors);
                 qn = 0;
               }
               if (hits) {
@@ -610,32 +644,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
       if (mt == 1 && ++J == nblk) J = ++I;
     }
     if (qn)  // the candidates still queued
-      tc_drain(q_i, q_j, q_d, qn, lane, inst, iplan, dtype, tp->lo, sk, EMIT, tl_pairs, tl_rechecks,
-               tl_near, max_err, overflow);
-    // tallies
-    for (int o = 16; o > 0; o >>= 1) {
-      tl_pairs += __shfl_xor_sync(full, tl_pairs, o);
-      tl_rechecks += __shfl_xor_sync(full, tl_rechecks, o);
-      tl_near += __shfl_xor_sync(full, tl_near, o);
-      max_err = fmaxf(max_err, __shfl_xor_sync(full, max_err, o));
-    }
-    if (lane == 0) {
-      atomicAdd(&s_cnt[0], tl_pairs);
-      atomicAdd(&s_cnt[1], tl_rechecks);
-      atomicAdd(&s_cnt[2], tl_near);
-      atomicMax(&s_err, __float_as_uint(max_err));
-    }
-    if (__any_sync(full, overflow) && lane == 0) atomicOr(&st->errors, kErrPairOverflow);
+      tc_drain(q_i, q_j, q_d, qn, lane, inst, iplan, dtype, tp->lo, sk, EMIT, &s_cnt, &st->errors);
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   if (tid == 0) {
     if (s_late) atomicOr(&st->errors, kErrTimeout);
-    if (s_cnt[0]) atomicAdd(&st->pairs, (unsigned long long)s_cnt[0]);
-    if (s_cnt[1]) atomicAdd(&st->dist_rechecks, (unsigned long long)s_cnt[1]);
-    if (s_cnt[2]) atomicAdd(&st->near_r, (unsigned long long)s_cnt[2]);
-    atomicMax(&st->tc_max_err_bits, s_err);
+    if (s_cnt.pairs) atomicAdd(&st->pairs, s_cnt.pairs);
+    if (s_cnt.rechecks) atomicAdd(&st->dist_rechecks, s_cnt.rechecks);
+    if (s_cnt.near_r) atomicAdd(&st->near_r, s_cnt.near_r);
+    atomicMax(&st->tc_max_err_bits, s_cnt.max_err);
   }
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
@@ -669,7 +688,7 @@ int launch_brute_tc(const BuildArgs& a, bool bf16, Mode mode, unsigned char* til
   const long long nb = (nt + 1) / 2, jobs = tc_first_job(nb, nb);
   // (more CTAs than that only where a CTA's jobs would not be counted in 31 bits)
   const unsigned grid = (unsigned)std::max<long long>(std::min<long long>(jobs, a.num_sms),
-                                                      (jobs + (1LL << 30) - 1) >> 30);
+                                                      (jobs + kTcMaxJobs - 1) / kTcMaxJobs);
   const bool emit = mode == kEmit;
 #define RTG_TC_LAUNCH1(B, E, F)                                                                \
   do {                                                                                         \
