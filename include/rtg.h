@@ -119,7 +119,8 @@ typedef struct {
   double phase_us[8];    /* with RTG_FLAG_TIMING: prep+plan, keys, sort, pairs, scan,
                             scatter (or write), rowsort, total (microseconds, device events) */
   double max_abs_err_d2; /* tensor-core brute force: max |tile d^2 - FP64 d^2| over the pairs
-                            the tiles did not reject */
+                            whose FP64 d^2 was taken (with RTG_FLAG_TC_FP16 or RTG_FLAG_TC_BF16
+                            all the tiles did not reject) */
   double band;           /* tensor-core brute force: half-width of the FP64 band around r^2 */
   int64_t phase_bytes[8]; /* device-memory bytes each phase must read and write by its design
                              (the phases of phase_us; [7] is their sum): the points, FP32 rows,
@@ -246,15 +247,16 @@ rtg_status rtg_batch_all_pairs(rtg_ctx* ctx, const rtg_instance* items, int coun
  * recall denominator for Alg. 1 and an exact reference.  Same argument conventions and
  * errors as rtg_all_pairs (no transforms).  With count_only != 0 only out->nnz and
  * out->stats.pairs are set (no device memory is returned beyond the row pointers).
- * With RTG_FLAG_TC_FP16 or RTG_FLAG_TC_BF16 the distances come from tensor-core tiles; without
- * either flag FP16 tiles are taken for n >= 4096 where their error bound is below r^2 / 8 (there
- * is room for them and the context has no budget), CUDA cores otherwise; the set is the same.
- * The tiles' distances
+ * With RTG_FLAG_TC_FP16 or RTG_FLAG_TC_BF16 the distances come from tensor-core tiles
  * (|x|^2 + |y|^2 - 2 x.y, x.y as hi.hi + hi.lo + lo.hi of a half-precision split of the
  * centred coordinates, FP32 accumulation); a pair is rejected on the tile only when its d^2
  * exceeds r^2 + band, band = max(1e-3 r^2, proven error bound), and every other pair is
  * decided with the FP64 sequence, so the set is unchanged.  stats.band and
- * stats.max_abs_err_d2 report the band and the largest observed tile error. */
+ * stats.max_abs_err_d2 report the band and the largest observed tile error.
+ * Without either flag FP16 tiles only leave out pairs that are beyond r for certain, for
+ * n >= 4096 where their band is below r^2 / 8, there is room for them
+ * and the context has no budget; the pairs they leave, or all pairs, are decided by the FP32
+ * filter with FP64 recheck of the CUDA-core kernel, and counted in the same counters. */
 rtg_status rtg_brute_force(rtg_ctx* ctx, const void* points, int dtype, int points_on_device,
                            int64_t n, int d, double r, uint32_t flags, int count_only,
                            rtg_csr* out);

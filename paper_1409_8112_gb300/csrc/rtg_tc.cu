@@ -70,8 +70,13 @@ __global__ void k_tc_plan(const Inst* __restrict__ inst, const unsigned long lon
   //   norms (two sums of d squares) 2 d 2^-24 d M^2
   //   epilogue (two roundings)      3 2^-24 (4 d M^2)
   const double E = fold ? tc_error_bound_folded(M, d, bf16 != 0) : tc_error_bound(M, d, bf16 != 0);
-  const double rr = iplan[0].rr;
-  const double band = fmax(1e-3 * rr, 1.25 * E);
+  const InstPlan IP = iplan[0];
+  const double rr = IP.rr;
+  double band = fmax(1e-3 * rr, 1.25 * E);
+  // Unasked, the pairs the tiles leave are decided as on the CUDA cores, by the FP32 rows first:
+  // every pair that filter would keep (FP32 d^2 <= s_hi, so d^2 <= s_hi + (s_hi - rr)) is left.
+  if (!always && IP.filter_on)
+    band = fmax(band, 2.0 * ((double)IP.s_hi - rr) * (1.0 + 1e-6) + 1.25 * E);
   tp->band = band;
   tp->bound = E;
   // Unasked, the tiles are taken when the FP64 band they need stays below an eighth of r^2 (so
@@ -82,6 +87,25 @@ __global__ void k_tc_plan(const Inst* __restrict__ inst, const unsigned long lon
   if (use) st->tc_band = band;
   tp->lo = __double2float_rd(rr - band);
   tp->hi = __double2float_ru(rr + band);
+}
+
+// FP32 squared distance of two rows, in the order the CUDA-core kernels take it (their padding
+// adds zeros).
+__device__ __forceinline__ float tc_row_dist2(const float* pa, const float* pb, int d) {
+  float s = 0.0f;
+  for (int v = 0; 4 * v < d; ++v) {
+    const float4 x = __ldg(reinterpret_cast<const float4*>(pa) + v);
+    const float4 y = __ldg(reinterpret_cast<const float4*>(pb) + v);
+    float e = x.x - y.x;
+    s = fmaf(e, e, s);
+    e = x.y - y.y;
+    s = fmaf(e, e, s);
+    e = x.z - y.z;
+    s = fmaf(e, e, s);
+    e = x.w - y.w;
+    s = fmaf(e, e, s);
+  }
+  return s;
 }
 
 // What the operand rows hold.  kTcPlain: [hi | lo], 16 halves each.  kTcFold (d <= 12): the
@@ -184,19 +208,31 @@ __device__ __forceinline__ double exact_dist2(const void* pts, int dtype, long l
 
 // What a warp's candidates add up to in one drain.
 struct TcTally {
-  unsigned int pairs = 0, rechecks = 0, near_r = 0;
+  unsigned int pairs = 0, owned = 0, rechecks = 0, near_r = 0;
   float max_err = 0.0f;
 };
 
-// Whether a pair the tile did not reject lies within r, by the FP64 reference sequence (only
-// rejections rely on the error bound); [lo, hi] is where the tile alone could not decide.
+// Whether a pair the tile did not reject lies within r.  With rows (pf; the unasked tiles, where
+// the FP32 filter holds) as the CUDA-core kernel decides it: FP32 outside its band, else the FP64
+// reference sequence.  Without, by the FP64 sequence.  Only rejections rely on the tile's error
+// bound; [lo, hi] is where the tile alone could not decide.
 __device__ __forceinline__ bool tc_decide(float d2, unsigned int gi, unsigned int gj, const Inst* Ip,
                                           const InstPlan* IPp, int dtype, float lo_thr,
-                                          TcTally& tl) {
+                                          const float* pf, int dpad, TcTally& tl) {
   const Inst& I = *Ip;  // (read where it is used: the epilogue has no registers to spare)
+  bool open = !(d2 < lo_thr);  // (with a band 1e-3 r^2 wide, all within 1e-12 r of r are open)
+  if (pf) {
+    const float s = tc_row_dist2(pf + (size_t)gi * dpad, pf + (size_t)gj * dpad, I.d);
+    if (s > IPp->s_hi) return false;
+    ++tl.owned;
+    if (s < IPp->s_lo) return true;
+    open = true;
+  } else {
+    ++tl.owned;
+  }
   const double s = exact_dist2(I.pts, dtype, gi, gj, I.d);
   tl.max_err = fmaxf(tl.max_err, (float)fabs((double)d2 - s));
-  if (!(d2 < lo_thr)) {  // (every pair within 1e-12 r of r lies in the band: it is 1e-3 r^2 wide)
+  if (open) {
     ++tl.rechecks;
     if (fabs(__dsub_rn(__dsqrt_rn(s), I.r)) <= __dmul_rn(1e-12, I.r)) ++tl.near_r;
   }
@@ -218,7 +254,7 @@ constexpr long long kTcMaxJobs = 1LL << 30;
 static_assert(std::numeric_limits<TcCount>::max() / kTcJobPairs >= (TcCount)kTcMaxJobs,
               "a CTA's pairs must be countable");
 struct TcCounts {
-  TcCount pairs, rechecks, near_r;
+  TcCount pairs, owned, rechecks, near_r;
   unsigned int max_err;  // float bits
 };
 
@@ -227,8 +263,9 @@ struct TcCounts {
 __device__ __forceinline__ void tc_drain(const unsigned int* q_i, const unsigned int* q_j,
                                          const float* q_d, unsigned int qn, int lane,
                                          const Inst* I, const InstPlan* IP, int dtype,
-                                         float lo_thr, const TcSink& sk, bool emit,
-                                         TcCounts* cnt, unsigned int* errors) {
+                                         float lo_thr, const float* pf, int dpad,
+                                         const TcSink& sk, bool emit, TcCounts* cnt,
+                                         unsigned int* errors) {
   const unsigned int full = 0xffffffffu;
   __syncwarp();
   TcTally tl;
@@ -236,13 +273,14 @@ __device__ __forceinline__ void tc_drain(const unsigned int* q_i, const unsigned
   unsigned int kept = 0;  // bit k: this lane's candidate of the k-th 32 is a pair
   for (unsigned int k = 0; 32 * k < qn; ++k) {
     const unsigned int e = 32 * k + lane;
-    if (e < qn && tc_decide(q_d[e], q_i[e], q_j[e], I, IP, dtype, lo_thr, tl)) {
+    if (e < qn && tc_decide(q_d[e], q_i[e], q_j[e], I, IP, dtype, lo_thr, pf, dpad, tl)) {
       kept |= 1u << k;
       atomicAdd(&sk.row_cnt[p0 + q_i[e]], 1u);
       if (sk.symmetric) atomicAdd(&sk.row_cnt[p0 + q_j[e]], 1u);
     }
   }
   tl.pairs = __reduce_add_sync(full, (unsigned int)__popc(kept));
+  tl.owned = __reduce_add_sync(full, tl.owned);
   tl.rechecks = __reduce_add_sync(full, tl.rechecks);
   tl.near_r = __reduce_add_sync(full, tl.near_r);
   if (emit && tl.pairs) {  // one reservation for the drain
@@ -262,6 +300,7 @@ __device__ __forceinline__ void tc_drain(const unsigned int* q_i, const unsigned
   const unsigned int err = __reduce_max_sync(full, __float_as_uint(tl.max_err));
   if (lane == 0) {
     atomicAdd(&cnt->pairs, (TcCount)tl.pairs);
+    atomicAdd(&cnt->owned, (TcCount)tl.owned);
     atomicAdd(&cnt->rechecks, (TcCount)tl.rechecks);
     if (tl.near_r) atomicAdd(&cnt->near_r, (TcCount)tl.near_r);
     atomicMax(&cnt->max_err, err);
@@ -355,8 +394,8 @@ template <bool BF16, bool EMIT, int FORM>
 __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
     const unsigned char* __restrict__ tiles, const float* __restrict__ norms,
     const Inst* __restrict__ inst, const InstPlan* __restrict__ iplan,
-    const TcPlan* __restrict__ tp, int dtype, Status* st, TcSink sk, long long nt,
-    unsigned int wait_limit, unsigned int inject) {
+    const TcPlan* __restrict__ tp, int dtype, const float* __restrict__ rows, int dpad, Status* st,
+    TcSink sk, long long nt, unsigned int wait_limit, unsigned int inject) {
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* s_a = smem;                      // row tiles 2 I, 2 I + 1, of two I
   unsigned char* s_b = smem + 4 * kTcTileBytes;   // kTcSlots pairs of column tiles
@@ -531,6 +570,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
     unsigned int* q_j = q_i + kTcQueue;
     float* q_d = reinterpret_cast<float*>(q_j + kTcQueue);
     unsigned int qn = 0;  // entries queued (warp-uniform)
+    // the rows that decide, where the tiles were not asked for and the FP32 filter holds
+    const float* pf = iplan[0].filter_on ? rows : nullptr;
     int I = (int)I0, J = (int)J0;
     for (int unit = 0; unit < 2 * count; ++unit) {
       const int q = unit >> 1, mt = unit & 1;
@@ -618,8 +659,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
             bool only = !edge && (hits & (hits - 1u)) == 0u;
             while (who) {
               if (qn + 32u > (unsigned int)kTcQueue) {
-                tc_drain(q_i, q_j, q_d, qn, lane, inst, iplan, dtype, tp->lo, sk, EMIT, &s_cnt,
-                         &st->errors);
+                tc_drain(q_i, q_j, q_d, qn, lane, inst, iplan, dtype, tp->lo, pf, dpad, sk, EMIT,
+                         &s_cnt, &st->errors);
                 qn = 0;
               }
               if (hits) {
@@ -644,7 +685,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
       if (mt == 1 && ++J == nblk) J = ++I;
     }
     if (qn)  // the candidates still queued
-      tc_drain(q_i, q_j, q_d, qn, lane, inst, iplan, dtype, tp->lo, sk, EMIT, &s_cnt, &st->errors);
+      tc_drain(q_i, q_j, q_d, qn, lane, inst, iplan, dtype, tp->lo, pf, dpad, sk, EMIT, &s_cnt,
+               &st->errors);
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
@@ -652,6 +694,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_brute_tc(
   if (tid == 0) {
     if (s_late) atomicOr(&st->errors, kErrTimeout);
     if (s_cnt.pairs) atomicAdd(&st->pairs, s_cnt.pairs);
+    if (rows && s_cnt.owned) atomicAdd(&st->owned_candidates, s_cnt.owned);
     if (s_cnt.rechecks) atomicAdd(&st->dist_rechecks, s_cnt.rechecks);
     if (s_cnt.near_r) atomicAdd(&st->near_r, s_cnt.near_r);
     atomicMax(&st->tc_max_err_bits, s_cnt.max_err);
@@ -702,7 +745,7 @@ int launch_brute_tc(const BuildArgs& a, bool bf16, Mode mode, unsigned char* til
       if (dev >= 0 && dev < 64) attr[dev] = smem;                                              \
     }                                                                                          \
     k_brute_tc<B, E, F><<<grid, kTcThreads, smem, s>>>(tiles, norms, a.inst, a.iplan, tp,       \
-                                                       a.dtype,                                \
+                                                       a.dtype, always ? nullptr : a.pf, a.dpad, \
                                                     a.st, sk, nt,                              \
                                                     spin_limit_of(a.spin_limit) * kTcWaitScale, \
                                                     a.inject);                                 \

@@ -116,3 +116,34 @@ def test_default_brute_force_by_either_kernel(ctx, n, d, dtype, scale, shift, de
             rp, col = res.download()
             assert np.array_equal(rp, ex.row_ptr) and np.array_equal(col, ex.col)
         res.release()
+
+
+def _cuda_cores():
+    # a context with a memory budget keeps the default brute force to the CUDA cores
+    return rtg.Context(0, 8 << 30)
+
+
+@pytest.mark.parametrize("n,d,dtype,degree", [(4096, 6, np.float64, 20.0), (5001, 9, np.float32, 12.0),
+                                              (4500, 12, np.float64, 12.0), (4300, 16, np.float32, 40.0),
+                                              (4097, 3, np.float32, 300.0), (4096, 0, np.float64, 0.0)])
+def test_default_brute_force_counts_as_on_cuda_cores(ctx, n, d, dtype, degree):
+    # the pairs the tiles leave are decided by the filter of the CUDA-core kernel, so its counters
+    # are the same; the last case is a lattice with many pairs at exactly r
+    if d:
+        pts = gen.points_uniform(60 + d, n, d, dtype)
+        r = gen.radius_for_degree(n, d, degree)
+    else:
+        pts = np.stack(np.meshgrid(*[np.arange(16) / 32.0] * 3), -1).reshape(-1, 3)
+        r = 3.0 / 32.0
+    with _cuda_cores() as plain:
+        for kw in ({}, {"count_only": True}, {"symmetric": True}):
+            a, b = ctx.brute_force(pts, r, **kw), plain.brute_force(pts, r, **kw)
+            assert a.stats["band"] > 0 or (degree > 100.0 and "count_only" in kw)
+            assert b.stats["band"] == 0
+            for key in ("pairs", "owned_candidates", "dist_rechecks", "near_r"):
+                assert a.stats[key] == b.stats[key], key
+            assert a.stats["owned_candidates"] >= a.stats["pairs"] > 0
+            assert d or a.stats["near_r"] > 0
+            a.release()
+            b.release()
+
