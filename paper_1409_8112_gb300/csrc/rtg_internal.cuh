@@ -151,7 +151,6 @@ struct Status {
 
 // Tensor-core brute force: centre of the points, error bound and decision band.
 struct TcPlan {
-  double center[kMaxDim];
   double band, bound;
   float lo, hi;  // FP32 d^2 below hi goes to the FP64 check; lo bounds the band from below
   int use;       // the tiles decide (always when asked for; else when the band is narrow)

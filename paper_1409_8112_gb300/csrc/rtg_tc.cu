@@ -39,6 +39,15 @@ constexpr int kTcTileBytes = kTcRows * kTcK * 2;  // 8 KB per 128-point tile
 constexpr int kTcEpiWarps = 8;
 constexpr int kTcThreads = (kTcEpiWarps + 2) * 32;  // and one that copies tiles, one for the MMAs
 constexpr int kTcSlots = 3;                       // pairs of column tiles in shared memory
+constexpr int kTcPrepThreads = 256;
+constexpr int kTcSample = 16;  // the plan's sample: pairs per thread of a block
+// Unasked, the tiles are taken while no more than this share of the sampled pairs may lie within r
+// (r^2 + band): each costs a check that the epilogue waits for, and on the CUDA cores, which also
+// pay for every reported pair, far less.  30,011 points in 6-D,
+// tiles against CUDA cores: 212 / 1075 us at a share of 0.03%, 1.5 / 6.1 ms at 3%, 3.3 / 9.1 at 10%,
+// 8.5 / 11.2 at 30%, 14.9 / 13.0 at 60%.  Counting only: 188 / 1049 us, 0.86 / 1.10 ms at 3%, 1.13
+// / 1.14 at 5%, 1.79 / 1.24 at 10%.  (16,000 points: 10% 1.0 / 2.7 ms, 60% 4.3 / 3.7.)
+constexpr double kTcShareEmit = 0.4, kTcShareCount = 0.03;
 // MMA completion waits: the context's spin limit times this (a commit takes far longer than
 // one look-back step)
 constexpr unsigned int kTcWaitScale = 16;
@@ -49,20 +58,27 @@ __device__ __forceinline__ double load_coord(const void* pts, int dtype, long lo
                     : (double)__ldg((const float*)pts + i * d + l);
 }
 
-// Band, thresholds and centre for instance 0 (one thread).
-__global__ void k_tc_plan(const Inst* __restrict__ inst, const unsigned long long* bbox,
-                          const InstPlan* __restrict__ iplan, TcPlan* tp, Status* st, int bf16,
-                          int fold, int always) {
+// Centre of the bounding box on axis l, and the half extent.
+__device__ __forceinline__ double tc_center(const unsigned long long* bbox, long long n, int l,
+                                            double* half) {
+  const double hi = n > 0 ? dec_double(bbox[l * 2 + 0]) : 0.0;
+  const double lo = n > 0 ? dec_double(~bbox[l * 2 + 1]) : 0.0;
+  *half = 0.5 * (hi - lo);
+  return 0.5 * (lo + hi);
+}
+
+// Band and thresholds of instance 0 (one thread); whether the error bound lets the tiles be taken.
+__device__ bool tc_plan_band(const Inst* __restrict__ inst, const unsigned long long* bbox,
+                             const InstPlan* __restrict__ iplan, TcPlan* tp, int bf16, int fold,
+                             int always) {
   const Inst I = inst[0];
   const int d = I.d;
   double M = 0.0;
   for (int l = 0; l < d; ++l) {
-    const double hi = I.n > 0 ? dec_double(bbox[l * 2 + 0]) : 0.0;
-    const double lo = I.n > 0 ? dec_double(~bbox[l * 2 + 1]) : 0.0;
-    tp->center[l] = 0.5 * (lo + hi);
-    M = fmax(M, 0.5 * (hi - lo) * (1.0 + 1e-12) + 1e-300);
+    double half;
+    tc_center(bbox, I.n, l, &half);
+    M = fmax(M, half * (1.0 + 1e-12) + 1e-300);
   }
-  for (int l = d; l < kMaxDim; ++l) tp->center[l] = 0.0;
   // Error bound of the FP32 d^2 (absolute), with u16 the unit roundoff of the half type:
   //   centring to FP32             8 sqrt(d) 2^-24 M (2 sqrt(d) M)
   //   hi/lo split + dropped lo.lo  2 d M^2 (2 u16^2 + 2^-22) + 2 d 2^-24 M   (x2 for -2x.y)
@@ -79,14 +95,13 @@ __global__ void k_tc_plan(const Inst* __restrict__ inst, const unsigned long lon
     band = fmax(band, 2.0 * ((double)IP.s_hi - rr) * (1.0 + 1e-6) + 1.25 * E);
   tp->band = band;
   tp->bound = E;
-  // Unasked, the tiles are taken when the FP64 band they need stays below an eighth of r^2 (so
-  // few pairs fall inside it) and nothing overflows a half (coordinates doubled, norms).
-  const double most = bf16 ? 1e30 : 60000.0;
-  const bool use = always || (band <= 0.125 * rr && 2.0 * M < most && (double)d * M * M < most);
-  tp->use = use ? 1 : 0;
-  if (use) st->tc_band = band;
   tp->lo = __double2float_rd(rr - band);
   tp->hi = __double2float_ru(rr + band);
+  // Unasked, the tiles are taken when the band they need stays below an eighth of r^2 (so few
+  // pairs fall inside it) and nothing overflows a half (coordinates doubled, norms).
+  const double most = bf16 ? 1e30 : 60000.0;
+  return always ||
+         (band <= 0.125 * rr && 2.0 * M < most && (double)d * M * M < most);
 }
 
 // FP32 squared distance of two rows, in the order the CUDA-core kernels take it (their padding
@@ -118,13 +133,57 @@ __device__ __forceinline__ float tc_row_dist2(const float* pa, const float* pb, 
 enum TcForm : int { kTcPlain = 0, kTcFold = 1, kTcPacked = 2 };
 inline TcForm tc_form(int d) { return d >= 1 && d <= 9 ? kTcPacked : (d <= 12 ? kTcFold : kTcPlain); }
 
+// The plan's block: band and thresholds, and whether the tiles are taken: always when asked for,
+// else by their error bound and by the share of a sample of the pairs that may lie within r.
+__device__ void tc_plan_block(const Inst* __restrict__ inst, const unsigned long long* bbox,
+                              const InstPlan* __restrict__ iplan, TcPlan* tp, Status* st, int bf16,
+                              int fold, int always, const float* __restrict__ pf, int dpad,
+                              unsigned int most_near) {
+  __shared__ unsigned int s_near;
+  __shared__ bool s_use;
+  const Inst I = inst[0];
+  float s[kTcSample];
+  if (!always) {
+#pragma unroll
+    for (int q = 0; q < kTcSample; ++q) {
+      // the multiples of 1 / p and 1 / p^2, p the plastic number, modulo 1 (a Kronecker sequence):
+      // spread evenly over the index square
+      const unsigned int k = threadIdx.x * kTcSample + q + 1;
+      const long long i = ((long long)(k * 3242174889u) * I.n) >> 32;
+      const long long j = ((long long)(k * 2447445414u) * I.n) >> 32;
+      s[q] = i == j ? FLT_MAX : tc_row_dist2(pf + i * dpad, pf + j * dpad, I.d);
+    }
+  }
+  if (threadIdx.x == 0) {
+    s_near = 0;
+    s_use = tc_plan_band(inst, bbox, iplan, tp, bf16, fold, always);
+  }
+  __syncthreads();
+  if (!always) {
+    const float hi = tp->hi;
+    unsigned int near = 0;
+#pragma unroll
+    for (int q = 0; q < kTcSample; ++q) near += s[q] <= hi ? 1u : 0u;
+    near = __reduce_add_sync(0xffffffffu, near);
+    if ((threadIdx.x & 31) == 0 && near) atomicAdd(&s_near, near);
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    const bool use = s_use && s_near <= most_near;
+    tp->use = use ? 1 : 0;
+    if (use) st->tc_band = tp->band;
+  }
+}
+
 // Half-precision rows in the tile layout, and FP32 norms of the centred points (read by the
-// plain form only).
+// plain form only).  Block 0 makes the plan meanwhile (a launch of its own: 114 us a call for 4096
+// points in 6-D, 109 so).
 template <bool BF16, int FORM>
-__global__ void __launch_bounds__(256) k_tc_prep(const Inst* __restrict__ inst, int dtype,
-                                                 const TcPlan* __restrict__ tp,
-                                                 unsigned char* __restrict__ tiles,
-                                                 float* __restrict__ norms, long long n_pad) {
+__global__ void __launch_bounds__(kTcPrepThreads) k_tc_prep(
+    const Inst* __restrict__ inst, int dtype, const unsigned long long* __restrict__ bbox,
+    const InstPlan* __restrict__ iplan, TcPlan* tp, Status* st, int always,
+    const float* __restrict__ pf, int dpad, unsigned int most_near,
+    unsigned char* __restrict__ tiles, float* __restrict__ norms, long long n_pad) {
   using H = typename std::conditional<BF16, __nv_bfloat16, __half>::type;
   auto to_h = [](float v) -> H {
     if constexpr (BF16) return __float2bfloat16_rn(v); else return __float2half_rn(v);
@@ -132,9 +191,21 @@ __global__ void __launch_bounds__(256) k_tc_prep(const Inst* __restrict__ inst, 
   auto to_f = [](H v) -> float {
     if constexpr (BF16) return __bfloat162float(v); else return __half2float(v);
   };
+  if (blockIdx.x == 0) {
+    tc_plan_block(inst, bbox, iplan, tp, st, BF16 ? 1 : 0, FORM != kTcPlain ? 1 : 0, always, pf,
+                  dpad, most_near);
+    return;
+  }
+  __shared__ double s_center[kMaxDim];
   const Inst I = inst[0];
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= n_pad || !tp->use) return;
+  if (threadIdx.x < kMaxDim) {
+    double half;
+    s_center[threadIdx.x] =
+        (int)threadIdx.x < I.d ? tc_center(bbox, I.n, (int)threadIdx.x, &half) : 0.0;
+  }
+  __syncthreads();
+  const long long i = (blockIdx.x - 1) * (long long)blockDim.x + threadIdx.x;
+  if (i >= n_pad) return;
   const long long ntile = n_pad / kTcRows;
   unsigned char* tile = tiles + (i / kTcRows) * (long long)kTcTileBytes;
   unsigned char* tileB = FORM != kTcPlain ? tile + ntile * (long long)kTcTileBytes : tile;
@@ -146,7 +217,7 @@ __global__ void __launch_bounds__(256) k_tc_prep(const Inst* __restrict__ inst, 
   for (int k = 0; k < width; ++k) {
     float xc = 0.0f;
     if (i < I.n && k < d)
-      xc = __double2float_rn(__dsub_rn(load_coord(I.pts, dtype, i, d, k), tp->center[k]));
+      xc = __double2float_rn(__dsub_rn(load_coord(I.pts, dtype, i, d, k), s_center[k]));
     nrm = fmaf(xc, xc, nrm);
     const H h = to_h(xc);
     const H l = to_h(xc - to_f(h));
@@ -715,16 +786,19 @@ int launch_brute_tc(const BuildArgs& a, bool bf16, Mode mode, unsigned char* til
   const long long nt = (n + kTcRows - 1) / kTcRows;
   const long long n_pad = nt * kTcRows;
   const TcForm form = tc_form(a.d_max);  // (one instance: its d)
-  k_tc_plan<<<1, 1, 0, s>>>(a.inst, a.bbox, a.iplan, tp, a.st, bf16 ? 1 : 0,
-                              form != kTcPlain ? 1 : 0, always ? 1 : 0);
-  const unsigned pblocks = (unsigned)((n_pad + 255) / 256);
+  const unsigned pblocks = (unsigned)((n_pad + kTcPrepThreads - 1) / kTcPrepThreads) + 1;
+  const bool emit = mode == kEmit;
+  const double share = always ? 1.0 : (emit ? kTcShareEmit : kTcShareCount);
   auto prep = bf16 ? (form == kTcPacked ? k_tc_prep<true, kTcPacked>
                                         : (form == kTcFold ? k_tc_prep<true, kTcFold>
                                                            : k_tc_prep<true, kTcPlain>))
                    : (form == kTcPacked ? k_tc_prep<false, kTcPacked>
                                         : (form == kTcFold ? k_tc_prep<false, kTcFold>
                                                            : k_tc_prep<false, kTcPlain>));
-  prep<<<pblocks, 256, 0, s>>>(a.inst, a.dtype, tp, tiles, norms, n_pad);
+  prep<<<pblocks, kTcPrepThreads, 0, s>>>(a.inst, a.dtype, a.bbox, a.iplan, tp, a.st,
+                                          always ? 1 : 0, a.pf, a.dpad,
+                                          (unsigned int)(share * kTcSample * kTcPrepThreads), tiles,
+                                          norms, n_pad);
   TcSink sk{a.row_cnt, a.pair_buf, a.pair_cap, &a.st->emitted, a.symmetric};
   // one CTA per SM (it takes all 512 TMEM columns): more than half of the shared memory
   const size_t smem = kTcSmem > 120 * 1024 ? kTcSmem : 120 * 1024;
@@ -732,7 +806,6 @@ int launch_brute_tc(const BuildArgs& a, bool bf16, Mode mode, unsigned char* til
   // (more CTAs than that only where a CTA's jobs would not be counted in 31 bits)
   const unsigned grid = (unsigned)std::max<long long>(std::min<long long>(jobs, a.num_sms),
                                                       (jobs + kTcMaxJobs - 1) / kTcMaxJobs);
-  const bool emit = mode == kEmit;
 #define RTG_TC_LAUNCH1(B, E, F)                                                                \
   do {                                                                                         \
     static size_t attr[64] = {};                                                               \
@@ -764,7 +837,7 @@ int launch_brute_tc(const BuildArgs& a, bool bf16, Mode mode, unsigned char* til
   }
 #undef RTG_TC_LAUNCH
 #undef RTG_TC_LAUNCH1
-  return grid > 0 ? 3 : 2;
+  return grid > 0 ? 2 : 1;
 }
 
 }  // namespace rtg

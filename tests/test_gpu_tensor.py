@@ -147,3 +147,24 @@ def test_default_brute_force_counts_as_on_cuda_cores(ctx, n, d, dtype, degree):
             a.release()
             b.release()
 
+
+@pytest.mark.parametrize("share,emit_tiles,count_tiles", [(0.002, True, True), (0.2, True, False),
+                                                          (0.6, False, False), (1.0, False, False)])
+def test_default_brute_force_of_dense_graphs(ctx, share, emit_tiles, count_tiles):
+    # many pairs within r: the tiles' candidates would cost more than they save
+    n, d = 4200, 6
+    pts = gen.points_uniform(61, n, d, np.float32)
+    k = np.random.default_rng(62).integers(0, n, (2, 20000))
+    k = k[:, k[0] != k[1]]
+    s = np.sort(((pts[k[0]].astype(np.float64) - pts[k[1]]) ** 2).sum(1))
+    r = float(np.sqrt(s[int(share * (len(s) - 1))])) * (3.0 if share == 1.0 else 1.0)
+    ex = oracle.brute(pts, r)
+    for kw, tiles in (({}, emit_tiles), ({"count_only": True}, count_tiles)):
+        res = ctx.brute_force(pts, r, **kw)
+        assert res.stats["pairs"] == ex.nnz
+        assert (res.stats["band"] > 0) == tiles
+        if not kw:
+            rp, col = res.download()
+            assert np.array_equal(rp, ex.row_ptr) and np.array_equal(col, ex.col)
+        res.release()
+
