@@ -168,3 +168,35 @@ def test_default_brute_force_of_dense_graphs(ctx, share, emit_tiles, count_tiles
             assert np.array_equal(rp, ex.row_ptr) and np.array_equal(col, ex.col)
         res.release()
 
+
+def _tile_error_bound(M, d, bf16):
+    """|tile d^2 - d^2| for coordinates within M of the centre: half-precision hi + lo of the
+    coordinates (and of the norms, for d <= 12) with unit roundoff u, FP32 sums of 48 or 52 terms
+    in any order."""
+    u, u32 = (2.0 ** -8 if bf16 else 2.0 ** -11), 2.0 ** -24
+    e = 16.0 * d * u32 * M * M + 2.0 * (2.0 * d * M * M * (2.0 * u * u + 2.0 ** -22) + d * 2.0 ** -24 * M)
+    if d <= 12:
+        return e + 2.0 * (d * u32 * d * M * M + u * u * d * M * M + 2.0 ** -25) + 2080.0 * u32 * d * M * M
+    return e + 768.0 * u32 * d * M * M + 2.0 * d * u32 * d * M * M + 12.0 * u32 * d * M * M
+
+
+@pytest.mark.parametrize("tensor", ["fp16", "bf16"])
+@pytest.mark.parametrize("d", [1, 2, 4, 5, 6, 9, 10, 12, 13, 16])
+@pytest.mark.parametrize("kind,scale", [("uniform", 1.0), ("corners", 1.0), ("mixed", 1.0),
+                                        ("uniform", 60.0), ("corners", 1e-3)])
+def test_tile_error_of_every_pair_is_within_its_bound(ctx, tensor, d, kind, scale):
+    # rejections rely on the error bound of the tiles.  With every pair within r none is rejected,
+    # and the largest error over all pairs is reported
+    n = 900
+    rng = np.random.default_rng(100 * d + len(kind))
+    pts = rng.uniform(-1.0, 1.0, (n, d))
+    if kind == "corners":  # halves of the same sign, all terms near their largest
+        pts = np.sign(pts) * (1.0 - rng.random((n, d)) * 2.0 ** -9)
+    elif kind == "mixed":  # large and tiny magnitudes next to each other
+        pts *= 2.0 ** -rng.integers(0, 24, (n, d)).astype(np.float64)
+    pts = np.vstack([pts, np.full((1, d), 1.0), np.full((1, d), -1.0)]) * scale
+    r = 4.0 * scale * np.sqrt(d)
+    res = ctx.brute_force(pts, r, tensor=tensor, count_only=True)
+    assert res.stats["pairs"] == (n + 2) * (n + 1) // 2
+    assert res.stats["max_abs_err_d2"] <= _tile_error_bound(scale, d, tensor == "bf16")
+    res.release()
