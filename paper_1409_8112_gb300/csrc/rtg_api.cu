@@ -182,6 +182,31 @@ void release_out(rtg_ctx* c, rtg_csr* csr) {
   std::memset(csr, 0, sizeof(*csr));
 }
 
+// Columns that leave much of their array unused (kColSlack) move to one of their own size; without
+// room for both they stay where they are.
+rtg_status fit_columns(rtg_ctx* c, rtg_csr* out, long long col_cap, long long nnz) {
+  if (!out->col || 2 * nnz >= col_cap || col_cap - nnz <= kColSlack) return RTG_OK;
+  const size_t bytes = sizeof(int32_t) * (size_t)nnz, old = sizeof(int32_t) * (size_t)col_cap;
+  void* p = nullptr;
+  const std::string err = c->err;
+  if (alloc_out(c, bytes, &p) != RTG_OK) {
+    c->err = err;
+    cudaGetLastError();
+    return RTG_OK;
+  }
+  if (p)
+    RTG_CUDA(c, cudaMemcpyAsync(p, out->col, bytes, cudaMemcpyDeviceToDevice, c->stream));
+  RTG_CUDA(c, cudaFreeAsync(out->col, c->stream));
+  out->col = (int32_t*)p;
+  {
+    std::lock_guard<std::mutex> lk(c->live_mu);
+    c->live[out->handle] -= old - bytes;
+    c->out_bytes -= old;  // (alloc_out has counted the new array)
+  }
+  RTG_CUDA(c, cudaStreamSynchronize(c->stream));
+  return RTG_OK;
+}
+
 rtg_status validate_common(int dtype, int64_t n, int d, double r, double c, const void* points) {
   if (dtype != RTG_DTYPE_F64 && dtype != RTG_DTYPE_F32)
     return fail(nullptr, RTG_E_INVALID, "dtype must be RTG_DTYPE_F64 or RTG_DTYPE_F32");
@@ -660,7 +685,7 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
       if ((s = ensure(c, c->pair_buf, (size_t)g.pair_cap * 8)) != RTG_OK) return s;
       a.pair_buf = (unsigned long long*)c->pair_buf.p;
       a.pair_cap = g.pair_cap;
-      const long long ccap = a.pair_cap * (sym ? 2 : 1);
+      const long long ccap = g.col_cap(sym != 0);
       void* cp = nullptr;
       if ((s = alloc_out(c, sizeof(int32_t) * (size_t)ccap, &cp)) != RTG_OK) {
         release_out(c, out);
@@ -731,7 +756,9 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
       // rows, as the two-pass form does, instead of running the whole build again.
       const unsigned int ovf = rtg::kErrPairOverflow | rtg::kErrColOverflow;
       const unsigned int herr = c->h_status->errors;
-      if ((herr & rtg::kErrPairOverflow) && !(herr & ~ovf)) {
+      // An undersized column array alone: the pairs are all there and are scattered again.
+      if ((herr & ovf) && !(herr & ~ovf)) {
+        const bool rewrite = (herr & rtg::kErrPairOverflow) != 0;
         const long long nnz = (long long)c->h_status->nnz;
         const size_t old_bytes = sizeof(int32_t) * (size_t)a.col_cap;
         cudaFreeAsync(out->col, st);
@@ -743,11 +770,13 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
         out->col = nullptr;
         a.col = nullptr;
         a.col_cap = 0;
-        // the pair buffer holds nothing the write pass needs
-        if (c->budget && total_held(c) + sizeof(int32_t) * (size_t)nnz > c->budget)
-          free_buf(c, c->pair_buf);
-        a.pair_buf = nullptr;
-        a.pair_cap = 0;
+        if (rewrite) {
+          // the pair buffer holds nothing the write pass needs
+          if (c->budget && total_held(c) + sizeof(int32_t) * (size_t)nnz > c->budget)
+            free_buf(c, c->pair_buf);
+          a.pair_buf = nullptr;
+          a.pair_cap = 0;
+        }
         void* cp = nullptr;
         if ((s = alloc_out(c, sizeof(int32_t) * (size_t)nnz, &cp)) != RTG_OK) {
           release_out(c, out);
@@ -768,7 +797,7 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
         RTG_CUDA(c, cudaMemsetAsync(&a.st->mid_rows, 0, sizeof(a.st->mid_rows), st));
         RTG_CUDA(c, cudaMemsetAsync(&a.st->rows_left, 0, sizeof(a.st->rows_left), st));
         set_slot();
-        launches += pairs(rtg::kWrite);
+        launches += rewrite ? pairs(rtg::kWrite) : rtg::launch_scatter(a, st);
         if (timing) RTG_CUDA(c, cudaEventRecord(c->ev[6], st));
         launches += rtg::launch_rowsort(a, st);
         if (timing) RTG_CUDA(c, cudaEventRecord(c->ev[7], st));
@@ -881,6 +910,7 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
       if (h.errors & rtg::kErrKeyBits) g.settle_bits((int)h.sort_bits, (int)h.cell_bits, false);
       if (h.errors & rtg::kErrPairOverflow)
         g.pair_cap = (long long)((double)h.emitted * 1.05) + 4096;
+      if (h.errors & rtg::kErrColOverflow) g.settle_cols((long long)h.emitted);
       continue;
     }
     if ((s = check_errors(c, ~0u)) != RTG_OK) {
@@ -889,7 +919,14 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
     }
     // remember the launch decisions for the next build of this shape
     if (m > 0) g.settle_bits((int)h.sort_bits, (int)h.cell_bits, !known);
-    if (!two_pass) g.settle_pairs((long long)h.emitted);
+    if (!two_pass) {
+      g.settle_pairs((long long)h.emitted);
+      g.settle_cols((long long)h.emitted);
+      if (known && (s = fit_columns(c, out, a.col_cap, (long long)h.nnz)) != RTG_OK) {
+        release_out(c, out);
+        return s;
+      }
+    }
     if (m > 0 && !bitset) {
       // with a margin, so that new data of the same shape seldom brings such work back
       g.settle_skip(0, h.max_cell <= (unsigned long long)rtg::kSkipMargin);  // kSkipDense

@@ -94,7 +94,33 @@ struct ShapeGuess {
       pair_cap = (e + e / 4 + 4096 + 4095) / 4096 * 4096;
   }
   long long last_pairs = -1;  // pairs of the shape's last build (-1: none)
+  // A result keeps its column array, so that one follows the pairs and not the pair buffer: room
+  // for the most pairs of the shape's recent builds (kCalmBuilds of less than half in a row bring
+  // it down), of one size while they differ little, which suits the pool.  The kernels read it
+  // from the output slot, so that a change does not change the launch sequence.
+  long long col_pairs = -1, sparse_most = 0;
+  int sparse = 0;
+  void settle_cols(long long e) {
+    sparse_most = std::max(sparse_most, e);
+    if (e > col_pairs + col_pairs / 32 || (2 * e < col_pairs && ++sparse >= kCalmBuilds)) {
+      col_pairs = sparse_most;
+    } else if (2 * e < col_pairs) {
+      return;
+    }
+    sparse = 0;
+    sparse_most = 0;
+  }
+  long long col_cap(bool sym) const {
+    const long long c = col_pairs < 0 ? pair_cap : std::min(pair_cap, tight_pairs(col_pairs));
+    return c * (sym ? 2 : 1);
+  }
 };
+
+// A result whose columns fill less than half of their array, and leave more than this many entries
+// of it unused, is copied to an array of its own size (but for a shape's first).  With four
+// fifths for the half, three clustered 50k sets in 9-D in turn took 3407 us a build instead of
+// 3262: one of them was copied, 0.4 GB.
+constexpr long long kColSlack = 1 << 16;
 
 // A build's launch sequence captured once and replayed for later builds of the same shape.
 struct GraphEntry {

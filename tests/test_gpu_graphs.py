@@ -134,3 +134,58 @@ def test_inputs_that_alternate_settle():
         assert np.array_equal(rp, refs[which].row_ptr) and np.array_equal(col, refs[which].col), k
         assert k < 4 or st["attempts"] == 1, (k, st["attempts"])
     ctx.close()
+
+
+@pytest.mark.parametrize("symmetric", [False, True])
+def test_more_columns_than_recent_builds(symmetric):
+    # the pairs fit the shape's pair buffer (16 a point at first) but not the column array, which
+    # follows the pairs of recent builds: they are scattered again
+    n, d, m, r = 6000, 3, 4, 0.05
+    T = gen.transforms(63, d, m, r)
+    few = gen.points_uniform(63, n, d)
+    more = gen.points_uniform(64, n, d) * 0.7  # (no dense cells or long rows either)
+    refs = {id(p): oracle.rtg(p, r, T, r).csr for p in (few, more)}
+    assert 2 * refs[id(few)].nnz + 4096 < refs[id(more)].nnz < 16 * n
+    with rtg.Context(0) as ctx:
+        for k, pts in enumerate((few, few, few, more, more, few, more)):
+            res = ctx.all_pairs(pts, r, T, r, symmetric=symmetric)
+            st, (rp, col) = res.stats, res.download()
+            res.release()
+            ref = refs[id(pts)]
+            if symmetric:
+                i = np.repeat(np.arange(n), np.diff(rp))
+                assert len(col) == 2 * ref.nnz
+                assert np.array_equal(np.sort(i * n + col), np.sort(col * np.int64(n) + i))
+                up = i < col
+                rp, col = np.concatenate([[0], np.cumsum(np.bincount(i[up], minlength=n))]), col[up]
+            assert np.array_equal(rp, ref.row_ptr) and np.array_equal(col, ref.col), k
+            assert st["attempts"] == (2 if k == 3 else 1), k
+
+
+def test_stored_results_hold_the_memory_of_their_pairs():
+    # results kept after a much denser input of their shape: each holds its own columns (as much
+    # again and 256 KB at most) and not the capacity the dense one needed
+    import torch
+    n, d, m, r = 20000, 3, 4, 0.05
+    T = gen.transforms(65, d, m, r)
+    few = gen.points_uniform(65, n, d)
+    dense = gen.points_mixture(66, n, d, k=8, sigma=0.06, dtype=np.float64)
+    with rtg.Context(0) as ctx:
+        for pts in (few, dense, dense):
+            res = ctx.all_pairs(pts, r, T, r)
+            pairs = res.nnz
+            res.release()
+        assert 500000 < pairs < 1200000
+        ref = oracle.rtg(few, r, T, r).csr
+        ctx.all_pairs(few, r, T, r).release()
+        before = torch.cuda.mem_get_info()[0]
+        kept = [ctx.all_pairs(few, r, T, r) for _ in range(100)]
+        held = before - torch.cuda.mem_get_info()[0]
+        for res in (kept[0], kept[50], kept[99]):
+            rp, col = res.download()
+            assert np.array_equal(rp, ref.row_ptr) and np.array_equal(col, ref.col)
+        each = 2 * 4 * ref.nnz + (4 << 16) + 8 * (n + 1)
+        # and room for one build's full capacity, and the pool's rounding
+        assert held <= 100 * each + 8 * pairs + (64 << 20), (held, each)
+        for res in kept:
+            res.release()
