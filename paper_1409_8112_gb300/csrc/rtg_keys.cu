@@ -12,7 +12,7 @@
 // chain's own error is below 2^-29 of that).  When [u - E, u + E] holds no integer the FP32
 // floor is exact; otherwise the coordinate is recomputed with the FP64 sequence.  E is widened
 // by 3e-12 / c so every coordinate within 1e-12 of a wall takes the FP64 path, where it is
-// counted.
+// counted, and by what roundings to subnormal numbers may add (plan_axis_item).
 //
 // The floor takes no conversion instruction (a quarter of a warp's issue rate or less): for
 // |u| < 2^22 the sum u + 1.5 2^23, rounded down, is 1.5 2^23 + floor(u) exactly, its low bits
@@ -254,7 +254,7 @@ __device__ void plan_axis_item(long long idx, const Inst* __restrict__ inst, int
   }
   const double* R = T64 + I.T0 + (size_t)t * (d * d + d);
   const double* s = R + d * d;
-  double ymin = s[k], ymax = s[k], A = fabs(s[k]);
+  double ymin = s[k], ymax = s[k], A = fabs(s[k]), sum_p = 1.0, sum_R = 0.0;
 #pragma unroll 3  // the loads of a few axes in flight together
   for (int l = 0; l < d; ++l) {
     const double hi = I.n > 0 ? dec_double(__ldcg(bbox + ((size_t)b * kMaxDim + l) * 2 + 0)) : 0.0;
@@ -264,6 +264,8 @@ __device__ void plan_axis_item(long long idx, const Inst* __restrict__ inst, int
     ymin += fmin(a, bb);
     ymax += fmax(a, bb);
     A += fabs(rkl) * fmax(fabs(lo), fabs(hi));
+    sum_p += fmax(fabs(lo), fabs(hi));
+    sum_R += fabs(rkl);
     G.Rf[k * kMaxDim + l] = __double2float_rn(rkl);
   }
   for (int l = d; l < kMaxDim; ++l) G.Rf[k * kMaxDim + l] = 0.0f;
@@ -281,7 +283,10 @@ __device__ void plan_axis_item(long long idx, const Inst* __restrict__ inst, int
     G.qlo[k] = (long long)qmin;
     G.ext[k] = (unsigned long long)((long long)qmax - (long long)qmin + 1);
   }
-  const double E = ((double)(d + 6) * 0x1.0p-24 * A + 3e-12) * I.inv_c * (1.0 + 1e-6);
+  // Roundings to a subnormal FP32 (of R, s, p, 1 / c, R / c or s / c) are off by up to 2^-150
+  // instead of 2^-24 of the value: nothing next to the first term unless magnitudes are extreme.
+  const double E = ((double)(d + 6) * 0x1.0p-24 * A + 3e-12) * I.inv_c * (1.0 + 1e-6) +
+                   0x1.0p-149 * (sum_p * (1.0 + I.inv_c) + sum_R * I.inv_c + A);
   G.E[k] = __double2float_ru(E);
 }
 

@@ -133,3 +133,33 @@ def test_fp64_coordinates_beyond_the_fp32_range_are_decided_in_fp64():
     assert np.array_equal(rp, ref.row_ptr)
     assert np.array_equal(col, ref.col)
     assert st["key_rechecks"] > 0 and st["dist_rechecks"] > 0
+
+
+def subnormal_scaled_rotation(n=400, d=8, m=3):
+    """Points, radius, transforms and cell side with R / c below the smallest normal FP32 number:
+    the first axis is near zero for all points (its terms cancel), on either side of the cell wall
+    there, and the roundings of R / c (multiples of 2^-149) add up over its terms."""
+    c = 2.0 ** 120
+    rng = np.random.default_rng(17)
+    sign = np.where(np.arange(d) % 2 == 0, 1.0, -1.0)
+    T = np.zeros((m, d * d + d))
+    for t in range(m):
+        T[t, :d] = 2.0 ** -29 * (512.0 + 3 * np.arange(d) + 7 * t + 0.5 + 0.04 * sign)
+    big = 2.0 ** 127 * rng.uniform(0.6, 0.9, (n, d)) * sign
+    y = big @ T[0, :d]
+    big[:, -1] -= (y - 2.0 ** 120 * rng.normal(0.0, 4e-7, n)) / T[0, d - 1]
+    return big, 2.0 ** 129, T, c
+
+
+def test_cells_whose_scaled_rotation_is_subnormal():
+    # the FP32 cell index is off by far more than its relative error bound: every such coordinate
+    # has to be decided in FP64
+    pts, r, T, c = subnormal_scaled_rotation()
+    ref = oracle.rtg(pts, r, T, c).csr
+    assert 0 < ref.nnz < len(pts) * (len(pts) - 1) // 2
+    with rtg.Context(0) as ctx:
+        res = ctx.all_pairs(pts, r, T, c)
+        rp, col = res.download()
+        res.release()
+    assert np.array_equal(rp, ref.row_ptr)
+    assert np.array_equal(col, ref.col)
