@@ -189,3 +189,23 @@ def test_stored_results_hold_the_memory_of_their_pairs():
         assert held <= 100 * each + 8 * pairs + (64 << 20), (held, each)
         for res in kept:
             res.release()
+
+
+def test_key_width_settles():
+    # keys wider than 32 bits once: the shape's builds keep that width while narrower keys come, give
+    # it up after a number of them, and take it again, each with the oracle's pairs
+    n, d, m = 3000, 6, 5
+    pts = gen.points_uniform(67, n, d)
+    small, wide = 0.03, 0.3
+    grids = {r: gen.transforms(67, d, m, r) for r in (small, wide)}
+    refs = {r: oracle.rtg(pts, r, grids[r], r).csr for r in grids}
+    passes = []
+    with rtg.Context(0) as ctx:
+        for r in (small, small, *[wide] * 20, small, small):
+            res = ctx.all_pairs(pts, r, grids[r], r)
+            st, (rp, col) = res.stats, res.download()
+            res.release()
+            assert np.array_equal(rp, refs[r].row_ptr) and np.array_equal(col, refs[r].col)
+            assert (st["key_bits"] > 32) == (r == small)
+            passes.append(st["sort_passes"])
+    assert passes[2] == passes[1] > passes[21] and passes[22] == passes[23] == passes[1], passes
