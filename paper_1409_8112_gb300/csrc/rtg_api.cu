@@ -76,6 +76,30 @@ bool injected_alloc_failure(rtg_ctx* c) {
   return c->fail_alloc_at > 0 && ++c->alloc_calls == c->fail_alloc_at;
 }
 
+void free_buf(rtg_ctx* c, DevBuf& b) {
+  if (b.p) cudaFree(b.p);
+  c->ws_bytes -= b.cap;
+  b = DevBuf();
+}
+
+// Frees the scratch that only makes calls faster, where the running call does not use it: the
+// answer slots of index queries and the operand tiles of the brute force.  True if there was any:
+// an allocation that failed is then tried again, so that what a context keeps of it refuses no
+// call.
+bool give_back(rtg_ctx* c) {
+  bool any = false;
+  auto drop = [&](DevBuf& b) {
+    any |= b.cap > 0;
+    free_buf(c, b);
+  };
+  if (!c->slots_in_use) drop(c->q_slots);
+  if (!c->tiles_in_use) {
+    drop(c->tc_tiles);
+    drop(c->tc_norms);
+  }
+  return any;
+}
+
 // Grow a workspace buffer to at least `bytes` (contents are not kept).
 rtg_status ensure(rtg_ctx* c, DevBuf& b, size_t bytes, bool zero) {
   if (bytes == 0) bytes = 16;
@@ -85,7 +109,7 @@ rtg_status ensure(rtg_ctx* c, DevBuf& b, size_t bytes, bool zero) {
   if (c->budget && total_held(c) - b.cap + bytes > c->budget)
     return fail(c, RTG_E_BUDGET, "workspace of " + std::to_string(bytes) +
                                      " bytes exceeds the memory budget");
-  if (injected_alloc_failure(c))
+  if (injected_alloc_failure(c) && !give_back(c))
     return fail(c, RTG_E_NOMEM, "device allocation failed (injected by rtg_set_test_hooks)");
   if (b.p) {
     cudaStreamSynchronize(c->stream);
@@ -94,18 +118,22 @@ rtg_status ensure(rtg_ctx* c, DevBuf& b, size_t bytes, bool zero) {
     b.p = nullptr;
     b.cap = 0;
   }
-  RTG_CUDA(c, cudaMalloc(&b.p, bytes));
+  cudaError_t e = cudaMalloc(&b.p, bytes);
+  if (e == cudaErrorMemoryAllocation && give_back(c)) {
+    cudaGetLastError();
+    e = cudaMalloc(&b.p, bytes);
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    b.p = nullptr;
+    return fail(c, e == cudaErrorMemoryAllocation ? RTG_E_NOMEM : RTG_E_CUDA,
+                std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  }
   b.cap = bytes;
   b.gen = ++c->alloc_gen;
   c->ws_bytes += bytes;
   if (zero) RTG_CUDA(c, cudaMemsetAsync(b.p, 0, bytes, c->stream));
   return RTG_OK;
-}
-
-void free_buf(rtg_ctx* c, DevBuf& b) {
-  if (b.p) cudaFree(b.p);
-  c->ws_bytes -= b.cap;
-  b = DevBuf();
 }
 
 rtg_status alloc_out_on(rtg_ctx* c, cudaStream_t s, size_t bytes, void** p) {
@@ -132,8 +160,15 @@ rtg_status alloc_out_on(rtg_ctx* c, cudaStream_t s, size_t bytes, void** p) {
   return RTG_OK;
 }
 
+// (the caller holds c->mu, or the context is its own)
 rtg_status alloc_out(rtg_ctx* c, size_t bytes, void** p) {
-  return alloc_out_on(c, c->stream, bytes, p);
+  rtg_status s = alloc_out_on(c, c->stream, bytes, p);
+  if (s == RTG_E_NOMEM && give_back(c)) {
+    c->err.clear();
+    cudaGetLastError();
+    s = alloc_out_on(c, c->stream, bytes, p);
+  }
+  return s;
 }
 
 // Register `bytes` (already counted in out_bytes) under a new CSR handle.
@@ -189,7 +224,7 @@ rtg_status fit_columns(rtg_ctx* c, rtg_csr* out, long long col_cap, long long nn
   const size_t bytes = sizeof(int32_t) * (size_t)nnz, old = sizeof(int32_t) * (size_t)col_cap;
   void* p = nullptr;
   const std::string err = c->err;
-  if (alloc_out(c, bytes, &p) != RTG_OK) {
+  if (alloc_out_on(c, c->stream, bytes, &p) != RTG_OK) {
     c->err = err;
     cudaGetLastError();
     return RTG_OK;
@@ -201,7 +236,7 @@ rtg_status fit_columns(rtg_ctx* c, rtg_csr* out, long long col_cap, long long nn
   {
     std::lock_guard<std::mutex> lk(c->live_mu);
     c->live[out->handle] -= old - bytes;
-    c->out_bytes -= old;  // (alloc_out has counted the new array)
+    c->out_bytes -= old;  // (alloc_out_on has counted the new array)
   }
   RTG_CUDA(c, cudaStreamSynchronize(c->stream));
   return RTG_OK;
@@ -298,6 +333,10 @@ rtg_status graph_for(rtg_ctx* c, const ShapeKey& key, const rtg::BuildArgs& a, b
 
 rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
   cudaStream_t st = c->stream;
+  struct Use {
+    rtg_ctx* c;
+    ~Use() { c->tiles_in_use = false; }
+  } use{c};
   c->ws_need = 0;
   const bool timing = (q.flags & RTG_FLAG_TIMING) != 0;
   const int sym = (q.flags & RTG_FLAG_SYMMETRIC) ? 1 : 0;
@@ -609,17 +648,29 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
     const bool tc = m == 0 && (q.flags & (RTG_FLAG_TC_FP16 | RTG_FLAG_TC_BF16)) != 0;
     // (not under a memory budget, whose room is for the pairs)
     bool tc_auto = m == 0 && !tc && n_total >= kBruteTcMin && c->budget == 0;
-    if (tc || tc_auto) {
-      if ((s = ensure(c, c->tc_tiles, rtg::tc_tiles_bytes(n_total))) != RTG_OK ||
-          (s = ensure(c, c->tc_norms, (size_t)(n_total + 128) * 4)) != RTG_OK ||
-          (s = ensure(c, c->tc_plan, sizeof(rtg::TcPlan))) != RTG_OK) {
-        if (tc) return s;
-        tc_auto = false;  // no room for the tiles: the CUDA-core kernel needs none
+    c->tiles_in_use = tc;
+    auto tile_room = [&]() -> rtg_status {
+      rtg_status e;
+      if ((e = ensure(c, c->tc_tiles, rtg::tc_tiles_bytes(n_total))) != RTG_OK ||
+          (e = ensure(c, c->tc_norms, (size_t)(n_total + 128) * 4)) != RTG_OK ||
+          (e = ensure(c, c->tc_plan, sizeof(rtg::TcPlan))) != RTG_OK)
+        return e;
+      return RTG_OK;
+    };
+    if (tc && (s = tile_room()) != RTG_OK) return s;
+    // the tiles nobody asked for come last, once the call has all it needs: without room for them
+    // the CUDA-core kernel, which needs none, takes every pair
+    auto optional_tiles = [&]() {
+      if (!tc_auto) return;
+      c->tiles_in_use = true;
+      if (tile_room() != RTG_OK) {
+        tc_auto = c->tiles_in_use = false;
         c->err.clear();
         cudaGetLastError();
       }
-    }
-    a.tc_auto = tc_auto ? (const rtg::TcPlan*)c->tc_plan.p : nullptr;
+      a.tc_auto = tc_auto ? (const rtg::TcPlan*)c->tc_plan.p : nullptr;
+    };
+    a.tc_auto = nullptr;
     // (known without running the sort: a replayed graph launches no kernel from here, and a
     // second enumeration after it reads the sorted keys)
     const int sorted = rtg::sorted_buffer(a);
@@ -698,6 +749,7 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
       }
       a.col = (int*)cp;
       a.col_cap = ccap;
+      optional_tiles();
       c->h_slot->row_ptr = a.row_ptr;
       c->h_slot->col = a.col;
       c->h_slot->col_cap = a.col_cap;
@@ -754,6 +806,7 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
       // build): every pair was still counted in its row and the scan has placed the rows, so
       // only the columns are missing.  A second enumeration writes them straight into their
       // rows, as the two-pass form does, instead of running the whole build again.
+      c->tiles_in_use = false;  // (columns are written without them)
       const unsigned int ovf = rtg::kErrPairOverflow | rtg::kErrColOverflow;
       const unsigned int herr = c->h_status->errors;
       // An undersized column array alone: the pairs are all there and are scattered again.
@@ -854,6 +907,7 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
       c->h_status->pairs = c->h_status->nnz / (sym ? 2 : 1);
       c->h_status->owned_candidates = 0;
     } else {
+      optional_tiles();
       set_slot();
       launches += front();
       launches += pairs(rtg::kCount);
@@ -866,6 +920,7 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
         release_out(c, out);
         return s;
       }
+      c->tiles_in_use = false;  // (columns are written without them)
       if (!(c->h_status->errors & rtg::kErrKeyBits) && !q.count_only && c->h_status->nnz > 0) {
         const long long nnz = (long long)c->h_status->nnz;
         void* cp = nullptr;

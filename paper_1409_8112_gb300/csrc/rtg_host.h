@@ -193,6 +193,8 @@ struct rtg_ctx {
   // the output-slot copy runs on a second stream beside the front of the build
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  // the optional scratch the running call uses (give_back leaves it)
+  bool slots_in_use = false, tiles_in_use = false;
   size_t ws_bytes = 0;
   size_t ws_need = 0;  // workspace bytes the current build asked for (at most ws_bytes)
   size_t out_bytes = 0;
@@ -276,6 +278,9 @@ size_t sort_scratch_bytes_max(long long N);
 void tune_load(rtg_ctx* c);
 
 // Workspace and status helpers (rtg_api.cu).
+void free_buf(rtg_ctx* c, DevBuf& b);
+// alloc_out_on(c, c->stream, ...), tried again without the optional scratch.  The caller holds c->mu.
+rtg_status alloc_out(rtg_ctx* c, size_t bytes, void** p);
 rtg_status ensure(rtg_ctx* c, DevBuf& b, size_t bytes, bool zero = false);
 rtg_status read_status(rtg_ctx* c);
 rtg_status check_errors(rtg_ctx* c, unsigned int mask);

@@ -693,7 +693,7 @@ rtg_status index_create(rtg_ctx* c, const rtg_instance& it, int m, int dtype, in
   ix->table_cap = cap;
   const size_t b_tab = align256(sizeof(unsigned long long) * (size_t)cap * m);
   const size_t total = b_pts + b_pf + b_kr + b_sk + b_sv + b_inst + b_ip + b_gp + b_T + b_tab;
-  if ((s = alloc_out_on(c, c->stream, total, &ix->mem)) != RTG_OK) {
+  if ((s = alloc_out(c, total, &ix->mem)) != RTG_OK) {
     delete ix;
     return s;
   }
@@ -780,7 +780,7 @@ rtg_status index_query(rtg_ctx* c, const rtg_index* ix, const void* queries, int
   if (ix->owner != c) return fail(c, RTG_E_INVALID, "the index belongs to another context");
   rtg_status s;
   void* rp = nullptr;
-  if ((s = alloc_out_on(c, st, sizeof(int64_t) * (size_t)(nq + 1), &rp)) != RTG_OK) return s;
+  if ((s = alloc_out(c, sizeof(int64_t) * (size_t)(nq + 1), &rp)) != RTG_OK) return s;
   out->row_ptr = (int64_t*)rp;
   out->handle = register_out(c, sizeof(int64_t) * (size_t)(nq + 1));
   out->n = nq;
@@ -804,9 +804,14 @@ rtg_status index_query(rtg_ctx* c, const rtg_index* ix, const void* queries, int
   // slots for the answers of light cells' queries (two searches without room for them, under a
   // memory budget, whose room is for the answers, and for more than 2^23 queries: 2 GB)
   int* slots = nullptr;
+  struct Use {  // (give_back leaves the slots while this call reads them)
+    rtg_ctx* c;
+    ~Use() { c->slots_in_use = false; }
+  } use{c};
   if (ix->thread_queries && c->budget == 0 && nq <= (int64_t(1) << 23)) {
     if (ensure(c, c->q_slots, (size_t)nq * rtg::kRowSlots * sizeof(int)) == RTG_OK) {
       slots = (int*)c->q_slots.p;
+      c->slots_in_use = true;
     } else {
       c->err.clear();
       cudaGetLastError();
@@ -853,7 +858,14 @@ rtg_status index_query(rtg_ctx* c, const rtg_index* ix, const void* queries, int
   const long long nnz = (long long)c->h_status->nnz;
   if (nnz > 0) {
     void* cp = nullptr;
-    if ((s = alloc_out_on(c, st, sizeof(int32_t) * (size_t)nnz, &cp)) != RTG_OK) {
+    s = alloc_out(c, sizeof(int32_t) * (size_t)nnz, &cp);
+    if (s == RTG_E_NOMEM && slots) {  // the answers have the slots' room and are searched again
+      slots = nullptr;
+      c->slots_in_use = false;
+      c->err.clear();
+      s = alloc_out(c, sizeof(int32_t) * (size_t)nnz, &cp);
+    }
+    if (s != RTG_OK) {
       release_out(c, out);
       return s;
     }

@@ -64,7 +64,7 @@ rtg_status query_neighbors(rtg_ctx* c, const rtg_csr* g, const int32_t* queries,
                 std::string(what) + ": " + cudaGetErrorString(e));
   };
   void* rp = nullptr;
-  if ((s = alloc_out_on(c, st, sizeof(int64_t) * (size_t)(nq + 1), &rp)) != RTG_OK) return s;
+  if ((s = alloc_out(c, sizeof(int64_t) * (size_t)(nq + 1), &rp)) != RTG_OK) return s;
   out->row_ptr = (int64_t*)rp;
   out->handle = register_out(c, sizeof(int64_t) * (size_t)(nq + 1));
   out->n = nq;
@@ -127,7 +127,7 @@ rtg_status query_neighbors(rtg_ctx* c, const rtg_csr* g, const int32_t* queries,
   const long long nnz = (long long)c->h_status->nnz;
   if (nnz > 0) {
     void* cp = nullptr;
-    if ((s = alloc_out_on(c, st, sizeof(int32_t) * (size_t)nnz, &cp)) != RTG_OK) {
+    if ((s = alloc_out(c, sizeof(int32_t) * (size_t)nnz, &cp)) != RTG_OK) {
       release_out(c, out);
       return s;
     }

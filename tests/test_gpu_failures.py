@@ -163,3 +163,71 @@ def test_cells_whose_scaled_rotation_is_subnormal():
         res.release()
     assert np.array_equal(rp, ref.row_ptr)
     assert np.array_equal(col, ref.col)
+
+
+def _same(res, ref):
+    rp, col = res.download()
+    band = res.stats["band"]
+    res.release()
+    assert np.array_equal(rp, ref.row_ptr)
+    assert np.array_equal(col, ref.col)
+    return band
+
+
+def test_scratch_kept_for_speed_refuses_no_call():
+    # the answer slots of index queries and the tiles of the default brute force are given back
+    # when an allocation fails; what then still fails is refused as before
+    n, d, m = 5000, 6, 8
+    pts = gen.points_uniform(21, n, d)
+    r = gen.radius_for_degree(n, d, 20.0)
+    T = gen.transforms(21, d, m, r)
+    q = gen.points_uniform(22, 700, d)
+    pairs, exact = oracle.rtg(pts, r, T, r).csr, oracle.brute(pts, r)
+    answers = oracle.rtg_query(pts, r, T, r, q)
+    with rtg.Context(0) as ctx:
+        ix = ctx.index(pts, r, T, r)
+        calls = {"query": (lambda: ix.query(q), answers), "pairs": (lambda: ctx.all_pairs(pts, r, T, r), pairs),
+                 "exact": (lambda: ctx.brute_force(pts, r), exact)}
+        for call, ref in calls.values():  # warm: only outputs are allocated from here on
+            for _ in range(2):
+                _same(call(), ref)
+        for name in ("pairs", "query", "exact"):
+            for after in (1, 2):  # the row pointers, then the columns
+                for warm, ref in (calls["query"], calls["exact"]):
+                    _same(warm(), ref)
+                rtg.rtg_set_test_hooks(ctx.handle, 0, 0, after)
+                _same(calls[name][0](), calls[name][1])
+                rtg.rtg_set_test_hooks(ctx.handle, 0, 0, 0)
+        for _ in range(2):  # the first failure takes what was kept, the second has nothing to take
+            rtg.rtg_set_test_hooks(ctx.handle, 0, 0, 1)
+            try:
+                _same(ctx.all_pairs(pts, r, T, r), pairs)
+            except rtg.RTGError as e:
+                assert e.status == rtg.RTG_E_NOMEM
+                break
+        else:
+            raise AssertionError("no allocation failed")
+        rtg.rtg_set_test_hooks(ctx.handle, 0, 0, 0)
+        _same(ctx.brute_force(pts, r), exact)
+        ix.close()
+
+
+def test_default_brute_force_without_room_for_tiles():
+    # whichever allocation of a first call fails: refused, or decided on the CUDA cores
+    n, d = 4500, 4
+    pts = gen.points_uniform(23, n, d, np.float32)
+    r = gen.radius_for_degree(n, d, 9.0)
+    ex = oracle.brute(pts, r)
+    refused, plain, tiles = 0, 0, 0
+    for after in range(1, 24):
+        with rtg.Context(0) as ctx:
+            rtg.rtg_set_test_hooks(ctx.handle, 0, 0, after)
+            try:
+                if _same(ctx.brute_force(pts, r), ex) > 0:
+                    tiles += 1
+                else:
+                    plain += 1
+            except rtg.RTGError as e:
+                assert e.status == rtg.RTG_E_NOMEM
+                refused += 1
+    assert plain == 3 and refused > 5 and tiles > 0, (refused, plain, tiles)
