@@ -791,6 +791,13 @@ def run_clustered(args):
     print(json.dumps(line), flush=True)
 
 
+def cuda_core_context(stream):
+    """A context whose default brute force keeps to the CUDA cores: one with a memory budget (without
+    one it takes tensor-core tiles from 4096 points on)."""
+    from paper_1409_8112_gb300 import rtg
+    return rtg.Context(0, mem_budget_bytes=64 << 30, stream=stream.cuda_stream)
+
+
 def run_table2(args):
     """Shift-only RTG with the paper's Table II parameters (Sec. IV-A): d = 6, m = 20 grids,
     c = 1.35 r, r from Eq. 2, n uniform points in [0,1]^6 (FP64, seed 0).  Reported pairs/s
@@ -827,9 +834,11 @@ def run_table2(args):
     ms, res = timed(lambda: ctx.all_pairs(pts, r, T, ct * r, timing=True), args.steps, args.warmup)
     pairs, st = res.nnz, res.stats
     res.release()
-    ex_ms, ex = timed(lambda: ctx.brute_force(pts, r, count_only=True), 3, 1)
+    plain = cuda_core_context(stream)
+    ex_ms, ex = timed(lambda: plain.brute_force(pts, r, count_only=True), 3, 1)
     exact = ex.nnz
     ex.release()
+    plain.close()
     tc_ms, tc = timed(lambda: ctx.brute_force(pts, r, count_only=True, tensor="fp16"), 3, 1)
     assert tc.nnz == exact
     tc.release()
@@ -1104,10 +1113,11 @@ def run_precision(args):
     rb = gen.radius_for_degree(nb, d)
     sample = torch.from_numpy(gen.points_uniform(1, nb, d, np.float32)).cuda()
     out = {}
-    for name, tensor in (("cuda_cores_fp32", None), ("tensor_fp16", "fp16"),
-                         ("tensor_bf16", "bf16")):
-        ctx.brute_force(sample, rb, count_only=True, tensor=tensor).release()
-        res, ms = timed(lambda: ctx.brute_force(sample, rb, count_only=True, tensor=tensor),
+    plain = cuda_core_context(stream)
+    for name, by, tensor in (("cuda_cores_fp32", plain, None), ("tensor_fp16", ctx, "fp16"),
+                             ("tensor_bf16", ctx, "bf16")):
+        by.brute_force(sample, rb, count_only=True, tensor=tensor).release()
+        res, ms = timed(lambda: by.brute_force(sample, rb, count_only=True, tensor=tensor),
                         max(2, args.steps // 3))
         st = res.stats
         out[name] = {"ms": round(ms, 3), "pairs": res.nnz,
@@ -1115,6 +1125,7 @@ def run_precision(args):
                      "fp64_band_rechecks": st["dist_rechecks"],
                      "band": st["band"], "max_abs_err_d2": st["max_abs_err_d2"]}
         res.release()
+    plain.close()
     line = {
         "metric": METRIC, "value": round(build.nnz / (build_ms / 1e3), 1), "unit": "pairs/s",
         "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "ms_per_step": round(build_ms, 3),

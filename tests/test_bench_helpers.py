@@ -62,3 +62,16 @@ def test_clock_samples_count_only_inside_the_timed_window():
     rec = c.stop()
     assert rec["samples"] == 2 and rec["reasons"] == [] and rec["sm_max_mhz"] == 2070.0
     assert 2055.0 <= rec["sm_mhz"] <= 2070.0
+
+
+def test_cuda_core_lines_are_timed_on_cuda_cores(monkeypatch):
+    # the default brute force of a context without a memory budget may take tensor-core tiles
+    import inspect
+
+    from paper_1409_8112_gb300 import rtg
+    made = {}
+    monkeypatch.setattr(rtg, "Context", lambda device, **kw: made.update(kw))
+    bench.cuda_core_context(type("S", (), {"cuda_stream": 7})())
+    assert made["mem_budget_bytes"] > 0 and made["stream"] == 7
+    for fn in (bench.run_table2, bench.run_precision):
+        assert "cuda_core_context(stream)" in inspect.getsource(fn)
