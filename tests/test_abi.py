@@ -81,3 +81,11 @@ def test_header_is_plain_c(tmp_path):
                         "-fsyntax-only", "-I", os.path.join(ROOT, "include"), str(src)],
                        capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
+
+
+def test_every_source_is_watched_for_changes():
+    # a library older than any of its sources is built again
+    from paper_1409_8112_gb300 import _build
+    have = {os.path.join(d, f) for d, _, fs in os.walk(_build.CSRC) for f in fs
+            if f.endswith((".cu", ".cuh", ".h", ".c"))}
+    assert have <= set(_build._deps())
