@@ -209,3 +209,25 @@ def test_key_width_settles():
             assert (st["key_bits"] > 32) == (r == small)
             passes.append(st["sort_passes"])
     assert passes[2] == passes[1] > passes[21] and passes[22] == passes[23] == passes[1], passes
+
+
+def test_wide_keys_are_given_up_soon():
+    # one build with keys of more than 32 bits does not leave the shape's next ones on 64-bit keys
+    # for long, and narrower ones now and then do not make every wide build run twice
+    n, d, m = 3000, 6, 5
+    pts = gen.points_uniform(68, n, d)
+    grids = {r: gen.transforms(68, d, m, r) for r in (0.03, 0.3)}
+
+    def build(r):
+        res = ctx.all_pairs(pts, r, grids[r], r)
+        st = res.stats
+        res.release()
+        return st
+
+    with rtg.Context(0) as ctx:
+        wide = [build(0.03) for _ in range(2)][1]["sort_passes"]
+        passes = [build(0.3)["sort_passes"] for _ in range(8)]
+        assert passes[:4] == [wide] * 4 and max(passes[4:]) < wide, (wide, passes)
+        assert build(0.03)["attempts"] == 2
+        for _ in range(3):
+            assert [build(r)["attempts"] for r in (0.3, 0.3, 0.3, 0.03)] == [1] * 4
