@@ -647,7 +647,10 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
     }
     const bool tc = m == 0 && (q.flags & (RTG_FLAG_TC_FP16 | RTG_FLAG_TC_BF16)) != 0;
     // (not under a memory budget, whose room is for the pairs)
-    bool tc_auto = m == 0 && !tc && n_total >= kBruteTcMin && c->budget == 0;
+    const bool tc_may = m == 0 && !tc && n_total >= kBruteTcMin && c->budget == 0;
+    const double r0 = B > 0 ? q.items[0].r : 0.0;
+    bool tc_auto = tc_may && g.ask_tiles(r0, two_pass);
+    const bool tc_left = tc_may && !tc_auto;
     c->tiles_in_use = tc;
     auto tile_room = [&]() -> rtg_status {
       rtg_status e;
@@ -973,6 +976,7 @@ rtg_status build(rtg_ctx* c, const Request& q, rtg_csr* out) {
       return s;
     }
     // remember the launch decisions for the next build of this shape
+    if (tc_auto || tc_left) g.settle_tiles(tc_auto, h.tc_band > 0.0, r0, two_pass);
     if (m > 0) g.settle_bits((int)h.sort_bits, (int)h.cell_bits, !known);
     if (!two_pass) {
       g.settle_pairs((long long)h.emitted);

@@ -118,6 +118,25 @@ struct ShapeGuess {
     const long long c = col_pairs < 0 ? pair_cap : std::min(pair_cap, tight_pairs(col_pairs));
     return c * (sym ? 2 : 1);
   }
+  // Default brute force: the radius (and form) at which the plan left the pairs to the CUDA cores,
+  // and the builds at that radius that keep to them without asking it again.  Operands, plan and
+  // the tiles' launch cost 8 to 20 us that such builds wait for (9000 points in 2-D 164 us without,
+  // 183 with); points of another extent at the same radius get the tiles kCalmBuilds builds late.
+  double no_tiles_r = 0.0;
+  bool no_tiles_two_pass = false;
+  int no_tiles = 0;
+  bool ask_tiles(double r, bool two_pass) const {
+    return no_tiles == 0 || r != no_tiles_r || two_pass != no_tiles_two_pass;
+  }
+  void settle_tiles(bool asked, bool used, double r, bool two_pass) {
+    if (!asked) {
+      --no_tiles;
+    } else {
+      no_tiles = used ? 0 : kCalmBuilds;
+      no_tiles_r = r;
+      no_tiles_two_pass = two_pass;
+    }
+  }
 };
 
 // A result whose columns fill less than half of their array, and leave more than this many entries

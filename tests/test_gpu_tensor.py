@@ -169,6 +169,32 @@ def test_default_brute_force_of_dense_graphs(ctx, share, emit_tiles, count_tiles
         res.release()
 
 
+def test_default_brute_force_does_not_ask_refused_tiles_again():
+    # a shape whose tiles were refused at a radius launches two kernels less for a while; another
+    # radius asks at once, the same one after 16 builds
+    n, d = 4300, 2
+    wide = gen.points_uniform(64, n, d)
+    r = gen.radius_for_degree(n, d, 0.02)
+    narrow = wide * (20.0 * r)  # the same radius, an extent the tiles resolve
+    with rtg.Context(0) as own:
+        def call(pts, radius):
+            res = own.brute_force(pts, radius)
+            ex, (rp, col), st = oracle.brute(pts, radius), res.download(), res.stats
+            assert np.array_equal(rp, ex.row_ptr) and np.array_equal(col, ex.col)
+            res.release()
+            return st["launches"], st["band"] > 0
+        asked = call(wide, r)
+        assert not asked[1]
+        for _ in range(3):
+            assert call(wide, r) == (asked[0] - 2, False)
+        assert call(wide, 8.0 * gen.radius_for_degree(n, d))[1]
+        assert call(wide, r) == asked
+        for _ in range(16):
+            assert not call(narrow, r)[1]
+        for _ in range(2):
+            assert call(narrow, r)[1]
+
+
 def _tile_error_bound(M, d, bf16):
     """|tile d^2 - d^2| for coordinates within M of the centre: half-precision hi + lo of the
     coordinates (and of the norms, for d <= 12) with unit roundoff u, FP32 sums of 48 or 52 terms
