@@ -227,6 +227,21 @@ __device__ void plan_band(int b, const Inst& I, int dtype, const unsigned long l
   }
 }
 
+// What roundings to a subnormal FP32 (of R, s, p, 1 / c, R / c or s / c), which are off by up to
+// 2^-150 instead of 2^-24 of the value, may add to the error of y / c on one axis (its rotation row
+// Rk): 2^-149 (P (1 + 1 / c) + Q / c + A), P = 1 + the sum of |p|, Q that of |R|.
+__device__ __noinline__ double subnormal_error(const Inst& I, const double* Rk, int d,
+                                               const unsigned long long* box, double A) {
+  double sum_p = 1.0, sum_R = 0.0;
+  for (int l = 0; l < d; ++l) {
+    const double hi = I.n > 0 ? dec_double(__ldcg(box + l * 2 + 0)) : 0.0;
+    const double lo = I.n > 0 ? dec_double(~__ldcg(box + l * 2 + 1)) : 0.0;
+    sum_p += fmax(fabs(lo), fabs(hi));
+    sum_R += fabs(Rk[l]);
+  }
+  return 0x1.0p-149 * (sum_p * (1.0 + I.inv_c) + sum_R * I.inv_c + A);
+}
+
 // Item (b, t, k): key layout of axis k of grid t of instance b (the bounding box is read from
 // L2).  Without grids (brute force) item (b, 0, 0) sets the instance's distance band; with
 // grids the key kernel sets it, off the critical path.
@@ -254,7 +269,8 @@ __device__ void plan_axis_item(long long idx, const Inst* __restrict__ inst, int
   }
   const double* R = T64 + I.T0 + (size_t)t * (d * d + d);
   const double* s = R + d * d;
-  double ymin = s[k], ymax = s[k], A = fabs(s[k]), sum_p = 1.0, sum_R = 0.0;
+  double ymin = s[k], ymax = s[k], A = fabs(s[k]);
+  int top_p = 0, top_r = 0;  // leading bits of the largest |p| and FP32 |R|, ordered as they are
 #pragma unroll 3  // the loads of a few axes in flight together
   for (int l = 0; l < d; ++l) {
     const double hi = I.n > 0 ? dec_double(__ldcg(bbox + ((size_t)b * kMaxDim + l) * 2 + 0)) : 0.0;
@@ -263,10 +279,12 @@ __device__ void plan_axis_item(long long idx, const Inst* __restrict__ inst, int
     const double a = rkl * lo, bb = rkl * hi;
     ymin += fmin(a, bb);
     ymax += fmax(a, bb);
-    A += fabs(rkl) * fmax(fabs(lo), fabs(hi));
-    sum_p += fmax(fabs(lo), fabs(hi));
-    sum_R += fabs(rkl);
-    G.Rf[k * kMaxDim + l] = __double2float_rn(rkl);
+    const double p = fmax(fabs(lo), fabs(hi));
+    A += fabs(rkl) * p;
+    top_p = max(top_p, __double2hiint(p));
+    const float rf = __double2float_rn(rkl);
+    top_r = max(top_r, __float_as_int(fabsf(rf)));
+    G.Rf[k * kMaxDim + l] = rf;
   }
   for (int l = d; l < kMaxDim; ++l) G.Rf[k * kMaxDim + l] = 0.0f;
   G.sf[k] = __double2float_rn(s[k]);
@@ -283,10 +301,14 @@ __device__ void plan_axis_item(long long idx, const Inst* __restrict__ inst, int
     G.qlo[k] = (long long)qmin;
     G.ext[k] = (unsigned long long)((long long)qmax - (long long)qmin + 1);
   }
-  // Roundings to a subnormal FP32 (of R, s, p, 1 / c, R / c or s / c) are off by up to 2^-150
-  // instead of 2^-24 of the value: nothing next to the first term unless magnitudes are extreme.
-  const double E = ((double)(d + 6) * 0x1.0p-24 * A + 3e-12) * I.inv_c * (1.0 + 1e-6) +
-                   0x1.0p-149 * (sum_p * (1.0 + I.inv_c) + sum_R * I.inv_c + A);
+  double E = ((double)(d + 6) * 0x1.0p-24 * A + 3e-12) * I.inv_c * (1.0 + 1e-6);
+  // Below these limits P + Q < 2^34 and c (P + A) < 2^89, so that subnormal_error is below 2^-60 / c
+  // and the 3e-18 / c that 1 + 1e-6 leaves covers it (its FP64 sums, taken for every item, took the
+  // prep phase of 40 roadmaps of 3, 6 and 9 dimensions from 117 to 133 us).
+  if (top_p >= __double2hiint(0x1.0p28) || top_r >= __float_as_int(0x1.0p28f) ||
+      __double2hiint(A) >= __double2hiint(0x1.0p60) ||
+      __double2hiint(I.inv_c) < __double2hiint(0x1.0p-28))
+    E += subnormal_error(inst[b], R + k * d, d, bbox + (size_t)b * kMaxDim * 2, A);
   G.E[k] = __double2float_ru(E);
 }
 

@@ -231,3 +231,21 @@ def test_default_brute_force_without_room_for_tiles():
                 assert e.status == rtg.RTG_E_NOMEM
                 refused += 1
     assert plain == 3 and refused > 5 and tiles > 0, (refused, plain, tiles)
+
+
+@pytest.mark.parametrize("scale", [2.0 ** 27, 2.0 ** 28, 2.0 ** 29, 2.0 ** 61, 2.0 ** -60])
+@pytest.mark.parametrize("d", [3, 8])
+def test_cells_on_either_side_of_the_limits_of_the_subnormal_term(d, scale):
+    # the error bound leaves the subnormal roundings out below 2^28 (coordinates, cells) and 2^60
+    # (shifts and rotated coordinates)
+    pts = gen.points_uniform(70 + d, 600, d) * scale
+    r = gen.radius_for_degree(600, d) * scale
+    T = gen.transforms(70 + d, d, 3, r)
+    ref = oracle.rtg(pts, r, T, r).csr
+    with rtg.Context(0) as ctx:
+        res = ctx.all_pairs(pts, r, T, r)
+        rp, col = res.download()
+        res.release()
+    assert ref.nnz > 0
+    assert np.array_equal(rp, ref.row_ptr)
+    assert np.array_equal(col, ref.col)
