@@ -257,7 +257,8 @@ rtg_status rtg_batch_all_pairs(rtg_ctx* ctx, const rtg_instance* items, int coun
  * n >= 4096 where their band is below r^2 / 8, at most 40% of the pairs of a sample (3% when
  * only counting) lie within r^2 + band, there is room for them and the context has no budget;
  * the pairs they leave, or all pairs, are decided by the FP32 filter with FP64 recheck of the
- * CUDA-core kernel, and counted in the same counters. */
+ * CUDA-core kernel, and counted in the same counters (where that filter cannot hold, only the
+ * pairs the tiles leave are counted as owned and rechecked). */
 rtg_status rtg_brute_force(rtg_ctx* ctx, const void* points, int dtype, int points_on_device,
                            int64_t n, int d, double r, uint32_t flags, int count_only,
                            rtg_csr* out);

@@ -39,7 +39,7 @@ thread_local std::string g_err;
 // best variant could save.
 constexpr long long kTuneMinElements = 1LL << 17;
 // Brute force of at least this many points takes its distances from tensor-core tiles when the
-// tiles' error bound allows (30,011 points in 6-D: 144 us against 989 on CUDA cores; below,
+// tiles' error bound allows (30,011 points in 6-D: 136 us against 988 on CUDA cores; below,
 // the tiles' set-up costs more than they save).
 constexpr long long kBruteTcMin = 4096;
 constexpr size_t kMaxGraphs = 32;  // executable graphs kept per context (one per shape)

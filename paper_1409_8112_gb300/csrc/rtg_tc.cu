@@ -10,10 +10,11 @@
 // norms ride in the hi block of three MMAs; beyond, three MMAs give x.y and the epilogue adds
 // the norms.  Operands sit in shared memory in the K-major layout without
 // swizzle: core matrices of 8 rows x 16 bytes, 128 bytes apart along K and 512 bytes apart
-// along M or N.  A CTA of 4 warps owns a 128 x 128 FP32 accumulator (128 TMEM columns);
-// warp w reads lanes 32w..32w+31.  The band is max(1e-3 r^2, E) where E bounds the error of
-// the FP32 d^2: the hi/lo representation and dropped lo.lo term, FP32 accumulation of the
-// 48 products, the norms, the epilogue and the centring (see tc_plan).
+// along M or N.  A CTA of ten warps (copies, MMAs, eight of epilogue) owns two 128 x 256 FP32
+// accumulators, all 512 TMEM columns of its SM (k_brute_tc).  The band is max(1e-3 r^2, 1.25 E),
+// and for unasked tiles at least what the CUDA-core filter keeps; E bounds the error of the FP32
+// d^2: the hi/lo representation and dropped lo.lo term, FP32 accumulation of the products, the
+// norms, the epilogue and the centring (tc_plan_band).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -458,7 +459,7 @@ __device__ __forceinline__ bool tc_elect() {
 // costs 16 KB of column tiles for four tile pairs (8 KB for each would be near 60 bytes a clock
 // and SM of L2 bandwidth).
 // 200k points in 6-D (2e10 pair tests), FP16: 7.26 ms with 128 x 128 jobs, 4 CTAs per SM, block
-// barriers and a mask for every chunk; 3.37 now: 1.84 without candidates (the TMEM reads alone
+// barriers and a mask for every chunk; 3.28 now: 1.84 without candidates (the TMEM reads alone
 // would take 0.8, the MMAs 0.5), the rest for the 1.8 million candidates, for each of which a
 // warp stops about 800 clocks and the others wait for its accumulator.
 template <bool BF16, bool EMIT, int FORM>
